@@ -1525,6 +1525,26 @@ static rd_status time_cfg(rd_graph* g, int64_t width, const rd_query_opts& o, co
     return RD_OK;
 }
 
+// Double-float degrees for RD_MODE_DF64, once per graph and before the first kernel of that
+// mode (a query's or the autotuner's).
+static rd_status ensure_df_degrees(rd_graph* g, const rd_query_opts& o, cudaStream_t st)
+{
+    if (mode_prec(o.mode) != 2 || g->degdf || g->n == 0) return RD_OK;
+    df64 *d = nullptr, *inv = nullptr;
+    RD_CUDA(cudaMalloc((void**)&d, sizeof(df64) * g->n));
+    const cudaError_t e = cudaMalloc((void**)&inv, sizeof(df64) * g->n);
+    if (e != cudaSuccess) {
+        cudaFree(d);
+        return cuda_status(e, "cudaMalloc (double-float degrees)");
+    }
+    g->degdf = d;
+    g->invdegdf = inv;
+    const int grid = std::max(1, std::min(g->sm_count * 8, (int)((g->n + 255) / 256)));
+    launch_split_df(st, grid, g->n, g->deg64, g->degdf);
+    launch_split_df(st, grid, g->n, g->invdeg64, g->invdegdf);
+    return RD_OK;
+}
+
 // Tune the width classes a query of P pairs can use (all of them down to the narrowest
 // tile when the query compacts), skipping classes already in g's table.
 static rd_status ensure_tuned(rd_graph* g, int64_t P, const rd_query_opts& o, bool plain, bool compact,
@@ -1574,13 +1594,7 @@ static rd_status prepare_run(RunCtx& c, rd_graph* g, int64_t P, const rd_query_o
     c.profile = (o.flags & RD_Q_PROFILE) != 0;
     c.compact = compact;
     c.lagged_polls = lagged_polls && c.ev != nullptr;
-    if (mode_prec(o.mode) == 2 && !g->degdf && g->n > 0) {  // double-float degrees, once per graph
-        RD_CUDA(cudaMalloc((void**)&g->degdf, sizeof(df64) * g->n));
-        RD_CUDA(cudaMalloc((void**)&g->invdegdf, sizeof(df64) * g->n));
-        const int grid = std::max(1, std::min(g->sm_count * 8, (int)((g->n + 255) / 256)));
-        launch_split_df(st, grid, g->n, g->deg64, g->degdf);
-        launch_split_df(st, grid, g->n, g->invdeg64, g->invdegdf);
-    }
+    RD_TRY(ensure_df_degrees(g, o, st));
     RD_TRY(ensure_tuned(g, P, o, plain, compact, st));
     RD_TRY(make_plan(g, P, o, plain, &c.pl));
     c.cur = c.pl;
@@ -1862,6 +1876,7 @@ rd_status rd_autotune(rd_graph* g, int64_t npairs, const rd_query_opts* opts, in
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool plain = (o.flags & RD_Q_PLAIN) != 0;
+    RD_TRY(ensure_df_degrees(g, o, st));
     RD_TRY(ensure_tuned(g, npairs, o, plain, !plain && (o.flags & RD_Q_NO_COMPACT) == 0, st));
     RD_CUDA(cudaStreamSynchronize(st));
     Plan pl;

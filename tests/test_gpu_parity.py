@@ -883,3 +883,15 @@ def test_direct_potential_matches_replay_pass(rd, mode, tol):
             fa, _ = G.flow(s[:6], t[:6], mode=mode, **kw)
             fb, _ = G.flow(s[:6], t[:6], mode=mode, potential_mode="replay", **kw)
             assert np.abs(fa - fb).max() <= tol * np.abs(fb).max()
+
+
+def test_autotune_in_double_float_mode_on_a_fresh_graph(rd):
+    """rd_autotune as the first call in RD_MODE_DF64: the candidates it times read the
+    double-float degrees, which it makes itself; the query that follows uses the table."""
+    g = F.grid_deleted(40, 0.05, 5)
+    s, t = F.random_pairs(g.n, 12, 8)
+    G = rd.Graph.from_csr(g)
+    cfg = G.autotune(12, mode="df64")
+    res = G.query(s, t, mode="df64", k_max=2000, rel_tol=0.0, resid_tol=1e-11)
+    assert G.last_stats()["tuned"] == 1 and G.last_stats()["rhs_tile"] == cfg["rhs_tile"]
+    assert rel(res.r, dense.DenseRD.of(g).r(s, t)).max() < FP64_TOL
