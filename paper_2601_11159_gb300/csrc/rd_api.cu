@@ -1796,6 +1796,11 @@ rd_status rd_graph_set_weights(rd_graph* g, const float* weights, void* stream)
     int64_t loops = 0;
     RD_TRY(check_csr(g, st, &loops));
     RD_TRY(compute_degrees(g, st));
+    if (g->degdf) {  // the double-float copies follow the new degrees
+        const int grid = std::max(1, std::min(g->sm_count * 8, (int)((g->n + 255) / 256)));
+        launch_split_df(st, grid, g->n, g->deg64, g->degdf);
+        launch_split_df(st, grid, g->n, g->invdeg64, g->invdegdf);
+    }
     return rows_sorted_symmetric(g, st, &g->rows_sorted_sym);
 }
 

@@ -895,3 +895,16 @@ def test_autotune_in_double_float_mode_on_a_fresh_graph(rd):
     res = G.query(s, t, mode="df64", k_max=2000, rel_tol=0.0, resid_tol=1e-11)
     assert G.last_stats()["tuned"] == 1 and G.last_stats()["rhs_tile"] == cfg["rhs_tile"]
     assert rel(res.r, dense.DenseRD.of(g).r(s, t)).max() < FP64_TOL
+
+
+def test_double_float_query_follows_new_weights(rd):
+    """rd_graph_set_weights after a double-float query: the next one uses the new degrees."""
+    g = F.grid_deleted(40, 0.05, 5)
+    s, t = F.random_pairs(g.n, 5, 8)
+    G = rd.Graph.from_csr(g)
+    kw = dict(mode="df64", k_max=3000, rel_tol=0.0, resid_tol=1e-11)
+    G.query(s, t, **kw)
+    g2 = F.weighted(g, F.lognormal_edge_weights(g.m, 0.0, 0.7, 91))
+    G.set_weights(g2.w)
+    res = G.query(s, t, **kw)
+    assert rel(res.r, dense.DenseRD.of(g2).r(s, t)).max() < FP64_TOL
