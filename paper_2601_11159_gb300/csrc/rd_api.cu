@@ -498,7 +498,9 @@ struct Buffers {
     int32_t* summary;
     int32_t* err_flag;
     int32_t* step_dev;        // step index of graph-replayed steps (zeroed per query)
-    int32_t* loop_saved;      // [4]: where the device-resident loop stopped (see launch_loop_cond)
+    int32_t* loop_norm;       // step index of the device-resident loop's normalise passes
+    int32_t* loop_ticket;     // finalize blocks done in the loop's current step
+    int32_t* loop_saved;      // [4]: where the device-resident loop stopped (see k_finalize)
     int32_t* loop_cfrom;      // first step at which the loop tests for a column compaction
     uint32_t* row_mask;       // n x ld bits: entries of q_2 the sparse first normalise pass wrote
     // gradient / potential
@@ -531,9 +533,9 @@ static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, boo
     b->heavy_part = c.take<char>(std::max<int64_t>(g->n_chunks, 1) * ld * pl.elem);
     // sized for any column tile and any grid of up to 8 blocks of kBlock threads per SM
     b->block_part = c.take<double>((size_t)ld * 3 * (size_t)std::max(pl.grid_main, g->sm_count * 8));
-    b->old_slot = c.take<int32_t>(ld);
-    b->slot_pair[0] = c.take<int32_t>(ld);
-    b->slot_pair[1] = c.take<int32_t>(ld);
+    b->old_slot = compact ? c.take<int32_t>(ld) : nullptr;
+    b->slot_pair[0] = compact ? c.take<int32_t>(ld) : nullptr;
+    b->slot_pair[1] = compact ? c.take<int32_t>(ld) : nullptr;
     c.off = (c.off + 255) & ~size_t(255);
     b->state_bytes_begin = c.off;
     b->cf_hist = compact ? nullptr : c.take<char>((K + 1) * 4 * ld * pl.elem);
@@ -541,14 +543,15 @@ static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, boo
     b->cf_cur[1] = compact ? c.take<char>(4 * ld * pl.elem) : nullptr;
     PairState& s = b->st;
     s.b2 = c.take<double>(ld);
+    s.bnorm = c.take<double>(ld);
     s.delta = c.take<double>(ld);
+    s.inv_delta = c.take<double>(ld);
     s.g = c.take<double>(ld);
     s.S = c.take<double>(ld);
     s.beta = c.take<double>(ld);
     s.ring = c.take<double>(kRing * ld);
     s.r = c.take<double>(ld);
     s.err = c.take<double>(ld);
-    s.resid = c.take<double>(ld);
     s.k = c.take<int32_t>(ld);
     s.status = c.take<int32_t>(ld);
     s.active = c.take<int32_t>(ld);
@@ -558,6 +561,8 @@ static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, boo
     b->summary = c.take<int32_t>(2);
     b->err_flag = c.take<int32_t>(1);
     b->step_dev = c.take<int32_t>(1);
+    b->loop_norm = c.take<int32_t>(1);
+    b->loop_ticket = c.take<int32_t>(1);
     b->loop_saved = c.take<int32_t>(4);
     b->loop_cfrom = c.take<int32_t>(1);
     // queries on graphs that take the sparse first step (rows sorted, symmetric)
@@ -1064,11 +1069,11 @@ static rd_status launch_step_graph(RunCtx& c, const FinArgs& base)
 }
 
 // The device-resident step loop: one CUDA graph whose conditional while node repeats a body of
-// one Lanczos step for each orientation of the two vector blocks, each step with a condition
-// before it and one after its finalize, so that the steps of a query run without the host
-// until every pair has stopped, k_max is reached or a column compaction is due (then after the
-// finalize of the step before it, so that the host runs that step's normalise pass fused with
-// the packing). Where it stopped is read back by the caller (loop_saved).
+// one Lanczos step for each orientation of the two vector blocks, after an entry condition; the
+// last block of each step's finalize decides how to go on, so that the steps of a query run
+// without the host until every pair has stopped, k_max is reached or a column compaction is due
+// (then after the finalize of the step before it, so that the host runs that step's normalise
+// pass fused with the packing). Where it stopped is read back by the caller (loop_saved).
 template <typename T>
 static rd_status launch_step_loop(RunCtx& c, const FinArgs& base, int compact_check, int lag)
 {
@@ -1080,6 +1085,17 @@ static rd_status launch_step_loop(RunCtx& c, const FinArgs& base, int compact_ch
     std::swap(c.b.q[0], c.b.q[1]);
     graph_step_args<T>(c, base, &sa[1], &fa[1], &na[1]);
     std::swap(c.b.q[0], c.b.q[1]);
+    for (int o = 0; o < 2; ++o) {
+        fa[o].loop = 1;
+        fa[o].loop_compact = compact_check;
+        fa[o].loop_lag = lag;
+        fa[o].loop_step = c.b.step_dev;
+        fa[o].loop_norm = c.b.loop_norm;
+        fa[o].loop_ticket = c.b.loop_ticket;
+        fa[o].loop_saved = c.b.loop_saved;
+        fa[o].loop_cfrom = c.b.loop_cfrom;
+        na[o].step_dev = c.b.loop_norm;
+    }
     const bool heavy = g->n_chunks > 0;
     int misc[10] = {c.cur.cfg.vec, c.cur.cfg.gs, c.cur.cfg.nzl, c.cur.cfg.kind, c.cur.grid_main, c.cur.grid_heavy,
                     c.cur.grid_norm, c.pl.k_max, compact_check, lag};
@@ -1104,13 +1120,24 @@ static rd_status launch_step_loop(RunCtx& c, const FinArgs& base, int compact_ch
         RD_CUDA(cudaGraphCreate(&graph, 0));
         cudaGraphConditionalHandle h;
         cudaError_t e = cudaGraphConditionalHandleCreate(&h, graph, 1u, cudaGraphCondAssignDefault);
+        fa[0].loop_handle = fa[1].loop_handle = (unsigned long long)h;
+        // the entry condition, then the while node
+        if (e == cudaSuccess)
+            e = cudaStreamBeginCaptureToGraph(cs, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            launch_loop_entry(cs, fa[0]);
+            cudaGraph_t same = nullptr;
+            e = cudaStreamEndCapture(cs, &same);
+        }
+        cudaGraphNode_t entry, node;
+        size_t nentry = 1;
+        if (e == cudaSuccess) e = cudaGraphGetNodes(graph, &entry, &nentry);
         cudaGraphNodeParams np = {};
         np.type = cudaGraphNodeTypeConditional;
         np.conditional.handle = h;
         np.conditional.type = cudaGraphCondTypeWhile;
         np.conditional.size = 1;
-        cudaGraphNode_t node;
-        if (e == cudaSuccess) e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np);
+        if (e == cudaSuccess) e = cudaGraphAddNode(&node, graph, &entry, nullptr, 1, &np);
         if (e == cudaSuccess)
             e = cudaStreamBeginCaptureToGraph(cs, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                               cudaStreamCaptureModeThreadLocal);
@@ -1120,16 +1147,11 @@ static rd_status launch_step_loop(RunCtx& c, const FinArgs& base, int compact_ch
         }
         bool ok = true;
         for (int o = 0; o < 2 && ok; ++o) {
-            launch_loop_cond(cs, h, c.b.step_dev, c.b.st.act_count, c.b.loop_saved, c.b.loop_cfrom, c.pl.k_max,
-                             c.cur.ld, compact_check, lag, 0);
             if (heavy) ok = launch_spmm_t(c.cur.cfg, g->weighted, true, c.cur.grid_heavy, cs, sa[o]);
             if (ok) ok = launch_spmm_t(c.cur.cfg, g->weighted, false, c.cur.grid_main, cs, sa[o]);
             if (ok) {
                 launch_finalize(cs, fa[o]);
-                launch_loop_cond(cs, h, c.b.step_dev, c.b.st.act_count, c.b.loop_saved, c.b.loop_cfrom,
-                                 c.pl.k_max, c.cur.ld, compact_check, lag, 1);
                 launch_normalize_t(c.cur.grid_norm, cs, na[o]);
-                launch_step_advance(cs, c.b.step_dev, c.pl.k_max);
             }
         }
         cudaGraph_t body = nullptr;
@@ -1237,7 +1259,7 @@ static rd_status run_forward(RunCtx& c)
     for (int j = 0; j < c.pl.k_max; ++j) {
         if (dloop && j > 0) {
             const int compact_check = c.compact ? 1 : 0;
-            const int per_step = (c.g->n_chunks > 0 ? 2 : 1) + 5;
+            const int per_step = (c.g->n_chunks > 0 ? 2 : 1) + 2;
             while (true) {
                 const int j0 = c.steps;
                 const double bytes_per_step = spmm_launch_bytes(c.g, c.cur);
@@ -1251,7 +1273,7 @@ static rd_status run_forward(RunCtx& c)
                 const int jn = h[8];
                 const int ran = jn - j0;  // steps run whole inside the loop
                 // body passes: the stop shows in pass ran/2 + 1, and every kernel of a pass launches
-                c.launches += (int64_t)(ran / 2 + 1) * 2 * per_step;
+                c.launches += (int64_t)(ran / 2 + 1) * 2 * per_step + 1;
                 c.spmm_launches += ran;
                 c.spmm_bytes += bytes_per_step * ran;
                 if (ran & 1) std::swap(c.b.q[0], c.b.q[1]);

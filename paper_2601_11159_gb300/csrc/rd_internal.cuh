@@ -153,14 +153,15 @@ struct NormPackArgs {
 // Per-pair FP64 state of the running LDL^T factorisation of I - T_k.
 struct PairState {
     double* b2;        // ||b||^2 = 1/d_s + 1/d_t
+    double* bnorm;     // ||b||
     double* delta;     // last pivot
+    double* inv_delta; // 1 / delta
     double* g;         // last entry of L^{-1} e_1
     double* S;         // e_1^T (I - T_k)^{-1} e_1
     double* beta;      // beta_{k+1}
     double* ring;      // kRing x ld increments
     double* r;         // b2 * S
     double* err;       // estimated relative error
-    double* resid;     // relative residual
     int32_t* k;        // steps done
     int32_t* status;   // rd_status per pair
     int32_t* active;   // 1 while iterating
@@ -188,6 +189,15 @@ struct FinArgs {
     int df;                             // 1: coefficients are stored as double-float pairs
     void* xcf;                          // nullable T [k_max][2][ld]: step j receives lambda_i, mu_i
                                         // of the potential's direct update (identity slot map only)
+    // device-resident step loop (see k_finalize and k_loop_entry)
+    int loop;                           // 1: this launch is in the loop's body
+    int loop_compact, loop_lag;         // test for a column compaction, on the count `lag` steps back
+    unsigned long long loop_handle;     // the while node's cudaGraphConditionalHandle
+    int32_t* loop_step;                 // step index of the body's pre-pass, SpMM and finalize
+    int32_t* loop_norm;                 // step index of the body's normalise pass
+    int32_t* loop_ticket;               // finalize blocks done (0 between steps)
+    int32_t* loop_saved;                // [4]: where the loop stopped
+    const int32_t* loop_cfrom;          // first step at which a compaction is tested for
 };
 
 // Whole recurrence of one pair per CTA with q_{i-1}, q_i and W in shared memory (graphs
@@ -340,16 +350,8 @@ void launch_split_df(cudaStream_t st, int grid, int64_t n, const double* src, df
 void launch_finalize(cudaStream_t st, const FinArgs& a);
 // Advance the device step index by one, saturating at `limit` (end of a replayed step).
 void launch_step_advance(cudaStream_t st, int32_t* step, int limit);
-// Condition kernels of the device-resident step loop (a conditional while node). Before step
-// j (*step = j): continue while pairs are active, k_max is not reached and no column
-// compaction is due. After step j's finalize (after_finalize = 1): stop if a compaction is
-// due before step j + 1, with step j's normalise pass still to run (the host runs it fused
-// with the packing). On stop, record j, the active count the compaction test read, the
-// active count entering the next step, and where the loop stopped (0 before the step, 1
-// after its finalize) in saved[0..3], and park *step at k_max + 1.
-void launch_loop_cond(cudaStream_t st, cudaGraphConditionalHandle h, int32_t* step, const int32_t* act_count,
-                      int32_t* saved, const int32_t* compact_from, int k_max, int64_t ld, int compact_check, int lag,
-                      int after_finalize);
+// Entry condition of the device-resident step loop, on its finalize launch's arguments.
+void launch_loop_entry(cudaStream_t st, const FinArgs& a);
 
 struct InitArgs {
     int64_t n, ld;

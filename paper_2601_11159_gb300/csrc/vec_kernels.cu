@@ -57,8 +57,8 @@ __global__ void k_init(const InitArgs a)
     q[(int64_t)s * a.ld + p] = (T)(1.0 / (ds * bn));
     q[(int64_t)t * a.ld + p] = (T)(-1.0 / (dt * bn));
     st.b2[p] = b2;
+    st.bnorm[p] = bn;
     st.err[p] = 1.0;
-    st.resid[p] = 1.0;
     st.status[p] = RD_OK;
     st.active[p] = 1;
     atomicAdd(&st.act_count[0], 1);
@@ -110,7 +110,7 @@ static_assert(kRing == 4, "PairScalars holds four ring slots");
 struct PairStepOut {
     bool ok;                       // false: a value was not finite or I - T_i lost definiteness
     bool warn_not_converged;       // k_max reached before a tolerance was met
-    double alpha, cdef, beta_next, incr, r, resid, est;
+    double alpha, cdef, beta_next, incr, gd, r, est;
 };
 
 __device__ __forceinline__ PairScalars pair_load(const PairState& st, int p, int64_t np)
@@ -121,7 +121,7 @@ __device__ __forceinline__ PairScalars pair_load(const PairState& st, int p, int
     s.g = st.g[p];
     s.S = st.S[p];
     s.beta = st.beta[p];
-    s.inv_delta = s.delta != 0.0 ? 1.0 / s.delta : 0.0;
+    s.inv_delta = st.inv_delta[p];
     s.r0 = st.ring[p];
     s.r1 = st.ring[np + p];
     s.r2 = st.ring[2 * np + p];
@@ -129,21 +129,38 @@ __device__ __forceinline__ PairScalars pair_load(const PairState& st, int p, int
     return s;
 }
 
-// The arithmetic of one step on the scalars (see pair_update); returns true when the pair
-// stops. The state in `s` is advanced exactly as pair_update advances the stored state.
-// FP64 division and square root are slow on this part (hundreds of cycles each, one thread
-// at a time on the whole-recurrence kernels' critical path), so the step takes four divisions
-// and one square root: 1/delta_{i-1} is kept from the previous step, 1/sum(d) is passed in,
-// 1/delta_i and 1/S_i serve every quotient by them, and the largest increment ratio is found
-// by cross-multiplication (increments are positive) before its one division.
-__device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int j, double A, double B, double C,
-                                          PairStepOut& o)
+// Finite: tested on the exponent bits (an FP64 comparison would occupy the FP64 unit).
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// What the next vector needs of the three sums: alpha_i, the deflation constant c_i,
+// beta_{i+1}^2, beta_{i+1} and 1/beta_{i+1}.
+struct StepCoef {
+    double alpha, cdef, beta2, beta, inv_beta;
+};
+
+__device__ __forceinline__ StepCoef step_coef(const FinArgs& a, double A, double B, double C)
 {
-    const double alpha = A;
+    StepCoef k;
+    k.alpha = A;
+    k.cdef = a.deflate ? C * a.inv_sumdeg : 0.0;
+    const double gamma2 = a.deflate ? C * k.cdef : 0.0;
+    k.beta2 = B - A * A - gamma2;
+    k.beta = sqrt(fmax(k.beta2, 0.0));
+    k.inv_beta = 1.0 / k.beta;  // not used when beta is 0 (the step is a breakdown) or not finite
+    return k;
+}
+
+// The rest of one step on the scalars (see pair_update): the LDL^T factors, the estimate and the
+// stop tests; returns true when the pair stops. The state in `s` is advanced exactly as
+// pair_update advances the stored state. Divisions are what this chain is made of, so
+// 1/delta_{i-1} is kept from the previous step, 1/sum(d) is passed in, 1/delta_i serves every
+// quotient by it, the largest increment ratio rho = num/den is found by cross-multiplication
+// (increments are positive), and the estimate incr rho / (1 - rho)^2 / S is one quotient,
+// incr num den / ((den - num)^2 S).
+__device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int j, const StepCoef& k, PairStepOut& o)
+{
+    const double alpha = k.alpha;
     const double beta_i = s.beta;
-    const double cdef = a.deflate ? C * a.inv_sumdeg : 0.0;
-    const double gamma2 = a.deflate ? C * cdef : 0.0;
-    const double beta2 = B - alpha * alpha - gamma2;
     double delta, g;
     if (j == 0) {
         delta = 1.0 - alpha;
@@ -154,11 +171,12 @@ __device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int 
         g = s.g * beta_i * idp;
     }
     bool stop = false;
-    o.ok = isfinite(alpha) && isfinite(beta2) && isfinite(delta) && delta > 0.0;
+    o.ok = finite64(alpha) && finite64(k.beta2) && finite64(delta) && delta > 0.0;
     o.warn_not_converged = false;
     o.alpha = alpha;
-    o.cdef = cdef;
+    o.cdef = k.cdef;
     o.beta_next = 0.0;
+    o.gd = 0.0;
     if (!o.ok) return true;  // frozen at its last good estimate
     const double inv_delta = 1.0 / delta;
     const double gd = g * inv_delta;
@@ -166,12 +184,12 @@ __device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int 
     const double S = s.S + incr;
     s.S = S;
     o.incr = incr;
+    o.gd = gd;
     o.r = s.b2 * S;
     s.set_ring(j % kRing, incr);
-    const double beta_next = sqrt(fmax(beta2, 0.0));
+    const double beta_next = k.beta;
     o.beta_next = beta_next;
     const double resid = beta_next * fabs(gd);
-    o.resid = resid;
     s.delta = delta;
     s.inv_delta = inv_delta;
     s.g = g;
@@ -187,11 +205,6 @@ __device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int 
     const bool use_est = !a.fixed_k && a.rel_tol > 0.0;
     double est = 0.0;
     if (!breakdown && (use_est || stop || j + 1 >= a.k_max)) {
-        const double inv_S = 1.0 / S;
-        double tail = 0.0;
-        const int nr = j + 1 < kRing ? j + 1 : kRing;
-        for (int q = 0; q < nr; ++q) tail += s.ring(q);
-        est = tail * inv_S;
         if (!a.est_delayed && j + 1 >= kRing) {
             // the largest num/den over the last kRing-1 pairs of consecutive increments
             double bn = s.ring(j % kRing), bd = s.ring((j - 1) % kRing);
@@ -203,9 +216,17 @@ __device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int 
                     bd = den;
                 }
             }
-            const double rho = fmax(0.5, bn / bd);
-            const double om = 1.0 - rho;
-            est = rho < 1.0 ? incr * rho * inv_S / (om * om) : INFINITY;
+            if (bn + bn <= bd) {  // rho at its floor 1/2
+                bn = 1.0;
+                bd = 2.0;
+            }
+            const double gap = bd - bn;
+            est = bn < bd ? incr * bn * bd / (gap * gap * S) : INFINITY;
+        } else {
+            double tail = 0.0;
+            const int nr = j + 1 < kRing ? j + 1 : kRing;
+            for (int q = 0; q < nr; ++q) tail += s.ring(q);
+            est = tail / S;
         }
         if (!stop && use_est && j + 1 >= kRing && est <= a.rel_tol) stop = true;
     }
@@ -228,12 +249,12 @@ __device__ __forceinline__ void pair_store(const PairState& st, int p, int j, in
         st.S[p] = s.S;
         st.r[p] = o.r;
         st.ring[(int64_t)(j % kRing) * np + p] = o.incr;
-        st.resid[p] = o.resid;
         st.err[p] = o.est;
         st.hist_alpha[(int64_t)j * np + p] = o.alpha;
         st.hist_beta[(int64_t)(j + 1) * np + p] = o.beta_next;
         st.k[p] = j + 1;
         st.delta[p] = s.delta;
+        st.inv_delta[p] = s.inv_delta;
         st.g[p] = s.g;
         if (o.warn_not_converged) st.status[p] = RD_WARN_NOT_CONVERGED;
     }
@@ -241,29 +262,39 @@ __device__ __forceinline__ void pair_store(const PairState& st, int p, int j, in
     else st.beta[p] = s.beta;
 }
 
+// One step of pair p on the stored state: writes the pair's state and history; returns true when
+// the pair stops (then active = 0). `k` and `o` receive the step's coefficients and results.
 __device__ __forceinline__ bool pair_update(const FinArgs& a, const PairState& st, int p, int j, double A, double B,
-                                            double C, double* alpha_o, double* cdef_o, double* beta_next_o)
+                                            double C, StepCoef& k, PairStepOut& o)
 {
     PairScalars s = pair_load(st, p, a.pstride);
-    PairStepOut o;
-    const bool stop = pair_core(a, s, j, A, B, C, o);
+    k = step_coef(a, A, B, C);
+    const bool stop = pair_core(a, s, j, k, o);
     pair_store(st, p, j, a.pstride, s, o, stop);
-    if (stop) return true;
-    *alpha_o = o.alpha;
-    *cdef_o = o.cdef;
-    *beta_next_o = o.beta_next;
-    return false;
+    return stop;
 }
 
-// Columns per finalize block: 32, or the next power of two >= ld for narrower tiles, so
-// that the remaining threads of the block split the sum over the SpMM blocks.
+// Columns per finalize block: 8 (one 64-byte segment of the block partials), or the next power
+// of two >= ld for narrower tiles; the other threads of the block split the sum over the SpMM
+// blocks. The kernel is bound by latency (a few dozen dependent loads and FP64 operations), so
+// the sum is spread wide: 64 columns and 608 partials took 12 us on 2 blocks of 32 columns.
 __host__ __device__ inline int fin_cols_per_block(int64_t ld)
 {
     int cb = 1;
-    while (cb < ld && cb < 32) cb <<= 1;
+    while (cb < ld && cb < 8) cb <<= 1;
     return cb;
 }
 
+// In the device-resident loop (a.loop) the last block also decides how the loop goes on after
+// step j (the step's count of active pairs is then complete), advances the step index and
+// sets the index the step's normalise pass reads: the body of a step is then three or four
+// kernels (pre-pass, SpMM, finalize, normalise) with no single-thread kernels between them.
+// The test for a column compaction before step j + 1 reads the count `lag` steps back, as
+// rd_query's host polls do, so that both pack the columns at the same step; when one is due, the
+// step's normalise pass is left to the host, which runs it fused with the packing. To stop, record
+// j (or j + 1 when nothing is left to do), the count the test read, the count entering the next
+// step and which of the two it is in saved[0..3], and park the step index at the sentinel
+// k_max + 1, whose active count is always 0, so that the remaining kernels of the body return.
 template <typename T>
 __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
 {
@@ -282,74 +313,94 @@ __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
         const int64_t slab = col / a.tp, cin = col % a.tp;
         const double* base = a.block_part + slab * a.nblocks * 3 * a.tp + cin;
         const int64_t bstride = 3 * (int64_t)a.tp;
-        int b = split;
-        for (; b + 3 * nsplit < a.nblocks; b += 4 * nsplit) {
+        for (int b = split; b < a.nblocks; b += 4 * nsplit) {
             double x[4][3];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const double* bp = base + (int64_t)(b + u * nsplit) * bstride;
-                x[u][0] = bp[0];
-                x[u][1] = bp[a.tp];
-                x[u][2] = bp[2 * a.tp];
+                if (b + u * nsplit < a.nblocks) {
+                    const double* bp = base + (int64_t)(b + u * nsplit) * bstride;
+                    x[u][0] = bp[0];
+                    x[u][1] = bp[a.tp];
+                    x[u][2] = bp[2 * a.tp];
+                }
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                s0 += x[u][0];
-                s1 += x[u][1];
-                s2 += x[u][2];
+                if (b + u * nsplit < a.nblocks) {
+                    s0 += x[u][0];
+                    s1 += x[u][1];
+                    s2 += x[u][2];
+                }
             }
-        }
-        for (; b < a.nblocks; b += nsplit) {
-            const double* bp = base + (int64_t)b * bstride;
-            s0 += bp[0];
-            s1 += bp[a.tp];
-            s2 += bp[2 * a.tp];
         }
     }
     part[0][threadIdx.x] = s0;
     part[1][threadIdx.x] = s1;
     part[2][threadIdx.x] = s2;
     __syncthreads();
-    // fixed-order tree over the splits
-    for (int h = nsplit >> 1; h >= 1; h >>= 1) {
-        if (split < h) {
-            part[0][threadIdx.x] += part[0][threadIdx.x + h * cb];
-            part[1][threadIdx.x] += part[1][threadIdx.x + h * cb];
-            part[2][threadIdx.x] += part[2][threadIdx.x + h * cb];
-        }
+    // fixed-order tree over the splits; the three sums go to different warps
+    for (int w = 128; w >= cb; w >>= 1) {
+        for (int i = threadIdx.x; i < 3 * w; i += 256) part[i / w][i % w] += part[i / w][i % w + w];
         __syncthreads();
     }
-    if (split != 0 || col >= a.ld) return;
-    const int p = a.slot_pair ? a.slot_pair[col] : (col < a.npairs ? (int)col : -1);
-    if (p < 0 || !st.active[p]) return;
-    const double A = part[0][lane], B = part[1][lane], C = part[2][lane];
-    const int64_t ld = a.ld;
-    const int64_t cfo = a.step_dev ? (int64_t)j * a.cf_stride : 0;
-    T* cfs = static_cast<T*>(a.cf_step) + cfo;
-    T* cfn = static_cast<T*>(a.cf_next) + cfo;
-    // factors of the previous step, for the potential's direct update below
-    const double lam = j > 0 ? st.beta[p] / st.delta[p] : 0.0;
-    double alpha, cdef, beta_next;
-    const bool stop = pair_update(a, st, p, j, A, B, C, &alpha, &cdef, &beta_next);
-    if (a.xcf && st.status[p] != RD_ERR_NUMERIC) {
-        // p_i = q_i + lambda_i p_{i-1}, x += mu_i p_i (a stopping step still contributes)
-        T* xc = static_cast<T*>(a.xcf) + (int64_t)j * 2 * ld;
-        xc[col] = (T)lam;
-        xc[ld + col] = (T)(sqrt(st.b2[p]) * st.g[p] / st.delta[p]);
+    const int p = split != 0 || col >= a.ld
+                      ? -1
+                      : (a.slot_pair ? a.slot_pair[col] : (col < a.npairs ? (int)col : -1));
+    if (p >= 0 && st.active[p]) {
+        const double A = part[0][lane], B = part[1][lane], C = part[2][lane];
+        const int64_t ld = a.ld;
+        const int64_t cfo = a.step_dev ? (int64_t)j * a.cf_stride : 0;
+        T* cfs = static_cast<T*>(a.cf_step) + cfo;
+        T* cfn = static_cast<T*>(a.cf_next) + cfo;
+        // factors of the previous step, for the potential's direct update below
+        const double lam = a.xcf && j > 0 ? st.beta[p] * st.inv_delta[p] : 0.0;
+        StepCoef k;
+        PairStepOut o;
+        const bool stop = pair_update(a, st, p, j, A, B, C, k, o);
+        if (a.xcf && o.ok) {
+            // p_i = q_i + lambda_i p_{i-1}, x += mu_i p_i (a stopping step still contributes)
+            T* xc = static_cast<T*>(a.xcf) + (int64_t)j * 2 * ld;
+            xc[col] = (T)lam;
+            xc[ld + col] = (T)(st.bnorm[p] * o.gd);
+        }
+        if (stop) {
+            // zero coefficients: the column's vectors become (and stay) zero
+            cfs[1 * ld + col] = T(0);
+            cfs[2 * ld + col] = T(0);
+            cfs[3 * ld + col] = T(0);
+            cfn[col] = T(0);
+        } else {
+            cfs[1 * ld + col] = (T)k.alpha;
+            cfs[2 * ld + col] = (T)k.cdef;
+            cfs[3 * ld + col] = (T)k.inv_beta;
+            cfn[col] = (T)k.beta;
+            atomicAdd(&st.act_count[j + 1], 1);
+        }
     }
-    if (stop) {
-        // zero coefficients: the column's vectors become (and stay) zero
-        cfs[1 * ld + col] = T(0);
-        cfs[2 * ld + col] = T(0);
-        cfs[3 * ld + col] = T(0);
-        cfn[col] = T(0);
-        return;
+    if (!a.loop) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    if (atomicAdd(a.loop_ticket, 1) != (int)gridDim.x - 1) return;
+    *a.loop_ticket = 0;
+    __threadfence();
+    const volatile int32_t* act_count = st.act_count;
+    const int jn = j + 1;
+    const int act = act_count[jn];
+    const int act_lag = act_count[jn >= a.loop_lag ? jn - a.loop_lag : 0];
+    const bool more = act > 0 && jn < a.k_max;
+    const bool compact_due = a.loop_compact && jn >= a.loop_lag + 1 && jn >= *a.loop_cfrom && a.ld > 16 &&
+                             (int64_t)act_lag * 2 <= a.ld;
+    const bool pack = more && compact_due;
+    *a.loop_norm = pack ? a.k_max + 1 : j;
+    *a.loop_step = more && !pack ? jn : a.k_max + 1;
+    if (pack || !more) {
+        a.loop_saved[0] = pack ? j : jn;
+        a.loop_saved[1] = act_lag;
+        a.loop_saved[2] = act;
+        a.loop_saved[3] = pack ? 1 : 0;
     }
-    cfs[1 * ld + col] = (T)alpha;
-    cfs[2 * ld + col] = (T)cdef;
-    cfs[3 * ld + col] = (T)(1.0 / beta_next);
-    cfn[col] = (T)beta_next;
-    atomicAdd(&st.act_count[j + 1], 1);
+    cudaGraphSetConditional((cudaGraphConditionalHandle)a.loop_handle, more && !pack ? 1 : 0);
 }
 
 void launch_finalize(cudaStream_t st, const FinArgs& a)
@@ -513,55 +564,31 @@ __global__ void k_step_advance(int32_t* step, int limit)
 
 void launch_step_advance(cudaStream_t st, int32_t* step, int limit) { k_step_advance<<<1, 1, 0, st>>>(step, limit); }
 
-// Conditions of the device-resident step loop (a conditional while node of a CUDA graph).
-// Before step j (j steps done): go on while pairs are active, k_max is not reached and no
-// column compaction is due. After step j's finalize: stop when a compaction is due before step
-// j + 1 (and step j + 1 is to run), leaving step j's normalise pass to the host, which runs it
-// fused with the packing. The compaction test reads the count `lag` steps back (active pairs
-// fit in half the width), as rd_query's host polls do, so that both pack the columns at the
-// same step; it is skipped before step *compact_from (the host moves that past a step where it
-// packed, or found no narrower layout). To stop, record j, the count the test read, the count
-// entering the next step, and where the loop stopped in saved[0..3] (one read for the host),
-// and move the step index to the sentinel k_max + 1, whose active count is always 0, so that
-// the remaining kernels of the loop body return at once; an index at the sentinel stays there.
-__global__ void k_loop_cond(cudaGraphConditionalHandle h, int32_t* step, const int32_t* act_count, int32_t* saved,
-                            const int32_t* compact_from, int k_max, int64_t ld, int compact_check, int lag,
-                            int after_finalize)
+// Entry of the device-resident step loop (before its conditional while node; k_finalize decides
+// after every step): whether step j = *step runs at all. It does not when every pair has
+// stopped, k_max is reached or a column compaction is due before it (tested as in k_finalize,
+// and skipped before step *compact_from: the host moves that past a step where it packed, or
+// found no narrower layout).
+__global__ void k_loop_entry(const FinArgs a)
 {
-    const int j = *step;
-    if (j > k_max) {
-        cudaGraphSetConditional(h, 0);
-        return;
+    const int j = *a.loop_step;
+    const int32_t* act_count = a.st.act_count;
+    const int act = act_count[j];
+    const int act_lag = act_count[j >= a.loop_lag ? j - a.loop_lag : 0];
+    const bool compact_due = a.loop_compact && j >= a.loop_lag + 1 && j >= *a.loop_cfrom && a.ld > 16 &&
+                             (int64_t)act_lag * 2 <= a.ld;
+    const bool go = act > 0 && j < a.k_max && !compact_due;
+    if (!go) {
+        a.loop_saved[0] = j;
+        a.loop_saved[1] = act_lag;
+        a.loop_saved[2] = act;
+        a.loop_saved[3] = 0;
+        *a.loop_step = a.k_max + 1;
     }
-    const int jn = j + after_finalize;  // the step the test is for
-    const int act = act_count[jn];
-    const bool compact_due = compact_check && jn >= lag + 1 && jn >= *compact_from && ld > 16 &&
-                             (int64_t)act_count[jn - lag] * 2 <= ld;
-    bool stop;
-    if (after_finalize) {
-        stop = compact_due && act > 0 && jn < k_max;  // otherwise the next condition decides
-    } else {
-        stop = act == 0 || j >= k_max || compact_due;
-    }
-    if (stop) {
-        saved[0] = j;
-        saved[1] = act_count[jn >= lag ? jn - lag : 0];
-        saved[2] = act;
-        saved[3] = after_finalize;
-        *step = k_max + 1;
-        cudaGraphSetConditional(h, 0);
-    } else if (!after_finalize) {
-        cudaGraphSetConditional(h, 1);
-    }
+    cudaGraphSetConditional((cudaGraphConditionalHandle)a.loop_handle, go ? 1 : 0);
 }
 
-void launch_loop_cond(cudaStream_t st, cudaGraphConditionalHandle h, int32_t* step, const int32_t* act_count,
-                      int32_t* saved, const int32_t* compact_from, int k_max, int64_t ld, int compact_check, int lag,
-                      int after_finalize)
-{
-    k_loop_cond<<<1, 1, 0, st>>>(h, step, act_count, saved, compact_from, k_max, ld, compact_check, lag,
-                                 after_finalize);
-}
+void launch_loop_entry(cudaStream_t st, const FinArgs& a) { k_loop_entry<<<1, 1, 0, st>>>(a); }
 
 // ------------------------------------------------------- sparse first step
 // q_1 is nonzero only in rows s and t of its column, so the first product
@@ -1204,7 +1231,7 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
 {
     extern __shared__ __align__(16) unsigned char onchip_raw[];
     __shared__ double red[3][kOnchipThreads / 32];
-    __shared__ double coef[3];
+    __shared__ double coef[4];
     __shared__ int stop_s;
     const int p = blockIdx.x;
     const PairState& st = a.fin.st;
@@ -1289,16 +1316,17 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
                 B += red[1][w];
                 C += red[2][w];
             }
-            double al = 0.0, cd = 0.0, bn = 0.0;
-            const bool stop = pair_update(a.fin, st, p, j, A, B, C, &al, &cd, &bn);
-            stop_s = stop ? 1 : 0;
-            coef[0] = al;
-            coef[1] = cd;
-            coef[2] = bn;
+            StepCoef k;
+            PairStepOut o;
+            stop_s = pair_update(a.fin, st, p, j, A, B, C, k, o) ? 1 : 0;
+            coef[0] = k.alpha;
+            coef[1] = k.cdef;
+            coef[2] = k.beta;
+            coef[3] = k.inv_beta;
         }
         __syncthreads();
         if (stop_s) break;
-        const T al = (T)coef[0], cd = (T)coef[1], ib = (T)(1.0 / coef[2]);
+        const T al = (T)coef[0], cd = (T)coef[1], ib = (T)coef[3];
         for (int64_t u = tid; u < n; u += nthr) W[u] = (W[u] - al * qc[u] - cd) * ib;
         bt = (T)coef[2];
         const int old_prev = iprev;
@@ -1335,7 +1363,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_lanczos_cluster(const Onchi
     extern __shared__ __align__(16) unsigned char cl_raw[];
     __shared__ double part[kClusterMax][3];
     __shared__ double tpart[3][kClusterThreads];  // per-thread partial sums of the step
-    __shared__ double coef[3];
+    __shared__ double coef[4];
     __shared__ int stop_s;
     __shared__ T* rbase[3][kClusterMax];  // generic addresses of every rank's buffers
     const int C = L.C;
@@ -1454,17 +1482,19 @@ __global__ void __launch_bounds__(kClusterThreads) k_lanczos_cluster(const Onchi
                 B += part[rr][1];
                 Cs += part[rr][2];
             }
+            const StepCoef k = step_coef(a.fin, A, B, Cs);
             PairStepOut o;
-            const bool stop = pair_core(a.fin, ps, j, A, B, Cs, o);
+            const bool stop = pair_core(a.fin, ps, j, k, o);
             if (rank == 0) pair_store(st, p, j, a.fin.pstride, ps, o, stop);
             stop_s = stop ? 1 : 0;
-            coef[0] = o.alpha;
-            coef[1] = o.cdef;
-            coef[2] = o.beta_next;
+            coef[0] = k.alpha;
+            coef[1] = k.cdef;
+            coef[2] = k.beta;
+            coef[3] = k.inv_beta;
         }
         __syncthreads();
         if (stop_s) break;  // the same decision in every CTA of the cluster
-        const T al = (T)coef[0], cd = (T)coef[1], ib = (T)(1.0 / coef[2]);
+        const T al = (T)coef[0], cd = (T)coef[1], ib = (T)coef[3];
         for (int64_t ul = tid; ul < nrow; ul += nthr) W[ul] = (W[ul] - al * qc[ul] - cd) * ib;
         bt = (T)coef[2];
         const int old_prev = iprev;
