@@ -35,7 +35,6 @@ rd_status cuda_status(cudaError_t e, const char* what)
 }
 
 rd_status check_csr(rd_graph* g, cudaStream_t st, int64_t* self_loops);
-rd_status compute_degrees(rd_graph* g, cudaStream_t st);
 int spmm_blocks_per_sm_f32(const SpmmCfg& c, bool weighted, bool heavy);
 int spmm_blocks_per_sm_f64(const SpmmCfg& c, bool weighted, bool heavy);
 int spmm_blocks_per_sm_df64(const SpmmCfg& c, bool weighted, bool heavy);
@@ -117,7 +116,7 @@ static void free_graph(rd_graph* g)
     if (!g) return;
     void* ptrs[] = {g->row_ptr, g->col, g->w, g->keep_idx, g->deg64, g->invdeg64, g->deg32, g->invdeg32,
                     g->comp, g->heavy_rows, g->heavy_first, g->chunk_beg, g->chunk_end, g->task_row,
-                    g->row_order, g->entry_row, g->degdf, g->invdegdf, g->ws.base};
+                    g->row_order, g->entry_row, g->degdf, g->invdegdf, g->ws.base, g->mirror, g->check_scratch};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (g->h_pinned) cudaFreeHost(g->h_pinned);
@@ -249,6 +248,11 @@ static rd_status symmetric_check(int64_t n, const std::vector<int64_t>& rp, cons
     return RD_OK;
 }
 
+static double* degree_sums(const rd_graph* g)
+{
+    return reinterpret_cast<double*>(static_cast<char*>(g->check_scratch) + kCheckFlagsBytes);
+}
+
 static rd_status graph_build(rd_graph* g, const int64_t* row_ptr, const int32_t* col_idx, const float* weights,
                              uint32_t flags, cudaStream_t st)
 {
@@ -311,9 +315,10 @@ static rd_status graph_build(rd_graph* g, const int64_t* row_ptr, const int32_t*
     RD_CUDA(cudaMalloc((void**)&g->invdeg64, sizeof(double) * n));
     RD_CUDA(cudaMalloc((void**)&g->deg32, sizeof(float) * n));
     RD_CUDA(cudaMalloc((void**)&g->invdeg32, sizeof(float) * n));
-    RD_TRY(compute_degrees(g, st));
     RD_TRY(build_heavy(g, rp));
-    RD_TRY(rows_sorted_symmetric(g, st, &g->rows_sorted_sym));
+    RD_CUDA(cudaMalloc(&g->check_scratch, kCheckFlagsBytes + sizeof(double) * degree_grid(g)));
+    RD_TRY(compute_degrees(g, st, g->check_scratch, degree_sums(g), false));
+    RD_TRY(rows_sorted_symmetric(g, st));
     if (flags & RD_LABEL_COMPONENTS) {
         std::vector<int32_t> lab;
         g->ncomp = label_components(n, rp, col, lab);
@@ -1815,15 +1820,17 @@ rd_status rd_graph_set_weights(rd_graph* g, const float* weights, void* stream)
         RD_CUDA(cudaMemcpyAsync(g->w, weights, sizeof(float) * g->nnz, cudaMemcpyDefault, st));
     }
     g->weighted = true;
-    int64_t loops = 0;
-    RD_TRY(check_csr(g, st, &loops));
-    RD_TRY(compute_degrees(g, st));
+    // the structure was checked when the graph was made; where its mirrors are known, one pass
+    // over the weights checks them and takes the degrees
+    const bool searched = !g->mirror_ok;
+    RD_TRY(compute_degrees(g, st, g->check_scratch, degree_sums(g), true));
     if (g->degdf) {  // the double-float copies follow the new degrees
         const int grid = std::max(1, std::min(g->sm_count * 8, (int)((g->n + 255) / 256)));
         launch_split_df(st, grid, g->n, g->deg64, g->degdf);
         launch_split_df(st, grid, g->n, g->invdeg64, g->invdegdf);
+        RD_CUDA(cudaStreamSynchronize(st));
     }
-    return rows_sorted_symmetric(g, st, &g->rows_sorted_sym);
+    return searched ? rows_sorted_symmetric(g, st) : RD_OK;
 }
 
 rd_status rd_graph_destroy(rd_graph* g)
@@ -2247,9 +2254,6 @@ extern "C" rd_status rd_triangle_weights(const rd_graph* g, float* w_out, void* 
 namespace rd {
 
 rd_status check_csr_scratch(rd_graph* g, cudaStream_t st, void* flags_dev, int64_t* self_loops);
-rd_status compute_degrees_scratch(rd_graph* g, cudaStream_t st, void* flags_dev, double* block_sums_dev,
-                                  double* block_sums_host);
-int degree_grid(const rd_graph* g);
 
 // 32 MiB of scratch, held by every GPU that loads this library until the process exits.
 constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
@@ -2317,7 +2321,6 @@ extern "C" rd_status rd_query_noalloc(int64_t n, int64_t nnz, const int64_t* row
     g.w = const_cast<float*>(weights);
     g.heavy_thr = INT32_MAX;  // no heavy-row chunk lists: the row-group kernel takes every row whole
     static thread_local int host_poll[16];
-    static thread_local double host_block_sums[1 << 14];
     g.h_pinned = host_poll;
 
     rd_query_opts o;
@@ -2333,7 +2336,7 @@ extern "C" rd_status rd_query_noalloc(int64_t n, int64_t nnz, const int64_t* row
     RD_TRY(noalloc_scratch_address(g.device, &base));
     // graph-derived arrays first, then the query workspace (same layout as rd_query's)
     Carver cg(base);
-    void* flags_dev = cg.take<char>(64);
+    void* flags_dev = cg.take<char>(kCheckFlagsBytes);
     double* bsum = cg.take<double>(1 << 14);
     g.deg64 = cg.take<double>(n);
     g.invdeg64 = cg.take<double>(n);
@@ -2363,7 +2366,7 @@ extern "C" rd_status rd_query_noalloc(int64_t n, int64_t nnz, const int64_t* row
         set_error("the CSR holds self-loops; rd_query_noalloc cannot rebuild it (use rd_graph_create)");
         return RD_ERR_UNSUPPORTED;
     }
-    RD_TRY(compute_degrees_scratch(&g, st, flags_dev, bsum, host_block_sums));
+    RD_TRY(compute_degrees(&g, st, flags_dev, bsum, false));
     g.ws.base = static_cast<char*>(base) + graph_bytes;
     g.ws.bytes = kNoAllocScratchBytes - graph_bytes;  // >= query_bytes, so nothing is allocated
     EventPool ev;

@@ -287,6 +287,9 @@ struct rd_graph {
     rd::df64* degdf = nullptr;        // double-float copies (built on first use)
     rd::df64* invdegdf = nullptr;
     double sumdeg = 0.0;
+    int32_t* mirror = nullptr;        // weighted graphs: entry (v, u) of each entry (u, v)
+    bool mirror_ok = false;           // rows sorted and the structure symmetric: mirror is whole
+    void* check_scratch = nullptr;    // flags and block sums of compute_degrees
     int32_t* comp = nullptr;
     int32_t ncomp = 0;
     // heavy-row chunks
@@ -450,8 +453,9 @@ void launch_step0_f64(cudaStream_t st, const Step0Args<double>& a);
 void launch_step0_df64(cudaStream_t st, const Step0Args<df64>& a);
 
 // Graph preparation kernels.
-rd_status graph_prepare(rd_graph* g, cudaStream_t st, uint32_t flags);
-rd_status rows_sorted_symmetric(rd_graph* g, cudaStream_t st, bool* out);
-rd_status graph_weights_changed(rd_graph* g, cudaStream_t st);
+constexpr size_t kCheckFlagsBytes = 64;
+rd_status rows_sorted_symmetric(rd_graph* g, cudaStream_t st);
+int degree_grid(const rd_graph* g);
+rd_status compute_degrees(rd_graph* g, cudaStream_t st, void* flags_dev, double* block_sums_dev, bool check_weights);
 
 }  // namespace rd

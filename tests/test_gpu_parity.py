@@ -908,3 +908,44 @@ def test_double_float_query_follows_new_weights(rd):
     G.set_weights(g2.w)
     res = G.query(s, t, **kw)
     assert rel(res.r, dense.DenseRD.of(g2).r(s, t)).max() < FP64_TOL
+
+
+@pytest.mark.parametrize("name", ["star700", "chunglu", "path3", "loops"])
+def test_new_weights_checked_and_followed(rd, name):
+    """rd_graph_set_weights in one pass over the weights: the same answers, bit for bit, as a graph
+    created with those weights (rows of one entry up to heavy rows, a first set on an unweighted
+    graph, dropped self-loops); asymmetric weights turn the sparse first step off and symmetric
+    ones on again; a bad weight is refused and the graph still takes good ones."""
+    if name == "chunglu":
+        g, s, t = W.chunglu(20000, 2.1, 20.0, 200000, 9, 77)
+        assert np.diff(g.row_ptr).max() > 256
+    else:
+        g = {"star700": lambda: F.star(700), "path3": lambda: F.path(3),
+             "loops": lambda: F.random_connected(300, 900, 3, None)}[name]()
+        s, t = F.random_pairs(g.n, 4, 3)
+    rp, col = g.row_ptr, g.col
+    w1, w2 = (F.weighted(g, F.lognormal_edge_weights(g.m, 0.0, 0.5, sd)).w for sd in (4, 5))
+    if name == "loops":  # a self-loop at vertex 0, in front of its row
+        col = np.concatenate([[0], col]).astype(np.int32)
+        rp = rp + (np.arange(rp.size) > 0)
+        w1, w2 = (np.concatenate([[1.0], w]).astype(np.float32) for w in (w1, w2))
+    kw = dict(mode="fp64", k_max=30, fixed_k=True, onchip=False, tune=False)
+    G = rd.Graph(rp, col)
+    ref = {k: rd.Graph(rp, col, w).query(s, t, **kw).r for k, w in (("w1", w1), ("w2", w2))}
+    for k, w in (("w1", w1), ("w2", w2), ("w1", w1)):
+        G.set_weights(w)
+        assert np.array_equal(G.query(s, t, **kw).r, ref[k])
+        assert G.last_stats()["sparse_first"] == 1
+    asym = w2.copy()
+    asym[-1] *= 2.0
+    G.set_weights(asym)
+    G.query(s, t, **kw)
+    assert G.last_stats()["sparse_first"] == 0
+    for bad in (0.0, -1.0, np.inf, np.nan):
+        wb = w2.copy()
+        wb[wb.size // 2] = bad
+        with pytest.raises(rd.RDError):
+            G.set_weights(wb)
+    G.set_weights(w2)
+    assert np.array_equal(G.query(s, t, **kw).r, ref["w2"])
+    assert G.last_stats()["sparse_first"] == 1
