@@ -1671,6 +1671,18 @@ static rd_status run_replay(RunCtx& c, int K)
     return RD_OK;
 }
 
+// Row of every stored entry, once per graph, for the per-entry kernels.
+static rd_status ensure_entry_rows(RunCtx& c)
+{
+    rd_graph* g = c.g;
+    if (g->entry_row || g->nnz == 0) return RD_OK;
+    RD_CUDA(cudaMalloc((void**)&g->entry_row, sizeof(int32_t) * g->nnz));
+    launch_entry_rows(std::max(1, std::min(g->sm_count * 8, (int)((g->n + 7) / 8))), c.st, g->n, g->row_ptr,
+                      g->entry_row);
+    ++c.launches;
+    return RD_OK;
+}
+
 static rd_status forward_and_potential(RunCtx& c, const int32_t* s, const int32_t* t, const double* grad_r,
                                        rd_status* call_status)
 {
@@ -1946,12 +1958,7 @@ rd_status rd_edge_grad(rd_graph* g, const int32_t* s, const int32_t* t, int64_t 
     rd_status call = RD_OK;
     RD_TRY(forward_and_potential(c, s, t, grad_r, &call));
     // edge kernel over internal entries, then map to the caller's entry order
-    if (!g->entry_row && g->nnz > 0) {
-        RD_CUDA(cudaMalloc((void**)&g->entry_row, sizeof(int32_t) * g->nnz));
-        launch_entry_rows(std::max(1, std::min(g->sm_count * 8, (int)((g->n + 7) / 8))), st, g->n, g->row_ptr,
-                          g->entry_row);
-        ++c.launches;
-    }
+    RD_TRY(ensure_entry_rows(c));
     const int grid = std::max<int>(1, (int)std::min<int64_t>((int64_t)g->sm_count * 8, (g->nnz + 255) / 256));
     float* gint = c.b.grad;
     if (c.pl.fp64) {
@@ -2002,19 +2009,6 @@ rd_status rd_edge_grad(rd_graph* g, const int32_t* s, const int32_t* t, int64_t 
 
 }  // extern "C"
 
-namespace rd {
-template <typename T>
-__global__ void k_phi_out(int64_t n, int64_t ld, int npairs, const T* phi, float* out)
-{
-    const int64_t total = n * (int64_t)npairs;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-        const int64_t p = i / n, u = i % n;
-        out[i] = (float)phi[u * ld + p];
-    }
-}
-}  // namespace rd
-
 extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs,
                                   const rd_query_opts* opts, float* phi_out, double* r_out, void* stream)
 {
@@ -2044,9 +2038,14 @@ extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* 
     } else {
         RD_CUDA(cudaMallocAsync((void**)&stage, bytes, st));
     }
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g->sm_count * 8, (g->n * npairs + 255) / 256));
-    if (c.pl.fp64) k_phi_out<double><<<grid, 256, 0, st>>>(g->n, c.pl.ld, (int)npairs, static_cast<double*>(c.b.phi), stage);
-    else k_phi_out<float><<<grid, 256, 0, st>>>(g->n, c.pl.ld, (int)npairs, static_cast<float*>(c.b.phi), stage);
+    PairMajorArgs pa{};
+    pa.items = g->n;
+    pa.ld = c.pl.ld;
+    pa.npairs = (int)npairs;
+    pa.phi = c.b.phi;
+    pa.out = stage;
+    pa.out_stride = g->n;
+    launch_pair_major(st, c.pl.fp64, pa);
     ++c.launches;
     if (!dev_out) {
         RD_CUDA(cudaMemcpyAsync(phi_out, stage, bytes, cudaMemcpyDeviceToHost, st));
@@ -2057,27 +2056,6 @@ extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* 
     record_stats(c);
     return outs;
 }
-
-namespace rd {
-// Potential differences along every stored entry (Section 6.3, Definition electric_flow:
-// f(e) = phi(u) - phi(v) for e = (u, v)); one warp per row, lanes over the row's entries,
-// output pair-major in the caller's entry order (dropped self-loops get 0).
-template <typename T>
-__global__ void k_flow(int64_t n, int64_t ld, int npairs, int64_t nnz_in, const int64_t* row_ptr,
-                       const int32_t* col, const int64_t* keep_idx, const T* phi, float* out)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps) {
-        for (int64_t e = row_ptr[u] + lane; e < row_ptr[u + 1]; e += 32) {
-            const int64_t v = col[e];
-            const int64_t oe = keep_idx ? keep_idx[e] : e;
-            for (int p = 0; p < npairs; ++p)
-                out[(int64_t)p * nnz_in + oe] = (float)(phi[u * ld + p] - phi[v * ld + p]);
-        }
-    }
-}
-}  // namespace rd
 
 extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs,
                              const rd_query_opts* opts, float* flow_out, double* r_out, void* stream)
@@ -2104,13 +2082,18 @@ extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, in
     float* stage = dev_out ? flow_out : nullptr;
     if (!dev_out && bytes) RD_CUDA(cudaMallocAsync((void**)&stage, bytes, st));
     if (g->keep_idx && bytes) RD_CUDA(cudaMemsetAsync(stage, 0, bytes, st));
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g->sm_count * 8, (g->n + 7) / 8));
-    if (c.pl.fp64)
-        k_flow<double><<<grid, 256, 0, st>>>(g->n, c.pl.ld, (int)npairs, g->nnz_in, g->row_ptr, g->col, g->keep_idx,
-                                             static_cast<const double*>(c.b.phi), stage);
-    else
-        k_flow<float><<<grid, 256, 0, st>>>(g->n, c.pl.ld, (int)npairs, g->nnz_in, g->row_ptr, g->col, g->keep_idx,
-                                            static_cast<const float*>(c.b.phi), stage);
+    RD_TRY(ensure_entry_rows(c));
+    PairMajorArgs pa{};
+    pa.items = g->nnz;
+    pa.ld = c.pl.ld;
+    pa.npairs = (int)npairs;
+    pa.phi = c.b.phi;
+    pa.row = g->entry_row;
+    pa.col = g->col;
+    pa.keep_idx = g->keep_idx;
+    pa.out = stage;
+    pa.out_stride = g->nnz_in;
+    launch_pair_major(st, c.pl.fp64, pa);
     ++c.launches;
     if (!dev_out && bytes) {
         RD_CUDA(cudaMemcpyAsync(flow_out, stage, bytes, cudaMemcpyDeviceToHost, st));

@@ -412,6 +412,19 @@ void launch_edge_grad_f64(int grid, cudaStream_t st, const EdgeGradArgs<double>&
 void launch_entry_rows(int grid, cudaStream_t st, int64_t n, const int64_t* row_ptr, int32_t* entry_row);
 
 
+// Pair-major float output of the potential block: out[p][i] = phi[i][p] of vertex i (potentials),
+// or, with `row`, phi[row[i]][p] - phi[col[i]][p] of entry i, stored at keep_idx[i] (flows).
+struct PairMajorArgs {
+    int64_t items, ld, out_stride;
+    int npairs;
+    const void* phi;              // T n x ld
+    const int32_t* row;           // nullable
+    const int32_t* col;
+    const int64_t* keep_idx;      // nullable: identity
+    float* out;
+};
+void launch_pair_major(cudaStream_t st, bool fp64, const PairMajorArgs& a);
+
 // First Lanczos step from the sparse start vector (two nonzeros per column).
 template <typename T>
 struct Step0Args {

@@ -949,3 +949,34 @@ def test_new_weights_checked_and_followed(rd, name):
     G.set_weights(w2)
     assert np.array_equal(G.query(s, t, **kw).r, ref["w2"])
     assert G.last_stats()["sparse_first"] == 1
+
+
+@pytest.mark.parametrize("mode", ["fp32", "fp64"])
+@pytest.mark.parametrize("pairs", [1, 3, 31, 33, 70])
+def test_pair_major_outputs(rd, mode, pairs):
+    """The transposed outputs of potentials and flows at the edges of their tiles (128 items by 32
+    pairs; vertex and entry counts no multiple of 128; dropped self-loops): each pair's row is the
+    one the pair has alone, and every flow is the difference of its two potentials."""
+    g = F.random_connected(301, 700, 23, "lognormal")
+    rows = np.concatenate([g.rows(), [7, 300]])
+    cols = np.concatenate([g.col, [7, 300]])
+    order = np.lexsort((cols, rows))
+    rows, cols = rows[order], cols[order].astype(np.int32)
+    w = np.concatenate([g.w, [1.0, 1.0]]).astype(np.float32)[order]
+    rp = np.zeros(g.n + 1, np.int64)
+    np.cumsum(np.bincount(rows, minlength=g.n), out=rp[1:])
+    G = rd.Graph(rp, cols, w)
+    assert G.nnz == g.nnz and g.nnz % 128 and g.n % 128
+    s, t = F.random_pairs(g.n, pairs, 8)
+    kw = dict(mode=mode, k_max=40, fixed_k=True)
+    phi, _ = G.potential(s, t, **kw)
+    f, _ = G.flow(s, t, **kw)
+    # FP32 potentials subtract exactly as the kernel subtracts them; FP64 ones are rounded to
+    # float first here (one rounding each, relative to the potential) and after in the kernel
+    tol = 0.0 if mode == "fp32" else 3 * 2.0**-24 * np.abs(phi).max()
+    assert np.abs(f - (phi[:, rows] - phi[:, cols])).max() <= tol
+    assert np.all(f[:, rows == cols] == 0.0)
+    for p in {0, pairs // 2, pairs - 1}:
+        one, _ = G.potential(s[p:p + 1], t[p:p + 1], **kw)
+        # the narrower kernel sums in another order: 40 steps of FP32 (FP64) rounding
+        assert np.abs(one[0] - phi[p]).max() < (1e-4 if mode == "fp32" else 1e-6) * np.abs(phi[p]).max()
