@@ -1223,6 +1223,7 @@ static rd_status run_forward(RunCtx& c)
     if (c.onchip) {
         OnchipArgs oa{};
         oa.n = c.g->n;
+        oa.nnz = c.g->nnz;
         oa.npairs = (int)c.P;
         oa.row_ptr = c.g->row_ptr;
         oa.col = c.g->col;

@@ -203,7 +203,7 @@ struct FinArgs {
 // Whole recurrence of one pair per CTA with q_{i-1}, q_i and W in shared memory (graphs
 // small enough); reads the CSR from global memory (L1/L2 resident).
 struct OnchipArgs {
-    int64_t n;
+    int64_t n, nnz;
     int npairs;
     const int64_t* row_ptr;
     const int32_t* col;

@@ -5,8 +5,6 @@
 // potential of Algorithm 5 and the edge-weight gradient.
 #include <math.h>
 
-#include <cooperative_groups.h>
-
 #include "spmm.cuh"
 
 namespace rd {
@@ -138,15 +136,29 @@ struct StepCoef {
     double alpha, cdef, beta2, beta, inv_beta;
 };
 
+// beta_{i+1} and its reciprocal by one rsqrt (366 cycles) with a Newton correction each, which
+// leaves both within rounding of sqrt and 1/sqrt (610 and 365 cycles): this chain stands between
+// the sums and the next vector.
 __device__ __forceinline__ StepCoef step_coef(const FinArgs& a, double A, double B, double C)
 {
     StepCoef k;
     k.alpha = A;
     k.cdef = a.deflate ? C * a.inv_sumdeg : 0.0;
     const double gamma2 = a.deflate ? C * k.cdef : 0.0;
-    k.beta2 = B - A * A - gamma2;
-    k.beta = sqrt(fmax(k.beta2, 0.0));
-    k.inv_beta = 1.0 / k.beta;  // not used when beta is 0 (the step is a breakdown) or not finite
+    const double b2 = B - A * A - gamma2;
+    k.beta2 = b2;
+    // zero, negative, denormal and non-finite squares (decided on the exponent bits): the plain
+    // forms, or a step that stops and uses neither
+    const int hi = __double2hiint(b2);
+    if (hi >= 0x00200000 && hi < 0x7ff00000) {
+        const double r = rsqrt(b2);
+        const double b = b2 * r;
+        k.beta = fma(0.5 * r, fma(-b, b, b2), b);
+        k.inv_beta = fma(r, fma(-k.beta, r, 1.0), r);
+    } else {
+        k.beta = sqrt(fmax(b2, 0.0));
+        k.inv_beta = 1.0 / k.beta;  // not used when beta is 0 (the step is a breakdown) or not finite
+    }
     return k;
 }
 
@@ -1400,177 +1412,315 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
 }
 
 // ---------------------------------------------------- on chip, one cluster per pair
-// The same recurrence for one pair spread over a thread-block cluster of C CTAs (C = 2..16):
-// CTA r holds rows [r R, (r+1) R) of q_{i-1}, q_i and W in its shared memory (R a power of
-// two), and the product gathers q_i[col] from the owning CTA's shared memory through the
-// cluster's distributed shared memory. Per step: every CTA's three FP64 block sums are
-// written into every CTA of the cluster, a cluster barrier, every CTA sums the C partials in
-// rank order and runs the same scalar update (pair_core) on its own copy of the pair's
-// scalars (identical inputs, identical results; rank 0 also stores them), normalises its
-// rows in place, and a second cluster barrier publishes the new vector. The FP64 work of a
-// step is spread over C SMs (one CTA per SM) instead of one.
-constexpr int kClusterThreads = 256;
+// The whole recurrence of one pair on a thread-block cluster of C CTAs (C = 1..16): CTA r holds
+// rows [r R, (r+1) R) of q_{i-1}, q_i and W, of d and 1/d, and (where they fit) of the CSR in its
+// shared memory. Per step: every CTA's three FP64 block sums are written into every CTA of the
+// cluster, a cluster barrier, every CTA sums the C partials in rank order and forms the same
+// coefficients and normalises its rows, and a second cluster barrier publishes the vector.
+//
+// A product reads q_i[col] in one of two ways. COPY: every CTA holds a whole copy of q_i, and the
+// normalise pass writes its rows into all C copies (whole segments, n (C - 1) / C elements into
+// each SM). Otherwise: each entry's column is kept as the 32-bit address of its element in the
+// owning CTA's shared memory and loaded through distributed shared memory (nnz / C single
+// elements into each SM). An element costs about half a cycle either way (measured on a first
+// form of the kernel: 64x64 grid, FP64, C = 16, 4.1 us a step with gathers and 5.3 with copies;
+// 1,000 vertices, 13,800 entries, FP32, C = 2, a query of 64 pairs x 20 steps 341 us with
+// gathers and 297 with copies), so the copies are
+// taken when n (C - 1) <= nnz.
+//
+// What bounds a step is the FP64 unit: an FP64 instruction of one warp occupies a quarter SM for
+// about 64 cycles (19 of the SM's) whatever the number of active lanes, an add has 57 cycles of
+// latency, a reciprocal 365, a square root 610 (measured). So the chain from the sums to the
+// next vector is kept to what it needs:
+//  - each of the three block sums is taken by one warp on its own quarter of the SM, and the
+//    C x 3 partials of the cluster by one warp (eight lanes a sum);
+//  - only alpha, c, beta and 1/beta are formed before the next vector (step_coef); the LDL^T
+//    update, the estimate and the stop test of step j - 1 (pair_core, three divisions) run in a
+//    fourth warp beside the sums of step j, so a pair stops one product late;
+// 64x64 grid, FP64, 16 CTAs: 8.0 us a step before (every partial and division on one thread's
+// chain, 39 FP64 instructions for the block sums, the CSR read from global memory), 4.0 us now:
+// 2,500 cycles for the product, 1,650 for the block sums, 1,300 and 950 for the barriers, 1,650
+// for the coefficients, 700 for the normalise pass. 64 pairs x 20 steps on 1,000 vertices, FP32:
+// 233 us before, 95 us now.
 constexpr int kClusterMax = 16;
+constexpr size_t kClusterSmemMax = 200 * 1024;  // of the 227 KB a block may have
 
 struct ClusterLayout {
-    int shift;        // log2 R: rows per CTA
     int C;            // CTAs per pair
+    int R;            // rows per CTA
+    int nnz_cap;      // entries of the CSR a CTA can hold in shared memory
 };
 
-template <typename T, bool WEIGHTED>
-__global__ void __launch_bounds__(kClusterThreads) k_lanczos_cluster(const OnchipArgs a, const ClusterLayout L)
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank)
 {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
+    uint32_t d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(local), "r"(rank));
+    return d;
+}
+__device__ __forceinline__ float cluster_ld(uint32_t a, float)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ double cluster_ld(uint32_t a, double)
+{
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void cluster_st(uint32_t a, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_st(uint32_t a, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// Bytes of shared memory before the entries: the copy of q_i (n elements, or none), a CTA's rows of
+// three vectors, d and 1/d, and its row offsets.
+__host__ __device__ inline size_t cluster_base_bytes(int64_t ncopy, int R, int elem)
+{
+    return ((((size_t)ncopy + 5 * (size_t)R) * elem + (size_t)4 * (R + 1)) + 15) & ~(size_t)15;
+}
+
+template <typename T, bool WEIGHTED, bool COPY, int NT>
+__global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, const ClusterLayout L)
+{
     extern __shared__ __align__(16) unsigned char cl_raw[];
-    __shared__ double part[kClusterMax][3];
-    __shared__ double tpart[3][kClusterThreads];  // per-thread partial sums of the step
-    __shared__ double coef[4];
+    __shared__ double part[3][kClusterMax];       // every CTA's sums of the step, by rank
+    __shared__ double tpart[3][NT];               // per-thread partial sums of the step
+    __shared__ StepCoef coef;                     // of the step last summed
+    __shared__ T next[4];                         // its 1/beta, alpha, c and beta as vector elements
     __shared__ int stop_s;
-    __shared__ T* rbase[3][kClusterMax];  // generic addresses of every rank's buffers
-    const int C = L.C;
-    const int rank = (int)cluster.block_rank();
+    __shared__ uint32_t rbase[kClusterMax];       // address of every rank's vectors
+    const int C = L.C, R = L.R;
+    const int rank = C > 1 ? blockIdx.x % C : 0;  // clusters are runs of C blocks along x
     const int p = blockIdx.x / C;
     const PairState& st = a.fin.st;
     // uniform over the cluster: no CTA changes active[p] before the first cluster barrier
     if (p >= a.npairs || !st.active[p]) return;
-    const int64_t n = a.n;
-    const int64_t R = (int64_t)1 << L.shift;
-    const int64_t row0 = (int64_t)rank * R;
-    const int64_t nrow = row0 >= n ? 0 : (n - row0 < R ? n - row0 : R);
+    const int n = (int)a.n;
+    const int row0 = rank * R;
+    const int nrow = row0 >= n ? 0 : (n - row0 < R ? n - row0 : R);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int nthr = kClusterThreads, nwarps = kClusterThreads / 32;
-    T* buf0 = reinterpret_cast<T*>(cl_raw);
-    if (tid < 3 * C) {
-        const int b = tid / C, rr = tid % C;
-        rbase[b][rr] = cluster.map_shared_rank(buf0 + b * R, rr);
+    constexpr int nthr = NT, nwarps = NT / 32;
+    constexpr uint32_t E = sizeof(T);
+    const int ncopy = COPY ? n : 0;
+    T* full = reinterpret_cast<T*>(cl_raw);  // q_i, every row (COPY)
+    T* buf0 = full + ncopy;
+    T* s_invd = buf0 + 3 * R;
+    T* s_deg = s_invd + R;
+    int* s_rp = reinterpret_cast<int*>(s_deg + R);
+    // the entries: weights, then the column (COPY) or the address of its element in buffer 0
+    using Col = typename std::conditional<COPY, uint16_t, uint32_t>::type;
+    float* s_w = reinterpret_cast<float*>(cl_raw + cluster_base_bytes(ncopy, R, (int)E));
+    Col* s_col = reinterpret_cast<Col*>(WEIGHTED ? s_w + L.nnz_cap : s_w);
+    if (tid < C) rbase[tid] = cluster_addr(smem_addr(full), tid);  // buf0 where there is no copy
+    for (int u = tid; u < ncopy + 3 * R; u += nthr) full[u] = T(0);
+    const int64_t ebase = nrow > 0 ? a.row_ptr[row0] : 0;
+    for (int u = tid; u <= nrow; u += nthr) s_rp[u] = nrow > 0 ? (int)(a.row_ptr[row0 + u] - ebase) : 0;
+    for (int u = tid; u < nrow; u += nthr) {
+        s_invd[u] = E == 8 ? (T)a.invdeg64[row0 + u] : (T)a.invdeg32[row0 + u];
+        s_deg[u] = E == 8 ? (T)a.deg64[row0 + u] : (T)a.deg32[row0 + u];
     }
-    for (int64_t u = tid; u < 3 * R; u += nthr) buf0[u] = T(0);
+    if (tid == 0) stop_s = 0;
     __syncthreads();
+    const int nent = s_rp[nrow];
+    const bool cached = nent <= L.nnz_cap;
+    auto locate = [&](int e) -> uint32_t {
+        const int v = __ldg(a.col + ebase + e);
+        if constexpr (COPY) return (uint32_t)v;
+        const int r = v / R;
+        return rbase[r] + (uint32_t)(v - r * R) * E;
+    };
+    if (cached)
+        for (int e = tid; e < nent; e += nthr) {
+            s_col[e] = (Col)locate(e);
+            if constexpr (WEIGHTED) s_w[e] = __ldg(a.w + ebase + e);
+        }
     PairScalars ps;
+    if (tid == 96) ps = pair_load(st, p, a.fin.pstride);
     if (tid == 0) {
-        ps = pair_load(st, p, a.fin.pstride);
         const int32_t s = a.s[p], t = a.t[p];
-        const double bn = sqrt(ps.b2);
-        if (s >= row0 && s < row0 + nrow) buf0[R + (s - row0)] = (T)(1.0 / (a.deg64[s] * bn));
-        if (t >= row0 && t < row0 + nrow) buf0[R + (t - row0)] = (T)(-1.0 / (a.deg64[t] * bn));
+        const double bn = st.bnorm[p];
+        const T qs = (T)(1.0 / (a.deg64[s] * bn)), qt = (T)(-1.0 / (a.deg64[t] * bn));
+        if constexpr (COPY) {
+            full[s] = qs;
+            full[t] = qt;
+        }
+        if (s >= row0 && s < row0 + nrow) buf0[R + (s - row0)] = qs;
+        if (t >= row0 && t < row0 + nrow) buf0[R + (t - row0)] = qt;
     }
-    cluster.sync();  // every slice of q_1 is in place
+    cluster_arrive();
+    cluster_wait();  // q_1 is in place, and every CTA of the cluster runs
     int iprev = 0, icur = 1, iw = 2;
-    const int64_t mask = R - 1;
     T bt = T(0);
-    for (int j = 0; j < a.fin.k_max; ++j) {
-        T* const* cur = rbase[icur];
+    // the scalar update of step j (thread 96), stored by rank 0
+    auto update = [&](int j, const StepCoef& k) {
+        PairStepOut o;
+        const bool stop = pair_core(a.fin, ps, j, k, o);
+        if (rank == 0) pair_store(st, p, j, a.fin.pstride, ps, o, stop);
+        return stop;
+    };
+    for (int j = 0;; ++j) {
+        if (j == a.fin.k_max) {  // the last step's update (it stops there)
+            if (tid == 96) update(j - 1, coef);
+            break;
+        }
         const T* qp = buf0 + iprev * R;
         const T* qc = buf0 + icur * R;
         T* W = buf0 + iw * R;
         double pa = 0.0, pb = 0.0, pc = 0.0;
-        for (int64_t ul = tid; ul < nrow; ul += nthr) {
-            const int64_t u = row0 + ul;
-            const int64_t e0 = a.row_ptr[u], e1 = a.row_ptr[u + 1];
-            if (e1 - e0 > a.heavy_thr) continue;
-            T acc = T(0);
-            for (int64_t e = e0; e < e1; ++e) {
-                const int32_t v = __ldg(a.col + e);
-                const T x = cur[v >> L.shift][v & mask];
-                if constexpr (WEIGHTED) acc += (T)__ldg(a.w + e) * x;
-                else acc += x;
-            }
-            const T invd = sizeof(T) == 8 ? (T)a.invdeg64[u] : (T)a.invdeg32[u];
-            const T du = sizeof(T) == 8 ? (T)a.deg64[u] : (T)a.deg32[u];
-            const T wv = invd * acc - bt * qp[ul];
+        bool first = true;
+        auto close_row = [&](int ul, T acc) {
+            const T wv = s_invd[ul] * acc - bt * qp[ul];
             W[ul] = wv;
-            const T dw = du * wv;
-            pa += (double)(dw * qc[ul]);
-            pb += (double)(dw * wv);
-            pc += (double)dw;
-        }
-        for (int64_t h = warp; h < a.n_heavy_rows; h += nwarps) {
-            const int64_t u = a.heavy_rows[h];
-            if (u < row0 || u >= row0 + nrow) continue;
-            T acc = T(0);
-            for (int64_t e = a.row_ptr[u] + lane; e < a.row_ptr[u + 1]; e += 32) {
-                const int32_t v = __ldg(a.col + e);
-                const T x = cur[v >> L.shift][v & mask];
-                if constexpr (WEIGHTED) acc += (T)__ldg(a.w + e) * x;
-                else acc += x;
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) acc += shfl_xor_t(0xffffffffu, acc, off);
-            if (lane == 0) {
-                const int64_t ul = u - row0;
-                const T invd = sizeof(T) == 8 ? (T)a.invdeg64[u] : (T)a.invdeg32[u];
-                const T du = sizeof(T) == 8 ? (T)a.deg64[u] : (T)a.deg32[u];
-                const T wv = invd * acc - bt * qp[ul];
-                W[ul] = wv;
-                const T dw = du * wv;
+            const T dw = s_deg[ul] * wv;
+            if (first) {  // no FP64 addition to zero
+                pa = (double)(dw * qc[ul]);
+                pb = (double)(dw * wv);
+                pc = (double)dw;
+                first = false;
+            } else {
                 pa += (double)(dw * qc[ul]);
                 pb += (double)(dw * wv);
                 pc += (double)dw;
             }
-        }
-        // the CTA's three sums by one warp (FP64 adds are slow here, and the shuffles of the
-        // other warps would contend for the same units): lane l adds threads l, l+32, ... in
-        // order, then a fixed xor tree; lane r < C writes them into slot `rank` of CTA r
+        };
+        const uint32_t cur = (uint32_t)(icur * R) * E;
+        auto fetch = [&](uint32_t at) {
+            if constexpr (COPY) return full[at];
+            else return cluster_ld(at + cur, T(0));
+        };
+        // the rows' products; `held`: the CTA's entries are in shared memory (a branch per entry
+        // would cost more than the loads)
+        auto product = [&](auto held) {
+            auto where = [&](int e) -> uint32_t {
+                if constexpr (decltype(held)::value) return s_col[e];
+                else return locate(e);
+            };
+            auto weight = [&](int e) {
+                if constexpr (decltype(held)::value) return (T)s_w[e];
+                else return (T)__ldg(a.w + ebase + e);
+            };
+            for (int ul = tid; ul < nrow; ul += nthr) {
+                int e = s_rp[ul];
+                const int e1 = s_rp[ul + 1];
+                if (e1 - e > a.heavy_thr) continue;
+                T acc = T(0);
+                // gathers in flight four at a time, added in order; the first is not added to zero
+                auto four = [&](bool open) {
+                    uint32_t at[4];
+                    T x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) at[u] = where(e + u);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = fetch(at[u]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if constexpr (WEIGHTED) {
+                            if (open && u == 0) acc = weight(e) * x[0];
+                            else acc += weight(e + u) * x[u];
+                        } else {
+                            if (open && u == 0) acc = x[0];
+                            else acc += x[u];
+                        }
+                    }
+                    e += 4;
+                };
+                if (e + 4 <= e1) four(true);
+                while (e + 4 <= e1) four(false);
+                for (; e < e1; ++e) {
+                    const T x = fetch(where(e));
+                    if constexpr (WEIGHTED) acc += weight(e) * x;
+                    else acc += x;
+                }
+                close_row(ul, acc);
+            }
+            for (int64_t h = warp; h < a.n_heavy_rows; h += nwarps) {
+                const int ul = a.heavy_rows[h] - row0;
+                if (ul < 0 || ul >= nrow) continue;
+                T acc = T(0);
+                for (int e = s_rp[ul] + lane; e < s_rp[ul + 1]; e += 32) {
+                    const T x = fetch(where(e));
+                    if constexpr (WEIGHTED) acc += weight(e) * x;
+                    else acc += x;
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) acc += shfl_xor_t(0xffffffffu, acc, off);
+                if (lane == 0) close_row(ul, acc);
+            }
+        };
+        if (cached) product(std::true_type{});
+        else product(std::false_type{});
         tpart[0][tid] = pa;
         tpart[1][tid] = pb;
         tpart[2][tid] = pc;
         __syncthreads();
-        if (warp == 0) {
-            double A = 0.0, B = 0.0, Cs = 0.0;
-            for (int w = 0; w < nwarps; ++w) {
-                A += tpart[0][w * 32 + lane];
-                B += tpart[1][w * 32 + lane];
-                Cs += tpart[2][w * 32 + lane];
-            }
+        // one warp a sum, each on its own quarter of the SM: lane l adds threads l, l+32, ... in
+        // order, then a fixed xor tree; lane r < C writes it into slot `rank` of CTA r
+        const bool updates = warp == 3 && j > 0;
+        StepCoef kprev;
+        if (warp < 3) {
+            double s = tpart[warp][lane];
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                A += __shfl_xor_sync(0xffffffffu, A, off);
-                B += __shfl_xor_sync(0xffffffffu, B, off);
-                Cs += __shfl_xor_sync(0xffffffffu, Cs, off);
-            }
-            if (lane < C) {
-                double* dst = cluster.map_shared_rank(&part[0][0], lane);
-                dst[rank * 3 + 0] = A;
-                dst[rank * 3 + 1] = B;
-                dst[rank * 3 + 2] = Cs;
-            }
+            for (int w = 1; w < nwarps; ++w) s += tpart[warp][w * 32 + lane];
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            if (lane < C) cluster_st(cluster_addr(smem_addr(&part[warp][rank]), lane), s);
+        } else if (updates) {
+            kprev = coef;  // rewritten behind the barrier
         }
-        cluster.sync();  // all partial sums have arrived
-        if (tid == 0) {
-            double A = 0.0, B = 0.0, Cs = 0.0;
-            for (int rr = 0; rr < C; ++rr) {
-                A += part[rr][0];
-                B += part[rr][1];
-                Cs += part[rr][2];
-            }
+        __syncwarp();
+        cluster_arrive();
+        if (updates && lane == 0) stop_s = update(j - 1, kprev) ? 1 : 0;
+        __syncwarp();
+        cluster_wait();  // all partial sums have arrived
+        if (warp == 0) {
+            // eight lanes a sum: partials i and i + 8, then a fixed xor tree
+            const int q = lane >> 3, i = lane & 7;
+            double s = 0.0;
+            if (q < 3 && i < C) s = part[q][i];
+            if (C > 8) s += q < 3 ? part[q][i + 8] : 0.0;
+            for (int off = (C < 8 ? C : 8) >> 1; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            const double A = __shfl_sync(0xffffffffu, s, 0), B = __shfl_sync(0xffffffffu, s, 8);
+            const double Cs = __shfl_sync(0xffffffffu, s, 16);
             const StepCoef k = step_coef(a.fin, A, B, Cs);
-            PairStepOut o;
-            const bool stop = pair_core(a.fin, ps, j, k, o);
-            if (rank == 0) pair_store(st, p, j, a.fin.pstride, ps, o, stop);
-            stop_s = stop ? 1 : 0;
-            coef[0] = k.alpha;
-            coef[1] = k.cdef;
-            coef[2] = k.beta;
-            coef[3] = k.inv_beta;
+            if (lane == 0) {
+                coef = k;
+                next[0] = (T)k.inv_beta;
+                next[1] = (T)k.alpha;
+                next[2] = (T)k.cdef;
+                next[3] = (T)k.beta;
+            }
         }
         __syncthreads();
-        if (stop_s) break;  // the same decision in every CTA of the cluster
-        const T al = (T)coef[0], cd = (T)coef[1], ib = (T)coef[3];
-        for (int64_t ul = tid; ul < nrow; ul += nthr) W[ul] = (W[ul] - al * qc[ul] - cd) * ib;
-        bt = (T)coef[2];
+        if (stop_s) break;  // step j - 1 ended the pair: the same decision in every CTA of the cluster
+        const T ib = next[0], al = next[1], cd = next[2];
+        bt = next[3];
+        for (int ul = tid; ul < nrow; ul += nthr) {
+            const T x = (W[ul] - al * qc[ul] - cd) * ib;
+            W[ul] = x;
+            if constexpr (COPY)
+                for (int r = 0; r < C; ++r) cluster_st(rbase[r] + (uint32_t)(row0 + ul) * E, x);
+        }
         const int old_prev = iprev;
         iprev = icur;
         icur = iw;
         iw = old_prev;
-        cluster.sync();  // the new q_i is complete in every CTA before the next product reads it
+        cluster_arrive();
+        cluster_wait();  // the new q_i is complete in every CTA before the next product reads it
     }
-    cluster.sync();  // no CTA leaves while another may still address its shared memory
+    cluster_arrive();
+    cluster_wait();  // no CTA leaves while another may still address its shared memory
 }
 
 // Cluster size for the whole-recurrence kernel: as many CTAs per pair as keep every pair's
-// cluster resident at once (npairs * C <= SMs), at least 32 rows per CTA, at most 16; 1 when
-// a cluster would not help (the single-CTA kernel then runs).
+// cluster resident at once (npairs * C <= SMs), at least 64 rows per CTA, at most 16.
 static int cluster_size(const OnchipArgs& a)
 {
     if (!a.allow_cluster || a.n_heavy_rows > 64) return 1;
@@ -1579,25 +1729,36 @@ static int cluster_size(const OnchipArgs& a)
     return C;
 }
 
-template <typename T, bool WEIGHTED>
+// Launches the kernel with C CTAs per pair; 0 if it does not fit. For C > 1 the entries get all the
+// shared memory that is left (one CTA of a cluster then occupies an SM: the FP64 rate per SM is
+// what a cluster multiplies); for C = 1 what the graph needs, or none where it does not fit, so
+// that several pairs share an SM.
+// Rows per CTA, even so that what follows them stays 8-byte aligned.
+static int cluster_rows(const OnchipArgs& a, int C) { return (int)(((a.n + C - 1) / C + 1) & ~1ll); }
+
+template <typename T, bool WEIGHTED, bool COPY, int NT>
 static int launch_cluster_t(cudaStream_t st, const OnchipArgs& a, int C)
 {
-    auto k = k_lanczos_cluster<T, WEIGHTED>;
+    auto k = k_lanczos_cluster<T, WEIGHTED, COPY, NT>;
     ClusterLayout L;
     L.C = C;
-    const int64_t rows = (a.n + C - 1) / C;
-    L.shift = 0;
-    while (((int64_t)1 << L.shift) < rows) ++L.shift;
-    // three row blocks, but at least 120 KB so that one CTA of the cluster occupies an SM (the
-    // FP64 rate per SM is what a cluster multiplies)
-    const size_t need = (size_t)3 * ((size_t)1 << L.shift) * sizeof(T);
-    if (need > 200 * 1024) return 0;
-    const size_t sm = need < 120 * 1024 ? 120 * 1024 : need;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return 0;
+    L.R = cluster_rows(a, C);
+    const size_t base = cluster_base_bytes(COPY ? a.n : 0, L.R, (int)sizeof(T));
+    constexpr size_t per = (WEIGHTED ? 4 : 0) + (COPY ? 2 : 4);
+    if (base > kClusterSmemMax || a.n > 65535) return 0;
+    size_t cap = (kClusterSmemMax - base) / per;
+    if (C == 1) {
+        cap = (size_t)a.nnz <= cap ? (size_t)a.nnz : 0;
+    }
+    cap = (cap + 1) & ~(size_t)1;
+    L.nnz_cap = (int)cap;
+    const size_t sm = base + cap * per;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemMax) != cudaSuccess)
+        return 0;
     if (C > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.npairs * C), 1, 1);
-    cfg.blockDim = dim3(kClusterThreads, 1, 1);
+    cfg.blockDim = dim3(NT, 1, 1);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -1608,7 +1769,7 @@ static int launch_cluster_t(cudaStream_t st, const OnchipArgs& a, int C)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, k, &cfg) != cudaSuccess || nclusters < 1) {
+    if (C > 1 && (cudaOccupancyMaxActiveClusters(&nclusters, k, &cfg) != cudaSuccess || nclusters < 1)) {
         cudaGetLastError();
         return 0;
     }
@@ -1619,15 +1780,32 @@ static int launch_cluster_t(cudaStream_t st, const OnchipArgs& a, int C)
     return C;
 }
 
+template <typename T, bool WEIGHTED, bool COPY>
+static int launch_cluster_n(cudaStream_t st, const OnchipArgs& a, int C)
+{
+    // a row per thread up to 512 rows: the products wait on shared-memory latency, and more warps
+    // hide it (1,000 vertices on 2 CTAs, FP32: 10,300 cycles a step with two rows a thread)
+    return cluster_rows(a, C) <= 256 ? launch_cluster_t<T, WEIGHTED, COPY, 256>(st, a, C)
+                                     : launch_cluster_t<T, WEIGHTED, COPY, 512>(st, a, C);
+}
+
+template <typename T>
+static int launch_cluster_e(cudaStream_t st, const OnchipArgs& a, int C, bool copy)
+{
+    if (copy) return a.weighted ? launch_cluster_n<T, true, true>(st, a, C) : launch_cluster_n<T, false, true>(st, a, C);
+    return a.weighted ? launch_cluster_n<T, true, false>(st, a, C) : launch_cluster_n<T, false, false>(st, a, C);
+}
+
 int launch_onchip(cudaStream_t st, const OnchipArgs& a)
 {
-    for (int C = cluster_size(a); C > 1; C >>= 1) {
-        int used = 0;
-        if (a.elem_size == 8) used = a.weighted ? launch_cluster_t<double, true>(st, a, C)
-                                                : launch_cluster_t<double, false>(st, a, C);
-        else used = a.weighted ? launch_cluster_t<float, true>(st, a, C) : launch_cluster_t<float, false>(st, a, C);
+    for (int C = cluster_size(a); C >= 1; C >>= 1) {
+        // copies of q_i against gathers from the other CTAs (see the kernel)
+        const bool copy = a.n * (C - 1) <= a.nnz;
+        const int used = a.elem_size == 8 ? launch_cluster_e<double>(st, a, C, copy)
+                                          : launch_cluster_e<float>(st, a, C, copy);
         if (used) return used;
     }
+    // graphs whose three vectors fit in one SM but not the degrees beside them
     const size_t sm = onchip_smem_bytes(a.n, a.elem_size);
     if (sm > 220 * 1024) return 0;
     if (a.elem_size == 8) {

@@ -980,3 +980,25 @@ def test_pair_major_outputs(rd, mode, pairs):
         one, _ = G.potential(s[p:p + 1], t[p:p + 1], **kw)
         # the narrower kernel sums in another order: 40 steps of FP32 (FP64) rounding
         assert np.abs(one[0] - phi[p]).max() < (1e-4 if mode == "fp32" else 1e-6) * np.abs(phi[p]).max()
+
+
+@pytest.mark.parametrize("mode,tol", [("fp64", FP64_TOL), ("fp32", FP32_TOL)])
+@pytest.mark.parametrize("n,extra,pairs", [(2, 0, 1), (33, 40, 1), (129, 300, 3), (257, 500, 40), (513, 6000, 5),
+                                           (1025, 1500, 2), (1500, 9000, 90), (4700, 60000, 1)])
+def test_whole_recurrence_sizes(rd, mode, tol, n, extra, pairs):
+    """The whole-recurrence kernel at the edges of its layouts: one vertex pair, row counts around
+    the thread counts and not divisible by the cluster size, sparse graphs that gather from the
+    other CTAs and dense ones that keep copies, entries that do not fit in shared memory, one CTA
+    per pair; against the dense pseudo-inverse, and repeatable bit for bit."""
+    g = F.random_connected(n, extra, 3, "lognormal" if n % 2 else None)
+    s, t = F.random_pairs(g.n, pairs, 11)
+    G = rd.Graph.from_csr(g)
+    kw = dict(mode=mode, k_max=2000, rel_tol=0.0, resid_tol=1e-11 if mode == "fp64" else 1e-6)
+    res = G.query(s, t, **kw)
+    assert G.last_stats()["onchip_ctas"] >= 1
+    assert np.all(res.status == 0)
+    assert rel(res.r, dense.DenseRD.of(g).r(s, t)).max() < tol
+    assert np.array_equal(G.query(s, t, **kw).r, res.r)
+    one = G.query(s, t, cluster=False, **kw)
+    assert G.last_stats()["onchip_ctas"] == 1
+    assert rel(one.r, res.r).max() < tol
