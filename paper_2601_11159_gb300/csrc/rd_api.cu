@@ -465,8 +465,7 @@ static rd_status make_plan_cfg(rd_graph* g, int64_t P, const rd_query_opts& o, c
     int bph = spmm_blocks_per_sm(pl->cfg, g->weighted, true, pl->prec);
     if (bph < 1) bph = 1;
     int64_t gh = (int64_t)bph * g->sm_count;
-    const int chunks_per_block = kWarps * heavy_cfg(pl->cfg).rpw();
-    gh = std::min<int64_t>(gh, (g->n_chunks + chunks_per_block - 1) / chunks_per_block);
+    gh = std::min<int64_t>(gh, g->n_chunks);  // chunks go round the blocks
     pl->grid_heavy = (int)std::max<int64_t>(gh, 1);
     const int64_t vunits = (g->n * pl->ld) / (16 / (int64_t)pl->elem) + 1;
     pl->grid_norm = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g->sm_count * 8, (vunits + 255) / 256));
