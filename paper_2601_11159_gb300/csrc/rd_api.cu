@@ -325,7 +325,8 @@ static rd_status graph_build(rd_graph* g, const int64_t* row_ptr, const int32_t*
         RD_CUDA(cudaMalloc((void**)&g->comp, sizeof(int32_t) * n));
         RD_CUDA(cudaMemcpy(g->comp, lab.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice));
     }
-    RD_CUDA(cudaMallocHost((void**)&g->h_pinned, 64));
+    RD_CUDA(cudaMallocHost((void**)&g->h_pinned, 64 + 2 * sizeof(int32_t) * kStagePairs));
+    g->h_stage = g->h_pinned + 16;
     return RD_OK;
 }
 
@@ -518,6 +519,8 @@ struct Buffers {
     size_t state_bytes_begin, state_bytes_end;  // offsets of the region zeroed per query
 };
 
+constexpr int kHostFlags = 8;  // ints at Buffers::summary
+
 // Byte size of an n x ld block rounded up to 256 bytes, so that every block that follows
 // another inside a region starts 256-byte aligned (the kernels use 16-byte vector accesses).
 static int64_t block_bytes(int64_t n, int64_t ld, size_t elem)
@@ -562,20 +565,21 @@ static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, boo
     s.hist_alpha = c.take<double>(K * ld);
     s.hist_beta = c.take<double>((K + 1) * ld);
     s.act_count = c.take<int32_t>(K + 2);
-    b->summary = c.take<int32_t>(2);
-    b->err_flag = c.take<int32_t>(1);
+    // read by the host in one copy: [0..1] summary, [2] error flag, [4..7] loop_saved
+    b->summary = c.take<int32_t>(kHostFlags);
+    b->err_flag = b->summary + 2;
+    b->loop_saved = b->summary + 4;
     b->step_dev = c.take<int32_t>(1);
     b->loop_norm = c.take<int32_t>(1);
     b->loop_ticket = c.take<int32_t>(1);
-    b->loop_saved = c.take<int32_t>(4);
     b->loop_cfrom = c.take<int32_t>(1);
     // queries on graphs that take the sparse first step (rows sorted, symmetric)
     b->row_mask = (!grad && g->rows_sorted_sym) ? c.take<uint32_t>((n * ld + 31) / 32) : nullptr;
     b->xcf = grad ? c.take<char>(K * 2 * ld * pl.elem) : nullptr;
     c.off = (c.off + 255) & ~size_t(255);
     b->state_bytes_end = c.off;
-    b->s = c.take<int32_t>(P);
-    b->t = c.take<int32_t>(P);
+    b->s = c.take<int32_t>(2 * P);
+    b->t = b->s + P;
     b->r = c.take<double>(P);
     b->iters = c.take<int32_t>(P);
     b->err = c.take<double>(P);
@@ -631,7 +635,6 @@ struct RunCtx {
     int cf_sel = 0, slot_sel = -1;  // slot_sel < 0: identity slot map
     bool in_region_x = false;
     bool lazy_walk = false;  // Power Method steps instead of Lanczos steps
-    bool onchip = false;     // whole recurrence per pair in one kernel (small graphs, queries only)
     int onchip_ctas = 0;     // CTAs per pair it ran with (1, or a cluster of 2..16)
     bool graph = false;      // steps replayed from a captured CUDA graph of one step
     bool device_loop = false;  // steps after the first run by the device-resident loop
@@ -1186,80 +1189,116 @@ static rd_status launch_step_loop(RunCtx& c, const FinArgs& base, int compact_ch
 // microseconds).
 constexpr double kNoLagBytes = 1.5e9;
 
-template <typename T>
-static rd_status run_forward(RunCtx& c)
+// Where a per-pair result is written: the caller's device array itself, or the workspace, from
+// which collect_outputs copies it once the call is known to be good.
+struct OutPtrs {
+    double* r;
+    int32_t* iters;
+    double* err;
+    int32_t* status;
+};
+
+static OutPtrs direct_outputs(const RunCtx& c, double* r_out, int32_t* iters_out, double* err_out,
+                              int32_t* status_out)
 {
-    c.cur = c.pl;
-    enqueue_init(c, false);
-    const int chunk = c.o.chunk_steps > 0 ? c.o.chunk_steps : 8;
+    return OutPtrs{is_device_ptr(r_out) ? r_out : c.b.r, is_device_ptr(iters_out) ? iters_out : c.b.iters,
+                   is_device_ptr(err_out) ? err_out : c.b.err, is_device_ptr(status_out) ? status_out : c.b.status};
+}
+
+// Stop rule and scalars of a run.
+static FinArgs fin_args(const RunCtx& c, bool fp64, bool df)
+{
     FinArgs fa{};
     fa.npairs = (int)c.P;
     fa.pstride = c.pl.ld;
     fa.k_max = c.pl.k_max;
     fa.deflate = (c.o.flags & RD_Q_NO_DEFLATE) ? 0 : 1;
     fa.fixed_k = (c.o.flags & RD_Q_FIXED_K) ? 1 : 0;
-    fa.fp64 = sizeof(T) == 8;
-    fa.df = std::is_same<T, df64>::value ? 1 : 0;
+    fa.fp64 = fp64 ? 1 : 0;
+    fa.df = df ? 1 : 0;
     fa.rel_tol = c.o.rel_tol;
     fa.resid_tol = c.o.resid_tol;
     fa.est_delayed = (c.o.flags & RD_Q_EST_DELAYED) ? 1 : 0;
     fa.sumdeg = c.g->sumdeg;
     fa.inv_sumdeg = c.g->sumdeg > 0.0 ? 1.0 / c.g->sumdeg : 0.0;
+    fa.elem_size = (int)c.pl.elem;
+    return fa;
+}
+
+// The whole-recurrence kernel, which takes the ids and writes the results itself: one memset, one
+// kernel and one read of the flags are the whole call. False if no configuration fits.
+static bool run_onchip(RunCtx& c, const OutPtrs& o)
+{
+    const rd_graph* g = c.g;
+    OnchipArgs oa{};
+    oa.n = g->n;
+    oa.nnz = g->nnz;
+    oa.npairs = (int)c.P;
+    oa.row_ptr = g->row_ptr;
+    oa.col = g->col;
+    oa.w = g->w;
+    oa.deg64 = g->deg64;
+    oa.invdeg64 = g->invdeg64;
+    oa.deg32 = g->deg32;
+    oa.invdeg32 = g->invdeg32;
+    oa.comp = g->comp;
+    oa.s = c.b.s;
+    oa.t = c.b.t;
+    oa.heavy_thr = g->heavy_thr;
+    oa.n_heavy_rows = g->n_heavy_rows;
+    oa.heavy_rows = g->heavy_rows;
+    oa.fin = fin_args(c, c.pl.fp64, false);
+    oa.elem_size = (int)c.pl.elem;
+    oa.weighted = g->weighted ? 1 : 0;
+    oa.sm_count = g->sm_count;
+    oa.allow_cluster = (c.o.flags & RD_Q_NO_CLUSTER) ? 0 : 1;
+    oa.r_out = o.r;
+    oa.iters_out = o.iters;
+    oa.err_out = o.err;
+    oa.status_out = o.status;
+    oa.summary = c.b.summary;
+    cudaMemsetAsync(c.b.summary, 0, kHostFlags * sizeof(int32_t), c.st);
+    c.onchip_ctas = launch_onchip(c.st, oa);
+    if (c.onchip_ctas == 0) return false;
+    ++c.launches;
+    return true;
+}
+
+template <typename T>
+static rd_status run_forward(RunCtx& c)
+{
+    c.cur = c.pl;
+    enqueue_init(c, false);
+    const int chunk = c.o.chunk_steps > 0 ? c.o.chunk_steps : 8;
+    FinArgs fa = fin_args(c, sizeof(T) == 8, std::is_same<T, df64>::value);
     fa.block_part = c.b.block_part;
     fa.st = c.b.st;
-    fa.elem_size = (int)c.pl.elem;
     fa.xcf = c.pot_x ? c.b.xcf : nullptr;
     int* h = c.g->h_pinned;
-    // first poll: ids valid and at least one active pair
-    RD_CUDA(cudaMemcpyAsync(h, c.b.err_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
-    RD_CUDA(cudaMemcpyAsync(h + 1, c.b.st.act_count, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
-    RD_CUDA(cudaStreamSynchronize(c.st));
-    if (h[0]) {
-        set_error("a pair id is outside [0, n)");
-        return RD_ERR_INVALID_ARG;
-    }
-    if (h[1] == 0) return RD_OK;
-    if (c.onchip) {
-        OnchipArgs oa{};
-        oa.n = c.g->n;
-        oa.nnz = c.g->nnz;
-        oa.npairs = (int)c.P;
-        oa.row_ptr = c.g->row_ptr;
-        oa.col = c.g->col;
-        oa.w = c.g->w;
-        oa.deg64 = c.g->deg64;
-        oa.invdeg64 = c.g->invdeg64;
-        oa.deg32 = c.g->deg32;
-        oa.invdeg32 = c.g->invdeg32;
-        oa.s = c.b.s;
-        oa.t = c.b.t;
-        oa.heavy_thr = c.g->heavy_thr;
-        oa.n_heavy_rows = c.g->n_heavy_rows;
-        oa.heavy_rows = c.g->heavy_rows;
-        oa.fin = fa;
-        oa.elem_size = (int)c.pl.elem;
-        oa.weighted = c.g->weighted ? 1 : 0;
-        oa.sm_count = c.g->sm_count;
-        oa.allow_cluster = (c.o.flags & RD_Q_NO_CLUSTER) ? 0 : 1;
-        const int ctas = launch_onchip(c.st, oa);
-        if (ctas > 0) {
-            c.onchip_ctas = ctas;
-            ++c.launches;
-            RD_CUDA(cudaGetLastError());
-            return RD_OK;
-        }
-    }
-    c.graph = !c.profile && (c.o.flags & RD_Q_NO_GRAPH) == 0;
-    constexpr int kSlots = 4;   // pinned poll slots h[4 .. 7]
-    cudaEvent_t poll_ev[kSlots] = {};
-    if (c.lagged_polls)
-        for (int i = 0; i < kSlots; ++i) poll_ev[i] = c.ev->get();
-    int last_known = h[1];
-    const bool sparse0 = sparse_first_step(c);
-    c.sparse_first = sparse0;
     // rd_query: after the first step, a device-resident loop over the steps (the host steps in
     // only for column compactions)
+    c.graph = !c.profile && (c.o.flags & RD_Q_NO_GRAPH) == 0;
     const bool dloop = c.graph && c.lagged_polls && (c.o.flags & RD_Q_NO_DEVICE_LOOP) == 0;
+    int last_known = (int)c.P;
+    if (!dloop) {
+        // first poll: ids valid and at least one active pair (the device-resident loop tests the
+        // count itself and the ids with its first report: kernels leave bad pairs alone)
+        RD_CUDA(cudaMemcpyAsync(h, c.b.err_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+        RD_CUDA(cudaMemcpyAsync(h + 1, c.b.st.act_count, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+        RD_CUDA(cudaStreamSynchronize(c.st));
+        if (h[0]) {
+            set_error("a pair id is outside [0, n)");
+            return RD_ERR_INVALID_ARG;
+        }
+        if (h[1] == 0) return RD_OK;
+        last_known = h[1];
+    }
+    constexpr int kSlots = 4;   // pinned poll slots h[4 .. 7]
+    cudaEvent_t poll_ev[kSlots] = {};
+    if (c.lagged_polls && !dloop)
+        for (int i = 0; i < kSlots; ++i) poll_ev[i] = c.ev->get();
+    const bool sparse0 = sparse_first_step(c);
+    c.sparse_first = sparse0;
     c.device_loop = dloop;
     for (int j = 0; j < c.pl.k_max; ++j) {
         if (dloop && j > 0) {
@@ -1270,20 +1309,30 @@ static rd_status run_forward(RunCtx& c)
                 const double bytes_per_step = spmm_launch_bytes(c.g, c.cur);
                 const int lag = bytes_per_step > kNoLagBytes ? 0 : 1;  // as the host polls below
                 RD_TRY(launch_step_loop<T>(c, fa, compact_check, lag));
-                // the step index back from the sentinel, for the next launch
-                RD_CUDA(cudaMemcpyAsync(c.b.step_dev, c.b.loop_saved, sizeof(int32_t), cudaMemcpyDeviceToDevice,
+                RD_CUDA(cudaMemcpyAsync(h + 8, c.b.summary, kHostFlags * sizeof(int32_t), cudaMemcpyDeviceToHost,
                                         c.st));
-                RD_CUDA(cudaMemcpyAsync(h + 8, c.b.loop_saved, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
                 RD_CUDA(cudaStreamSynchronize(c.st));
-                const int jn = h[8];
+                if (h[10]) {
+                    set_error("a pair id is outside [0, n)");
+                    return RD_ERR_INVALID_ARG;
+                }
+                const int jn = h[12];
                 const int ran = jn - j0;  // steps run whole inside the loop
                 // body passes: the stop shows in pass ran/2 + 1, and every kernel of a pass launches
                 c.launches += (int64_t)(ran / 2 + 1) * 2 * per_step + 1;
                 c.spmm_launches += ran;
                 c.spmm_bytes += bytes_per_step * ran;
                 if (ran & 1) std::swap(c.b.q[0], c.b.q[1]);
-                const int act_lag = h[9], act = h[10];  // the count the compaction test read; entering the next step
-                if (h[11]) {
+                const int act_lag = h[13], act = h[14];  // the count the compaction test read; entering the next step
+                const bool pending = h[15] != 0;
+                if (!pending && (act == 0 || jn >= c.pl.k_max)) {
+                    c.steps = jn;
+                    break;
+                }
+                // the step index back from the sentinel, for the next launch
+                RD_CUDA(cudaMemcpyAsync(c.b.step_dev, c.b.loop_saved, sizeof(int32_t), cudaMemcpyDeviceToDevice,
+                                        c.st));
+                if (pending) {
                     // stopped after step jn's finalize: its normalise pass, fused with the packing
                     ++c.spmm_launches;
                     c.spmm_bytes += bytes_per_step;
@@ -1299,12 +1348,11 @@ static rd_status run_forward(RunCtx& c)
                     c.steps = jn + 1;
                 } else {
                     c.steps = jn;
-                    if (act == 0 || jn >= c.pl.k_max) break;
                     RD_TRY(enqueue_compaction<T>(c, act_lag));
                 }
                 // the next test after one more step, as the host polls make it
-                h[12] = c.steps + 1;
-                RD_CUDA(cudaMemcpyAsync(c.b.loop_cfrom, h + 12, sizeof(int32_t), cudaMemcpyHostToDevice, c.st));
+                h[3] = c.steps + 1;
+                RD_CUDA(cudaMemcpyAsync(c.b.loop_cfrom, h + 3, sizeof(int32_t), cudaMemcpyHostToDevice, c.st));
             }
             break;
         }
@@ -1370,37 +1418,69 @@ static rd_status run_forward(RunCtx& c)
     return RD_OK;
 }
 
+// Pair ids where the kernels read them: the caller's own device arrays (the call ends
+// synchronised), or a copy, made through pinned memory in one piece where it fits.
 static rd_status stage_pairs(RunCtx& c, const int32_t* s, const int32_t* t)
 {
-    RD_CUDA(cudaMemcpyAsync(c.b.s, s, sizeof(int32_t) * c.P, cudaMemcpyDefault, c.st));
-    RD_CUDA(cudaMemcpyAsync(c.b.t, t, sizeof(int32_t) * c.P, cudaMemcpyDefault, c.st));
+    const bool s_dev = is_device_ptr(s), t_dev = is_device_ptr(t);
+    if (!s_dev && !t_dev && c.g->h_stage && c.P <= kStagePairs) {
+        memcpy(c.g->h_stage, s, sizeof(int32_t) * c.P);
+        memcpy(c.g->h_stage + c.P, t, sizeof(int32_t) * c.P);
+        RD_CUDA(cudaMemcpyAsync(c.b.s, c.g->h_stage, 2 * sizeof(int32_t) * c.P, cudaMemcpyHostToDevice, c.st));
+        return RD_OK;
+    }
+    if (s_dev) c.b.s = const_cast<int32_t*>(s);
+    else RD_CUDA(cudaMemcpyAsync(c.b.s, s, sizeof(int32_t) * c.P, cudaMemcpyDefault, c.st));
+    if (t_dev) c.b.t = const_cast<int32_t*>(t);
+    else RD_CUDA(cudaMemcpyAsync(c.b.t, t, sizeof(int32_t) * c.P, cudaMemcpyDefault, c.st));
+    return RD_OK;
+}
+
+// Wait for the stream, read the flags and hand out the results that were not written in place.
+static rd_status collect_outputs(RunCtx& c, const OutPtrs& o, double* r_out, int32_t* iters_out, double* err_out,
+                                 int32_t* status_out, rd_status* call_status)
+{
+    int* h = c.g->h_pinned;
+    RD_CUDA(cudaMemcpyAsync(h, c.b.summary, kHostFlags * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+    RD_CUDA(cudaStreamSynchronize(c.st));
+    RD_CUDA(cudaGetLastError());
+    if (h[2]) {
+        set_error("a pair id is outside [0, n)");
+        return RD_ERR_INVALID_ARG;
+    }
+    *call_status = h[0] ? RD_WARN_NOT_CONVERGED : RD_OK;
+    const size_t P = (size_t)c.P;
+    bool copied = false;
+    auto hand = [&](void* dst, const void* src, size_t bytes) {
+        if (!dst || dst == src) return cudaSuccess;
+        copied = true;
+        return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c.st);
+    };
+    RD_CUDA(hand(r_out, o.r, sizeof(double) * P));
+    RD_CUDA(hand(iters_out, o.iters, sizeof(int32_t) * P));
+    RD_CUDA(hand(err_out, o.err, sizeof(double) * P));
+    RD_CUDA(hand(status_out, o.status, sizeof(int32_t) * P));
+    if (copied) RD_CUDA(cudaStreamSynchronize(c.st));
     return RD_OK;
 }
 
 static rd_status finish_outputs(RunCtx& c, double* r_out, int32_t* iters_out, double* err_out, int32_t* status_out,
                                 rd_status* call_status)
 {
+    const OutPtrs o = direct_outputs(c, r_out, iters_out, err_out, status_out);
     OutArgs oa{};
     oa.npairs = (int)c.P;
     oa.ld = c.pl.ld;
     oa.st = c.b.st;
-    oa.r_out = c.b.r;
-    oa.iters_out = c.b.iters;
-    oa.err_out = c.b.err;
-    oa.status_out = c.b.status;
+    oa.r_out = o.r;
+    oa.iters_out = o.iters;
+    oa.err_out = o.err;
+    oa.status_out = o.status;
     oa.summary = c.b.summary;
+    oa.err_flag = c.b.err_flag;
     launch_output(c.st, oa);
     ++c.launches;
-    if (r_out) RD_CUDA(cudaMemcpyAsync(r_out, c.b.r, sizeof(double) * c.P, cudaMemcpyDefault, c.st));
-    if (iters_out) RD_CUDA(cudaMemcpyAsync(iters_out, c.b.iters, sizeof(int32_t) * c.P, cudaMemcpyDefault, c.st));
-    if (err_out) RD_CUDA(cudaMemcpyAsync(err_out, c.b.err, sizeof(double) * c.P, cudaMemcpyDefault, c.st));
-    if (status_out) RD_CUDA(cudaMemcpyAsync(status_out, c.b.status, sizeof(int32_t) * c.P, cudaMemcpyDefault, c.st));
-    int* h = c.g->h_pinned;
-    RD_CUDA(cudaMemcpyAsync(h, c.b.summary, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
-    RD_CUDA(cudaStreamSynchronize(c.st));
-    RD_CUDA(cudaGetLastError());
-    *call_status = h[0] ? RD_WARN_NOT_CONVERGED : RD_OK;
-    return RD_OK;
+    return collect_outputs(c, o, r_out, iters_out, err_out, status_out, call_status);
 }
 
 static void record_stats(RunCtx& c)
@@ -1642,8 +1722,16 @@ static rd_status query_batch(rd_graph* g, const int32_t* s, const int32_t* t, in
     RunCtx c;
     c.ev = ev;
     RD_TRY(prepare_run(c, g, P, o, plain, false, st, compact && !plain, lagged_polls));
-    c.onchip = (o.flags & RD_Q_NO_ONCHIP) == 0 && onchip_smem_bytes(g->n, (int)c.pl.elem) <= 220 * 1024;
     RD_TRY(stage_pairs(c, s, t));
+    // small graphs: every pair's whole recurrence in one kernel
+    if ((o.flags & RD_Q_NO_ONCHIP) == 0 && onchip_smem_bytes(g->n, (int)c.pl.elem) <= 220 * 1024) {
+        const OutPtrs op = direct_outputs(c, r_out, iters_out, err_out, status_out);
+        if (run_onchip(c, op)) {
+            RD_TRY(collect_outputs(c, op, r_out, iters_out, err_out, status_out, call_status));
+            record_stats(c);
+            return RD_OK;
+        }
+    }
     rd_status rs = c.pl.prec == 2 ? run_forward<df64>(c)
                    : (c.pl.prec == 1 ? run_forward<double>(c) : run_forward<float>(c));
     if (rs < 0) return rs;

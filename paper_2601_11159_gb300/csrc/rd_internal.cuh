@@ -221,6 +221,14 @@ struct OnchipArgs {
     int elem_size, weighted;
     int sm_count;                 // SMs of the device (cluster size choice)
     int allow_cluster;            // 0: one CTA per pair (RD_Q_NO_CLUSTER)
+    const int32_t* comp;          // nullable: component of each vertex
+    // results per pair, and the call's flags (zero on entry): [0] a pair did not converge, [1] a
+    // pair ended RD_ERR_NUMERIC, [2] a pair id is out of range (then nothing else is written)
+    double* r_out;
+    int32_t* iters_out;
+    double* err_out;
+    int32_t* status_out;
+    int32_t* summary;
 };
 size_t onchip_smem_bytes(int64_t n, int elem_size);
 // Launches the whole-recurrence kernel; returns the CTAs per pair used (1: one CTA per pair,
@@ -263,6 +271,8 @@ struct PmArgs {
 };
 void launch_pm_init(cudaStream_t st, const PmArgs& a);
 void launch_pm_accum(cudaStream_t st, const PmArgs& a);
+
+constexpr int kStagePairs = 2048;
 
 // --------------------------------------------------------------- graph
 struct Workspace {
@@ -312,7 +322,8 @@ struct rd_graph {
     double mean_deg = 0.0;
     rd::Workspace ws;
     rd_call_stats stats{};
-    int* h_pinned = nullptr;          // small pinned host buffer for polls
+    int* h_pinned = nullptr;          // small pinned host buffer for polls (16 ints)
+    int32_t* h_stage = nullptr;       // behind it, pinned: ids of up to kStagePairs pairs on their way in
     int64_t l2_bytes = 0;             // device L2 size
     // SpMM configurations chosen by the autotuner on this graph, per width class
     struct TunedCfg {
@@ -380,6 +391,7 @@ struct OutArgs {
     double* err_out;
     int32_t* status_out;
     int32_t* summary;            // [0]: any not converged, [1]: any numeric
+    const int32_t* err_flag;     // set: a pair id is out of range, and nothing is written
 };
 void launch_output(cudaStream_t st, const OutArgs& a);
 

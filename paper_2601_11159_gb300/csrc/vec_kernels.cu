@@ -904,7 +904,7 @@ void launch_split_df(cudaStream_t st, int grid, int64_t n, const double* src, df
 __global__ void k_output(const OutArgs a)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.npairs) return;
+    if (p >= a.npairs || *a.err_flag) return;
     const PairState& st = a.st;
     const int status = st.status[p];
     a.r_out[p] = st.r[p];
@@ -1295,10 +1295,78 @@ void launch_pm_accum(cudaStream_t st, const PmArgs& a)
 // ------------------------------------------------------------- on chip
 // One pair per CTA, every step in one launch: SpMV from shared memory (one thread per light
 // row, one warp per row above heavy_thr), three FP64 block sums in a fixed order, the same
-// per-pair update as k_finalize (pair_update) by thread 0, normalisation in shared memory.
+// per-pair update as k_finalize (pair_core) by thread 0, normalisation in shared memory.
 constexpr int kOnchipThreads = 1024;
 
 size_t onchip_smem_bytes(int64_t n, int elem_size) { return (size_t)3 * (size_t)n * (size_t)elem_size + 64; }
+
+// The pair's state across the steps of a whole-recurrence kernel, and its results.
+struct OnchipPair {
+    PairScalars s;
+    double r = 0.0, est = 1.0;
+    int k = 0, status = RD_OK;
+};
+
+// Start of a whole-recurrence kernel for pair p: true when its recurrence runs. Every block looks
+// all ids over first, so that a call with a bad id writes nothing but the flag; a pair that
+// needs no recurrence is answered at once (`writer`: the thread that stores).
+template <int NT>
+__device__ __forceinline__ bool onchip_start(const OnchipArgs& a, int p, bool writer)
+{
+    int bad = 0;
+    for (int i = threadIdx.x; i < a.npairs; i += NT) {
+        const int32_t s = a.s[i], t = a.t[i];
+        bad |= s < 0 || s >= a.n || t < 0 || t >= a.n;
+    }
+    if (__syncthreads_or(bad)) {
+        if (writer) a.summary[2] = 1;
+        return false;
+    }
+    if (p >= a.npairs) return false;
+    const int32_t s = a.s[p], t = a.t[p];
+    const bool apart = a.comp && a.comp[s] != a.comp[t];
+    if (s != t && !apart) return true;
+    if (writer) {
+        a.r_out[p] = apart ? INFINITY : 0.0;
+        a.iters_out[p] = 0;
+        a.err_out[p] = 0.0;
+        a.status_out[p] = apart ? RD_ERR_DISCONNECTED : RD_OK;
+    }
+    return false;
+}
+
+// Step j's scalar update of the pair; when it ends the pair and `writer` is set, its results.
+__device__ __forceinline__ bool onchip_update(const OnchipArgs& a, OnchipPair& q, int p, int j, const StepCoef& k,
+                                              bool writer)
+{
+    PairStepOut o;
+    const bool stop = pair_core(a.fin, q.s, j, k, o);
+    if (o.ok) {
+        q.r = o.r;
+        q.est = o.est;
+        q.k = j + 1;
+        if (o.warn_not_converged) q.status = RD_WARN_NOT_CONVERGED;
+    } else {
+        q.status = RD_ERR_NUMERIC;  // the last good estimate stands
+    }
+    if (stop && writer) {
+        a.r_out[p] = q.r;
+        a.iters_out[p] = q.k;
+        a.err_out[p] = q.est;
+        a.status_out[p] = q.status;
+        if (q.status == RD_WARN_NOT_CONVERGED) atomicOr(&a.summary[0], 1);
+        if (q.status == RD_ERR_NUMERIC) atomicOr(&a.summary[1], 1);
+    }
+    return stop;
+}
+
+__device__ __forceinline__ OnchipPair onchip_pair(const OnchipArgs& a, int p)
+{
+    OnchipPair q;
+    q.s = PairScalars{};
+    q.s.b2 = 1.0 / a.deg64[a.s[p]] + 1.0 / a.deg64[a.t[p]];
+    return q;
+}
 
 template <typename T, bool WEIGHTED>
 __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipArgs a)
@@ -1308,8 +1376,7 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
     __shared__ double coef[4];
     __shared__ int stop_s;
     const int p = blockIdx.x;
-    const PairState& st = a.fin.st;
-    if (p >= a.npairs || !st.active[p]) return;  // uniform over the block
+    if (!onchip_start<kOnchipThreads>(a, p, threadIdx.x == 0)) return;  // uniform over the block
     const int64_t n = a.n;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nthr = blockDim.x, nwarps = nthr >> 5;
@@ -1320,10 +1387,12 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
     int iprev = 0, icur = 1, iw = 2;
     for (int64_t u = tid; u < 3 * n; u += nthr) buf[0][u] = T(0);
     __syncthreads();
+    OnchipPair pr;
     if (tid == 0) {
+        pr = onchip_pair(a, p);
         const int32_t s = a.s[p], t = a.t[p];
         const double ds = a.deg64[s], dt = a.deg64[t];
-        const double bn = sqrt(st.b2[p]);
+        const double bn = sqrt(pr.s.b2);
         buf[icur][s] = (T)(1.0 / (ds * bn));
         buf[icur][t] = (T)(-1.0 / (dt * bn));
     }
@@ -1390,9 +1459,8 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
                 B += red[1][w];
                 C += red[2][w];
             }
-            StepCoef k;
-            PairStepOut o;
-            stop_s = pair_update(a.fin, st, p, j, A, B, C, k, o) ? 1 : 0;
+            const StepCoef k = step_coef(a.fin, A, B, C);
+            stop_s = onchip_update(a, pr, p, j, k, true) ? 1 : 0;
             coef[0] = k.alpha;
             coef[1] = k.cdef;
             coef[2] = k.beta;
@@ -1500,9 +1568,7 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
     const int C = L.C, R = L.R;
     const int rank = C > 1 ? blockIdx.x % C : 0;  // clusters are runs of C blocks along x
     const int p = blockIdx.x / C;
-    const PairState& st = a.fin.st;
-    // uniform over the cluster: no CTA changes active[p] before the first cluster barrier
-    if (p >= a.npairs || !st.active[p]) return;
+    if (!onchip_start<NT>(a, p, rank == 0 && threadIdx.x == 0)) return;  // uniform over the cluster
     const int n = (int)a.n;
     const int row0 = rank * R;
     const int nrow = row0 >= n ? 0 : (n - row0 < R ? n - row0 : R);
@@ -1542,11 +1608,11 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
             s_col[e] = (Col)locate(e);
             if constexpr (WEIGHTED) s_w[e] = __ldg(a.w + ebase + e);
         }
-    PairScalars ps;
-    if (tid == 96) ps = pair_load(st, p, a.fin.pstride);
+    OnchipPair pr;
+    if (tid == 96) pr = onchip_pair(a, p);
     if (tid == 0) {
         const int32_t s = a.s[p], t = a.t[p];
-        const double bn = st.bnorm[p];
+        const double bn = sqrt(1.0 / a.deg64[s] + 1.0 / a.deg64[t]);
         const T qs = (T)(1.0 / (a.deg64[s] * bn)), qt = (T)(-1.0 / (a.deg64[t] * bn));
         if constexpr (COPY) {
             full[s] = qs;
@@ -1559,13 +1625,8 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
     cluster_wait();  // q_1 is in place, and every CTA of the cluster runs
     int iprev = 0, icur = 1, iw = 2;
     T bt = T(0);
-    // the scalar update of step j (thread 96), stored by rank 0
-    auto update = [&](int j, const StepCoef& k) {
-        PairStepOut o;
-        const bool stop = pair_core(a.fin, ps, j, k, o);
-        if (rank == 0) pair_store(st, p, j, a.fin.pstride, ps, o, stop);
-        return stop;
-    };
+    // the scalar update of step j (thread 96), its results stored by rank 0
+    auto update = [&](int j, const StepCoef& k) { return onchip_update(a, pr, p, j, k, rank == 0); };
     for (int j = 0;; ++j) {
         if (j == a.fin.k_max) {  // the last step's update (it stops there)
             if (tid == 96) update(j - 1, coef);
