@@ -76,6 +76,17 @@ static bool is_device_ptr(const void* p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Ordinary host memory: not pinned (whose contents earlier work on the stream may still write).
+static bool is_pageable_ptr(const void* p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeUnregistered;
+}
+
 struct Carver {
     char* base;
     size_t off = 0;
@@ -1419,11 +1430,12 @@ static rd_status run_forward(RunCtx& c)
 }
 
 // Pair ids where the kernels read them: the caller's own device arrays (the call ends
-// synchronised), or a copy, made through pinned memory in one piece where it fits.
+// synchronised), or a copy in stream order; of ordinary host memory in one piece through the
+// graph's pinned buffer where it fits.
 static rd_status stage_pairs(RunCtx& c, const int32_t* s, const int32_t* t)
 {
     const bool s_dev = is_device_ptr(s), t_dev = is_device_ptr(t);
-    if (!s_dev && !t_dev && c.g->h_stage && c.P <= kStagePairs) {
+    if (c.g->h_stage && c.P <= kStagePairs && is_pageable_ptr(s) && is_pageable_ptr(t)) {
         memcpy(c.g->h_stage, s, sizeof(int32_t) * c.P);
         memcpy(c.g->h_stage + c.P, t, sizeof(int32_t) * c.P);
         RD_CUDA(cudaMemcpyAsync(c.b.s, c.g->h_stage, 2 * sizeof(int32_t) * c.P, cudaMemcpyHostToDevice, c.st));
