@@ -329,8 +329,8 @@ struct rd_graph {
     struct TunedCfg {
         int prec = 0, single = 0;     // element precision (0 FP32, 1 FP64, 2 double-float); one column or many
         int64_t width = 0;            // width class (power-of-two tile holding the pairs; 1 if single)
-        rd::SpmmCfg cfg;
-        float us = 0.f;               // measured time of one SpMM launch pair
+        // every candidate with the measured time of one SpMM launch pair at `width` columns
+        std::vector<std::pair<rd::SpmmCfg, float>> times;
     };
     std::vector<TunedCfg> tuned;
     // instantiated CUDA graphs of two Lanczos steps, keyed by the bytes of their launch
