@@ -3,6 +3,8 @@
 // 1/d_u per row because vectors are kept as q = D^{-1/2} v).
 #include <math.h>
 
+#include <algorithm>
+
 #include "rd_internal.cuh"
 
 namespace rd {
@@ -146,10 +148,13 @@ __global__ void __launch_bounds__(256) k_degrees(const DegArgs a)
     __shared__ double sd[256];
     const int tid = threadIdx.x;
     double local = 0.0;
-    for (int64_t r0 = (int64_t)blockIdx.x * 256; r0 < a.n; r0 += (int64_t)gridDim.x * 256) {
+    // 256 rows at a time, in octets dealt round the blocks: the long rows of a graph often have
+    // neighbouring ids, and a block of 256 of them would hold up the rest
+    auto row_of = [&](int64_t it, int k) { return ((it * 32 + k / 8) * gridDim.x + blockIdx.x) * 8 + k % 8; };
+    for (int64_t it = 0; row_of(it, 0) < a.n; ++it) {
         if (a.w) {
             for (int k = tid / L; k < 256; k += 256 / L) {
-                const int64_t u = r0 + k;
+                const int64_t u = row_of(it, k);
                 int64_t beg = 0, end = 0;
                 if (u < a.n) {
                     beg = a.rp[u];
@@ -157,13 +162,14 @@ __global__ void __launch_bounds__(256) k_degrees(const DegArgs a)
                 }
                 const bool light = end - beg <= a.heavy_thr;
                 double d = light ? deg_sum(a, beg + tid % L, end, L) : 0.0;
+                __syncwarp();
 #pragma unroll
                 for (int off = L / 2; off >= 1; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
                 if (tid % L == 0) sd[k] = light ? d : -1.0;
             }
             __syncthreads();
         }
-        const int64_t u = r0 + tid;
+        const int64_t u = row_of(it, tid);
         if (u < a.n) {
             const double d = a.w ? sd[tid] : (double)(a.rp[u + 1] - a.rp[u]);
             if (d != -1.0) {  // heavy rows below
@@ -176,6 +182,7 @@ __global__ void __launch_bounds__(256) k_degrees(const DegArgs a)
     if (a.w)
         for (int64_t h = blockIdx.x; h < a.n_heavy_rows; h += gridDim.x) {
             const int64_t u = a.heavy_rows[h];
+            if (a.rp[u + 1] - a.rp[u] <= a.heavy_thr) continue;  // summed above
             sd[tid] = deg_sum(a, a.rp[u] + tid, a.rp[u + 1], 256);
             __syncthreads();
             for (int s = 128; s > 0; s >>= 1) {
@@ -292,7 +299,7 @@ rd_status compute_degrees(rd_graph* g, cudaStream_t st, void* flags_dev, double*
     a.w = g->w;
     a.mirror = check_weights && g->mirror_ok ? g->mirror : nullptr;
     a.n_heavy_rows = g->n_heavy_rows;
-    a.heavy_thr = g->heavy_thr;
+    a.heavy_thr = std::max(g->heavy_thr, 256);
     a.heavy_rows = g->heavy_rows;
     a.deg64 = g->deg64;
     a.invdeg64 = g->invdeg64;
