@@ -545,7 +545,7 @@ static rd_status make_plan(rd_graph* g, int64_t P, const rd_query_opts& o, bool 
 // ---------------------------------------------------------- workspace map
 struct Buffers {
     void* q[2];               // current q_{i-1}/W (slot 0) and q_i (slot 1)
-    void* region_a;           // the two n x ld0 blocks q[] start in
+    void* region_a;           // the two n x ld0 blocks q[] start in (the pass's blocks with pot_steps)
     void* region_x;           // two n x packed_columns(ld0) blocks: target of a column compaction (NULL if off)
     void* heavy_part;
     double* block_part;
@@ -563,6 +563,8 @@ struct Buffers {
     int32_t* summary;
     int32_t* err_flag;
     int32_t* step_dev;        // step index of graph-replayed steps (zeroed per query)
+    int32_t* pot_base;        // first step of the potential's current pass
+    int32_t* pot_ticket;
     int32_t* loop_norm;       // step index of the device-resident loop's normalise passes
     int32_t* loop_ticket;     // finalize blocks done in the loop's current step
     int32_t* loop_saved;      // [4]: where the device-resident loop stopped (see k_finalize)
@@ -596,11 +598,20 @@ static int64_t packed_columns(int64_t ld)
     return (half + tile - 1) / tile * tile;
 }
 
+// Steps whose vectors a gradient or potential call keeps between updates of the potential: as many
+// as kPotSteps while the blocks take at most 8 GB, else 0 (the update runs with every step).
+static int pot_steps_for(const rd_graph* g, const Plan& pl)
+{
+    const int64_t fit = (int64_t)(8e9 / (double)block_bytes(g->n, pl.ld, pl.elem)) - 1;
+    const int m = (int)std::min<int64_t>({fit, (int64_t)kPotSteps, (int64_t)pl.k_max});
+    return m >= 2 ? m : 0;
+}
+
 static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, bool grad, Buffers* b,
-                    bool compact = false)
+                    bool compact = false, int pot_steps = 0)
 {
     const int64_t ld = pl.ld, n = g->n, K = pl.k_max;
-    b->region_a = c.take<char>(2 * block_bytes(n, ld, pl.elem));
+    b->region_a = c.take<char>(std::max(2, pot_steps + 1) * block_bytes(n, ld, pl.elem));
     b->q[0] = b->region_a;
     b->q[1] = static_cast<char*>(b->region_a) + block_bytes(n, ld, pl.elem);
     // spare region: two packed blocks
@@ -638,11 +649,13 @@ static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, boo
     b->err_flag = b->summary + 2;
     b->loop_saved = b->summary + 4;
     b->step_dev = c.take<int32_t>(1);
+    b->pot_base = grad ? c.take<int32_t>(1) : nullptr;
+    b->pot_ticket = grad ? c.take<int32_t>(1) : nullptr;
     b->loop_norm = c.take<int32_t>(1);
     b->loop_ticket = c.take<int32_t>(1);
     b->loop_cfrom = c.take<int32_t>(1);
     // queries on graphs that take the sparse first step (rows sorted, symmetric)
-    b->row_mask = (!grad && g->rows_sorted_sym) ? c.take<uint32_t>((n * ld + 31) / 32) : nullptr;
+    b->row_mask = ((!grad || pot_steps) && g->rows_sorted_sym) ? c.take<uint32_t>((n * ld + 31) / 32) : nullptr;
     b->xcf = grad ? c.take<char>(K * 2 * ld * pl.elem) : nullptr;
     c.off = (c.off + 255) & ~size_t(255);
     b->state_bytes_end = c.off;
@@ -707,7 +720,9 @@ struct RunCtx {
     bool graph = false;      // steps replayed from a captured CUDA graph of one step
     bool device_loop = false;  // steps after the first run by the device-resident loop
     bool sparse_first = false;  // first step run by k_step0_sparse
-    bool pot_x = false;      // potential accumulated during the forward steps (k_normalize_pot)
+    bool pot_x = false;      // potential accumulated during the forward steps
+    int pot_steps = 0;       // with pot_x: after passes of this many steps (k_potential_pass), or with
+                             // every step (0: k_normalize_pot)
     int compactions = 0;
     EventPool* ev = nullptr;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> spmm_ev;
@@ -748,7 +763,8 @@ static StepArgs<T> step_args(RunCtx& c, int j, bool reduce)
         a.deg = g->deg32;
     }
     a.qcur = static_cast<const T*>(c.b.q[1]);
-    a.qprev_w = static_cast<T*>(c.b.q[0]);
+    a.qprev = static_cast<const T*>(c.b.q[0]);
+    a.w_out = static_cast<T*>(c.b.q[0]);
     a.cf_beta = coef_block<T>(c, j);
     a.heavy_thr = g->heavy_thr;
     a.n_heavy_rows = g->n_heavy_rows;
@@ -860,7 +876,7 @@ static bool sparse_first_step(const RunCtx& c)
 // and whole 16-byte units per row.
 static bool sparse_norm_ok(const RunCtx& c)
 {
-    return !c.pot_x && !c.lazy_walk && c.b.row_mask && c.cur.ld % (16 / (int64_t)c.cur.elem) == 0;
+    return (!c.pot_x || c.pot_steps) && !c.lazy_walk && c.b.row_mask && c.cur.ld % (16 / (int64_t)c.cur.elem) == 0;
 }
 
 static void launch_step0_t(cudaStream_t st, const Step0Args<float>& a) { launch_step0_f32(st, a); }
@@ -1786,11 +1802,18 @@ static rd_status prepare_run(RunCtx& c, rd_graph* g, int64_t P, const rd_query_o
     RD_TRY(ensure_tuned(g, P, o, plain, compact, st));
     RD_TRY(make_plan(g, P, o, plain, &c.pl));
     c.cur = c.pl;
-    Carver dry(nullptr);
-    const size_t bytes = carve(dry, g, c.pl, P, grad, &c.b, compact);
-    RD_TRY(ensure_ws(g, bytes));
+    // a gradient or potential call that steps from captured graphs keeps a pass's vectors, memory
+    // permitting
+    c.pot_steps = grad && !c.profile && !(o.flags & (RD_Q_NO_GRAPH | RD_Q_REPLAY_POTENTIAL)) ? pot_steps_for(g, c.pl) : 0;
+    for (;;) {
+        Carver dry(nullptr);
+        const rd_status ws = ensure_ws(g, carve(dry, g, c.pl, P, grad, &c.b, compact, c.pot_steps));
+        if (ws >= 0) break;
+        if (c.pot_steps == 0) return ws;
+        c.pot_steps = 0;
+    }
     Carver real(g->ws.base);
-    carve(real, g, c.pl, P, grad, &c.b, compact);
+    carve(real, g, c.pl, P, grad, &c.b, compact, c.pot_steps);
     return RD_OK;
 }
 
@@ -1818,6 +1841,166 @@ static rd_status query_batch(rd_graph* g, const int32_t* s, const int32_t* t, in
     if (rs < 0) return rs;
     RD_TRY(finish_outputs(c, r_out, iters_out, err_out, status_out, call_status));
     record_stats(c);
+    return RD_OK;
+}
+
+static void launch_pot_pass_t(int grid, cudaStream_t st, const PotPassArgs<float>& a)
+{
+    launch_potential_pass_f32(grid, st, a);
+}
+static void launch_pot_pass_t(int grid, cudaStream_t st, const PotPassArgs<double>& a)
+{
+    launch_potential_pass_f64(grid, st, a);
+}
+
+// The forward steps of a gradient or potential call in passes of c.pot_steps steps whose vectors
+// are kept (see PotPassArgs): each pass is one CUDA graph -- the steps, each writing W into the
+// next block, and k_potential_pass -- the first of them without step 0, which is launched before
+// it (the sparse first step where it applies). The host waits for the count of active pairs after
+// each pass; steps after the last active pair return at once.
+template <typename T>
+static rd_status run_potential(RunCtx& c)
+{
+    rd_graph* g = c.g;
+    const int m = c.pot_steps;
+    c.cur = c.pl;
+    const int64_t bb = block_bytes(g->n, c.pl.ld, c.pl.elem);
+    auto block = [&](int i) { return reinterpret_cast<T*>(static_cast<char*>(c.b.region_a) + i * bb); };
+    c.b.q[0] = block(0);
+    c.b.q[1] = block(1);
+    enqueue_init(c, false);
+    c.graph = true;
+    FinArgs base = fin_args(c, sizeof(T) == 8, false);
+    base.block_part = c.b.block_part;
+    base.st = c.b.st;
+    base.xcf = c.b.xcf;
+    const bool heavy = g->n_chunks > 0;
+    // step at position o of a pass: q_{i-1} and q_i in blocks o and o + 1, W into block o + 2, the
+    // last position's into block 0
+    auto step_o = [&](int o, StepArgs<T>* sa, FinArgs* fa, NormArgs<T>* na) {
+        graph_step_args<T>(c, base, sa, fa, na);
+        sa->qprev = block(o);
+        sa->qcur = block(o + 1);
+        sa->w_out = block(o + 1 < m ? o + 2 : 0);
+        fa->loop = 2;
+        fa->loop_step = c.b.step_dev;
+        fa->loop_norm = c.b.loop_norm;
+        fa->loop_ticket = c.b.loop_ticket;
+        na->w_to_qnext = sa->w_out;
+        na->qcur = sa->qcur;
+        na->step_dev = c.b.loop_norm;
+        na->pvec = na->xvec = nullptr;
+        na->xcf = nullptr;
+        na->xcf_stride = 0;
+    };
+    StepArgs<T> sa;
+    FinArgs fa;
+    NormArgs<T> na;
+    // step 0
+    step_o(0, &sa, &fa, &na);
+    c.sparse_first = sparse_first_step(c);
+    if (c.sparse_first) {
+        c.b.q[0] = sa.w_out;
+        if (!sparse_norm_ok(c)) RD_CUDA(cudaMemsetAsync(sa.w_out, 0, bb, c.st));
+        enqueue_step0<T>(c, true);
+        fa.nblocks = 1;
+        launch_finalize(c.st, fa);
+        if (sparse_norm_ok(c)) enqueue_normalize_step0<T>(c);
+        else launch_normalize_t(c.cur.grid_norm, c.st, na);
+        c.b.q[0] = block(0);
+        c.launches += 2;
+    } else {
+        bool ok = !heavy || launch_spmm_t(c.cur.cfg, g->weighted, true, c.cur.grid_heavy, c.st, sa);
+        ok = ok && launch_spmm_t(c.cur.cfg, g->weighted, false, c.cur.grid_main, c.st, sa);
+        if (!ok) return RD_ERR_UNSUPPORTED;
+        launch_finalize(c.st, fa);
+        launch_normalize_t(c.cur.grid_norm, c.st, na);
+        c.launches += heavy ? 4 : 3;
+        ++c.spmm_launches;
+        c.spmm_bytes += spmm_launch_bytes(g, c.cur);
+    }
+    PotPassArgs<T> pa;
+    memset(&pa, 0, sizeof(pa));
+    pa.n = g->n;
+    pa.ld = c.pl.ld;
+    pa.stride = bb / (int64_t)sizeof(T);
+    pa.m = m;
+    pa.k_max = c.pl.k_max;
+    pa.blocks = block(0);
+    pa.pvec = static_cast<T*>(c.b.pvec);
+    pa.xvec = static_cast<T*>(c.b.phi);
+    pa.cf = static_cast<const T*>(c.b.cf_hist);
+    pa.xcf = static_cast<const T*>(c.b.xcf);
+    pa.act_count = c.b.st.act_count;
+    pa.base = c.b.pot_base;
+    pa.ticket = c.b.pot_ticket;
+    int* h = g->h_pinned;
+    for (int done = 0; done < c.pl.k_max; done += m) {
+        const int first = done == 0 ? 1 : 0;  // position the pass's graph starts at
+        step_o(first, &sa, &fa, &na);
+        int misc[9] = {c.cur.cfg.vec, c.cur.cfg.gs, c.cur.cfg.nzl, c.cur.cfg.kind, c.cur.grid_main, c.cur.grid_heavy,
+                       c.cur.grid_norm, m, first};
+        std::string key("pot");
+        key.append(reinterpret_cast<const char*>(misc), sizeof(misc));
+        key.append(reinterpret_cast<const char*>(&sa), sizeof(sa));
+        key.append(reinterpret_cast<const char*>(&fa), sizeof(fa));
+        key.append(reinterpret_cast<const char*>(&na), sizeof(na));
+        key.append(reinterpret_cast<const char*>(&pa), sizeof(pa));
+        key.push_back(sizeof(T) == 8 ? 'd' : 'f');
+        cudaGraphExec_t exec = nullptr;
+        for (const auto& kv : g->graphs)
+            if (kv.first == key) {
+                exec = kv.second;
+                break;
+            }
+        if (!exec) {
+            if (!g->capture_stream) RD_CUDA(cudaStreamCreateWithFlags(&g->capture_stream, cudaStreamNonBlocking));
+            cudaStream_t cs = g->capture_stream;
+            RD_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+            bool ok = true;
+            for (int o = first; o < m && ok; ++o) {
+                step_o(o, &sa, &fa, &na);
+                if (heavy) ok = launch_spmm_t(c.cur.cfg, g->weighted, true, c.cur.grid_heavy, cs, sa);
+                if (ok) ok = launch_spmm_t(c.cur.cfg, g->weighted, false, c.cur.grid_main, cs, sa);
+                launch_finalize(cs, fa);
+                if (o + 1 < m) launch_normalize_t(c.cur.grid_norm, cs, na);
+            }
+            launch_pot_pass_t(c.cur.grid_norm, cs, pa);
+            cudaGraph_t graph = nullptr;
+            const cudaError_t ec = cudaStreamEndCapture(cs, &graph);
+            if (!ok) {
+                if (graph) cudaGraphDestroy(graph);
+                set_error("no SpMM kernel for this configuration");
+                return RD_ERR_UNSUPPORTED;
+            }
+            RD_CUDA(ec);
+            const cudaError_t ei = cudaGraphInstantiate(&exec, graph, 0);
+            cudaGraphDestroy(graph);
+            RD_CUDA(ei);
+            if (g->graphs.size() >= kGraphCache) {
+                cudaGraphExecDestroy(g->graphs.front().second);
+                g->graphs.erase(g->graphs.begin());
+            }
+            g->graphs.emplace_back(std::move(key), exec);
+        }
+        RD_CUDA(cudaGraphLaunch(exec, c.st));
+        const int steps = m - first;
+        c.launches += steps * (heavy ? 4 : 3);
+        c.spmm_launches += steps;
+        c.spmm_bytes += spmm_launch_bytes(g, c.cur) * steps;
+        c.steps = std::min(c.pl.k_max, done + m);
+        if (c.steps == c.pl.k_max && done > 0) break;
+        if (done > 0 && base.fixed_k) continue;  // every pair goes on but for breakdowns
+        RD_CUDA(cudaMemcpyAsync(h, c.b.err_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+        RD_CUDA(cudaMemcpyAsync(h + 1, c.b.st.act_count + c.steps, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+        RD_CUDA(cudaStreamSynchronize(c.st));
+        if (h[0]) {
+            set_error("a pair id is outside [0, n)");
+            return RD_ERR_INVALID_ARG;
+        }
+        if (h[1] == 0) break;
+    }
+    RD_CUDA(cudaGetLastError());
     return RD_OK;
 }
 
@@ -1859,12 +2042,13 @@ static rd_status forward_and_potential(RunCtx& c, const int32_t* s, const int32_
     // the potential: accumulated during the forward steps (direct update), or, with
     // RD_Q_REPLAY_POTENTIAL, by a second pass that regenerates the vectors
     c.pot_x = (c.o.flags & RD_Q_REPLAY_POTENTIAL) == 0;
-    if (c.pot_x) {
+    if (c.pot_x && !c.pot_steps) {
         const int64_t vbytes = c.g->n * c.pl.ld * (int64_t)c.pl.elem;
         RD_CUDA(cudaMemsetAsync(c.b.phi, 0, vbytes, c.st));
         RD_CUDA(cudaMemsetAsync(c.b.pvec, 0, vbytes, c.st));
     }
-    rd_status rs = c.pl.fp64 ? run_forward<double>(c) : run_forward<float>(c);
+    rd_status rs = c.pot_x && c.pot_steps ? (c.pl.fp64 ? run_potential<double>(c) : run_potential<float>(c))
+                                          : (c.pl.fp64 ? run_forward<double>(c) : run_forward<float>(c));
     if (rs < 0) return rs;
     // z-solve and gbar; a host grad_r is staged in the output buffer (free until the end)
     const double* d_grad = nullptr;
@@ -1881,7 +2065,7 @@ static rd_status forward_and_potential(RunCtx& c, const int32_t* s, const int32_
     za.ld = c.pl.ld;
     za.k_max = c.pl.k_max;
     za.st = c.b.st;
-    za.coef_hist = c.b.coef_hist;
+    za.coef_hist = c.pot_x ? nullptr : c.b.coef_hist;
     za.gbar = c.b.gbar;
     za.zscratch = c.b.zscratch;
     za.elem_size = (int)c.pl.elem;

@@ -77,7 +77,8 @@ struct StepArgs {
     const T* invdeg;               // 1/d_u
     const T* deg;                  // d_u
     const T* qcur;                 // q_i  (n x ld)
-    T* qprev_w;                    // in: q_{i-1}; out: W = D^{-1} W_adj q_i - beta_i q_{i-1}
+    const T* qprev;                // q_{i-1}
+    T* w_out;                      // W = D^{-1} W_adj q_i - beta_i q_{i-1} (may be qprev's block)
     const T* cf_beta;              // beta_i per column (ld)
     // heavy rows (degree > heavy_thr): chunk partial sums made by the heavy kernel
     int heavy_thr;
@@ -138,6 +139,24 @@ struct NormArgs {
     int64_t xcf_stride;
 };
 
+// End of a pass of up to `m` steps whose vectors were kept (k_potential_pass). Blocks of n x ld
+// elements, `stride` elements apart: block 0 holds W of the pass's last step, block 1 + i the
+// vector q of its step i.
+constexpr int kPotSteps = 8;
+template <typename T>
+struct PotPassArgs {
+    int64_t n, ld, stride;
+    int m, k_max;
+    T* blocks;
+    T* pvec;                      // p of the last step before the pass in, of its last step out
+    T* xvec;                      // x += sum over the pass's steps of mu_i p_i
+    const T* cf;                  // [k_max + 1][4][ld] coefficients by step
+    const T* xcf;                 // [k_max][2][ld]: lambda_i, mu_i by step
+    const int32_t* act_count;
+    int32_t* base;                // first step of the pass; advanced by m at its end
+    int32_t* ticket;              // blocks done (0 between launches)
+};
+
 // Normalise pass fused with a column compaction (k_normalize_pack).
 template <typename T>
 struct NormPackArgs {
@@ -190,7 +209,8 @@ struct FinArgs {
     void* xcf;                          // nullable T [k_max][2][ld]: step j receives lambda_i, mu_i
                                         // of the potential's direct update (identity slot map only)
     // device-resident step loop (see k_finalize and k_loop_entry)
-    int loop;                           // 1: this launch is in the loop's body
+    int loop;                           // 1: this launch is in the loop's body; 2: it only advances
+                                        // loop_step and loop_norm (no conditional node)
     int loop_compact, loop_lag;         // test for a column compaction, on the count `lag` steps back
     unsigned long long loop_handle;     // the while node's cudaGraphConditionalHandle
     int32_t* loop_step;                 // step index of the body's pre-pass, SpMM and finalize
@@ -353,6 +373,8 @@ bool launch_spmm_f64(const SpmmCfg& c, bool weighted, bool heavy, int grid, cuda
 int spmm_blocks_per_sm(const SpmmCfg& c, bool weighted, bool heavy, int prec);
 std::vector<SpmmCfg> spmm_configs(bool fp64);
 
+void launch_potential_pass_f32(int grid, cudaStream_t st, const PotPassArgs<float>& a);
+void launch_potential_pass_f64(int grid, cudaStream_t st, const PotPassArgs<double>& a);
 void launch_normalize_f32(int grid, cudaStream_t st, const NormArgs<float>& a);
 void launch_normalize_f64(int grid, cudaStream_t st, const NormArgs<double>& a);
 void launch_normalize_df64(int grid, cudaStream_t st, const NormArgs<df64>& a);

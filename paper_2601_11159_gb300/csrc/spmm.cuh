@@ -376,7 +376,7 @@ __device__ __forceinline__ void row_epilogue(const StepArgs<T>& a, int64_t row, 
 #pragma unroll
         for (int i = 0; i < VEC; ++i) wv[i] = invd * acc[i] - bt[i] * qp[i];
     }
-    st_stream<T, VEC>(a.qprev_w + row * a.ld + c0, wv);
+    st_stream<T, VEC>(a.w_out + row * a.ld + c0, wv);
     if (a.do_reduce) {
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
@@ -572,7 +572,7 @@ __device__ __forceinline__ void row_epilogue_s(const StepArgs<T>& a, int64_t row
 #pragma unroll
         for (int i = 0; i < VEC; ++i) wv[i] = invd * acc[i] - bt[i] * qp[i];
     }
-    st_stream<T, VEC>(a.qprev_w + row * a.ld + c0, wv);
+    st_stream<T, VEC>(a.w_out + row * a.ld + c0, wv);
     if (a.do_reduce) {
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
@@ -634,7 +634,7 @@ __device__ __forceinline__ void row_epilogue_b(const StepArgs<T>& a, int row, in
 #pragma unroll
         for (int i = 0; i < VEC; ++i) wv[i] = invd * acc[i] - bt[i] * qp[i];
     }
-    st_stream<T, VEC>(a.qprev_w + (int64_t)row * a.ld + c0, wv);
+    st_stream<T, VEC>(a.w_out + (int64_t)row * a.ld + c0, wv);
     if (a.do_reduce) {
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
@@ -698,7 +698,7 @@ __global__ void __launch_bounds__(kBlock, kGroupMinBlocks<T, VEC>) k_spmm(const 
 #pragma unroll
             for (int i = 0; i < VEC; ++i) acc[i] = T(0);
             if (zl == 0) {  // own-row operands of the epilogue, issued before the gather
-                ld_stream<T, VEC>(qp, a.qprev_w + row * ld + c0);
+                ld_stream<T, VEC>(qp, a.qprev + row * ld + c0);
                 ld_gather<T, VEC>(qc, a.qcur + row * ld + c0);
             }
             if (end - beg > a.heavy_thr) {
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
 #pragma unroll
             for (int i = 0; i < VEC; ++i) acc[i] = T(0);
             if (r1 == r0 + 1 && e_end - e_beg > a.heavy_thr) {
-                ld_stream<T, VEC>(qp, a.qprev_w + (int64_t)r0 * ld + c0);
+                ld_stream<T, VEC>(qp, a.qprev + (int64_t)r0 * ld + c0);
                 ld_gather<T, VEC>(qc, q + (int64_t)r0 * ld);
                 heavy_row_sum<T, VEC, 1>(a, r0, c0, 0, acc);
                 row_epilogue_b<T, VEC>(a, r0, c0, a.invdeg[r0], a.deg[r0], acc, bt, qp, qc, rb, sacc);
@@ -793,7 +793,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
             int row_end = __shfl_sync(mask, my_end, 0, GS);
-            ld_stream<T, VEC>(qp, a.qprev_w + (int64_t)row * ld + c0);
+            ld_stream<T, VEC>(qp, a.qprev + (int64_t)row * ld + c0);
             ld_gather<T, VEC>(qc, q + (int64_t)row * ld);
             for (int base = e_beg; base < e_end; base += CH) {
                 const int cnt = e_end - base < CH ? e_end - base : CH;
@@ -855,7 +855,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                                 my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                             }
                             row_end = __shfl_sync(mask, my_end, row - w0, GS);
-                            ld_stream<T, VEC>(qp, a.qprev_w + (int64_t)row * ld + c0);
+                            ld_stream<T, VEC>(qp, a.qprev + (int64_t)row * ld + c0);
                             ld_gather<T, VEC>(qc, q + (int64_t)row * ld);
                         }
                         if constexpr (WEIGHTED) {
@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                     my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }
-                ld_stream<T, VEC>(qp, a.qprev_w + (int64_t)row * ld + c0);
+                ld_stream<T, VEC>(qp, a.qprev + (int64_t)row * ld + c0);
                 ld_gather<T, VEC>(qc, q + (int64_t)row * ld);
             }
         }
@@ -1156,7 +1156,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
             T acc[V], qp[V], qc[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) acc[i] = T(0);
-            ld_stream<T, V>(qp, a.qprev_w + (int64_t)r * ld + c0);
+            ld_stream<T, V>(qp, a.qprev + (int64_t)r * ld + c0);
             ld_gather<T, V>(qc, q + (int64_t)r * ld);
             heavy_chunks_sum<T, V, 1>(a, f, l, c0, 0, acc);
             row_epilogue<T, V>(a, r, c0, a.invdeg[r], a.deg[r], acc, bt, qp, qc, sA, sB, sC);
@@ -1174,14 +1174,14 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
             int row_end = __shfl_sync(mask, my_end, 0, GS);
-            ld_stream<T, V>(qp, a.qprev_w + (int64_t)row * ld + c0);
+            ld_stream<T, V>(qp, a.qprev + (int64_t)row * ld + c0);
             ld_gather<T, V>(qc, q + (int64_t)row * ld);
             // the own-row operands of the next PD rows into L2 (no registers held): short rows
             // end before a load from DRAM would return
 #pragma unroll
             for (int d = 1; d <= PD; ++d)
                 if (row + d < r1) {
-                    prefetch_l2(a.qprev_w + (int64_t)(row + d) * ld + c0);
+                    prefetch_l2(a.qprev + (int64_t)(row + d) * ld + c0);
                     prefetch_l2(q + (int64_t)(row + d) * ld);
                 }
             // close the current row and open the next one
@@ -1203,10 +1203,10 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }
                 row_end = __shfl_sync(mask, my_end, row - w0, GS);
-                ld_stream<T, V>(qp, a.qprev_w + (int64_t)row * ld + c0);
+                ld_stream<T, V>(qp, a.qprev + (int64_t)row * ld + c0);
                 ld_gather<T, V>(qc, q + (int64_t)row * ld);
                 if (PD > 0 && row + PD < r1) {
-                    prefetch_l2(a.qprev_w + (int64_t)(row + PD) * ld + c0);
+                    prefetch_l2(a.qprev + (int64_t)(row + PD) * ld + c0);
                     prefetch_l2(q + (int64_t)(row + PD) * ld);
                 }
             };
@@ -1304,7 +1304,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_tasks(const StepArgs<T> a)
             for (int off = 16; off > 0; off >>= 1) acc[0] += shfl_xor_t(0xffffffffu, acc[0], off);
             if (lane == 0) {
                 T qp[1], qc[1], bt1[1] = {bt};
-                qp[0] = a.qprev_w[r0];
+                qp[0] = a.qprev[r0];
                 qc[0] = a.qcur[r0];
                 Acc<T> tA[1] = {sA}, tB[1] = {sB}, tC[1] = {sC};
                 row_epilogue<T, 1>(a, r0, 0, a.invdeg[r0], a.deg[r0], acc, bt1, qp, qc, tA, tB, tC);
@@ -1323,7 +1323,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_tasks(const StepArgs<T> a)
         if (rf < r1) {
             fb0 = (int)(a.row_ptr[rf] - e0);
             fb1 = (int)(a.row_ptr[rf + 1] - e0);
-            fqp = a.qprev_w[rf];
+            fqp = a.qprev[rf];
             fqc = a.qcur[rf];
             finvd = a.invdeg[rf];
             fdu = a.deg[rf];
@@ -1360,7 +1360,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_tasks(const StepArgs<T> a)
             T sum = T(0);
             for (int k = b0; k < b1; ++k) sum += pw[k];
             T acc[1] = {sum}, qp[1], qc[1], bt1[1] = {bt};
-            qp[0] = first ? fqp : a.qprev_w[r];
+            qp[0] = first ? fqp : a.qprev[r];
             qc[0] = first ? fqc : a.qcur[r];
             const T invd = first ? finvd : a.invdeg[r];
             const T du = first ? fdu : a.deg[r];

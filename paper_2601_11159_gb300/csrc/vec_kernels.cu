@@ -317,7 +317,11 @@ __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
     const int64_t col = (int64_t)blockIdx.x * cb + lane;
     const PairState& st = a.st;
     const int j = a.step_dev ? *a.step_dev : a.step;  // 0-based step index; Lanczos step i = j + 1
-    if (st.act_count[j] == 0) return;
+    if (st.act_count[j] == 0) {
+        // the step's normalise pass has nothing to do either
+        if (a.loop == 2 && blockIdx.x == 0 && threadIdx.x == 0) *a.loop_norm = a.k_max + 1;
+        return;
+    }
     // block partials b = split, split + nsplit, ...: four rows of loads in flight, summed
     // in block order (the order depends only on nblocks and ld, so runs are repeatable)
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
@@ -398,6 +402,11 @@ __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
     __threadfence();
     const volatile int32_t* act_count = st.act_count;
     const int jn = j + 1;
+    if (a.loop == 2) {
+        *a.loop_norm = j;
+        *a.loop_step = jn;
+        return;
+    }
     const int act = act_count[jn];
     const int act_lag = act_count[jn >= a.loop_lag ? jn - a.loop_lag : 0];
     const bool more = act > 0 && jn < a.k_max;
@@ -554,6 +563,89 @@ __global__ void __launch_bounds__(256) k_normalize_pot(const NormArgs<T> a)
         st_plain<T, V>(a.w_to_qnext + e0, qn);
     }
 }
+
+// The same potential with the vectors of up to kPotSteps steps kept: at the end of a pass its
+// vectors are read once, p and x go through registers step by step (the operations and rounding of
+// k_normalize_pot), and where the pass is full and pairs go on, the last step's normalise pass is
+// made on the way: q_{i+1} and q_i go to blocks 1 and 0, where the next pass starts. Bound by HBM:
+// a step streams 3 blocks in its normalise pass and 1 here, plus 4 per pass for p and x (none in
+// and no p out where one pass is all), against 7 per step; 32 FP32 columns of a 4M-vertex graph
+// (511 MB a block), 8 steps: 4.45 ms with k_normalize_pot and 0.3 ms of zeroing; the call 17.5 ->
+// 16.0 ms (18.1 -> 16.6 on another GPU).
+template <typename T, bool VECD>
+__global__ void __launch_bounds__(256) k_potential_pass(const PotPassArgs<T> a)
+{
+    constexpr int V = VECD ? 16 / (int)sizeof(T) : 1;
+    const int base = *a.base;
+    int cnt = 0;
+    while (cnt < a.m && base + cnt < a.k_max && a.act_count[base + cnt] > 0) ++cnt;
+    if (cnt == 0 && base > 0) return;
+    const bool more = cnt == a.m && base + a.m < a.k_max && a.act_count[base + a.m] > 0;
+    const int64_t ld = a.ld;
+    const int64_t units = a.n * ld / V;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const T* xcf = a.xcf + (int64_t)base * 2 * ld;
+    const T* cf = a.cf + (int64_t)(base + cnt - 1) * 4 * ld;
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += stride) {
+        const int64_t e0 = u * V, c0 = e0 % ld;
+        T q[kPotSteps][V], pv[V], xv[V];
+#pragma unroll
+        for (int s = 0; s < kPotSteps; ++s)
+            if (s < cnt) ld_stream<T, V>(q[s], a.blocks + (int64_t)(1 + s) * a.stride + e0);
+        if (base > 0) {
+            ld_stream<T, V>(pv, a.pvec + e0);
+            ld_stream<T, V>(xv, a.xvec + e0);
+        } else {
+#pragma unroll
+            for (int i = 0; i < V; ++i) pv[i] = xv[i] = T(0);
+        }
+#pragma unroll
+        for (int s = 0; s < kPotSteps; ++s)
+            if (s < cnt) {
+                T lam[V], mu[V];
+                ld_plain<T, V>(lam, xcf + (int64_t)s * 2 * ld + c0);
+                ld_plain<T, V>(mu, xcf + (int64_t)s * 2 * ld + ld + c0);
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    pv[i] = q[s][i] + lam[i] * pv[i];
+                    xv[i] += mu[i] * pv[i];
+                }
+            }
+        st_plain<T, V>(a.xvec + e0, xv);
+        if (more) {
+            T w[V], al[V], c[V], ib[V], ql[V], qn[V];
+            ld_stream<T, V>(w, a.blocks + e0);
+            ld_plain<T, V>(al, cf + ld + c0);
+            ld_plain<T, V>(c, cf + 2 * ld + c0);
+            ld_plain<T, V>(ib, cf + 3 * ld + c0);
+#pragma unroll
+            for (int s = 0; s < kPotSteps; ++s)
+                if (s == cnt - 1)
+#pragma unroll
+                    for (int i = 0; i < V; ++i) ql[i] = q[s][i];
+#pragma unroll
+            for (int i = 0; i < V; ++i) qn[i] = lanczos_next<T>(w[i], al[i], ql[i], c[i], ib[i]);
+            st_plain<T, V>(a.pvec + e0, pv);
+            st_plain<T, V>(a.blocks + e0, ql);
+            st_plain<T, V>(a.blocks + a.stride + e0, qn);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(a.ticket, 1) != (int)gridDim.x - 1) return;
+    *a.ticket = 0;
+    *a.base = base + a.m;
+}
+
+template <typename T>
+static void launch_pot_pass(int grid, cudaStream_t st, const PotPassArgs<T>& a)
+{
+    if (a.ld % (16 / (int64_t)sizeof(T)) == 0) k_potential_pass<T, true><<<grid, 256, 0, st>>>(a);
+    else k_potential_pass<T, false><<<grid, 256, 0, st>>>(a);
+}
+void launch_potential_pass_f32(int grid, cudaStream_t st, const PotPassArgs<float>& a) { launch_pot_pass(grid, st, a); }
+void launch_potential_pass_f64(int grid, cudaStream_t st, const PotPassArgs<double>& a) { launch_pot_pass(grid, st, a); }
 
 template <typename T>
 static void launch_norm(int grid, cudaStream_t st, const NormArgs<T>& a)
@@ -938,6 +1030,10 @@ __global__ void k_zsolve(const ZsolveArgs a)
     const int status = p < a.npairs ? st.status[p] : RD_ERR_INVALID_ARG;
     const int k = p < a.npairs ? st.k[p] : 0;
     const bool use = (status == RD_OK || status == RD_WARN_NOT_CONVERGED) && k > 0;
+    if (!coef) {  // the potential was accumulated during the steps: gbar is all that is needed
+        gbar[p] = use ? (T)(a.grad_r ? a.grad_r[p] : 1.0) : T(0);
+        return;
+    }
     if (!use) {
         for (int j = 0; j < a.k_max; ++j) coef[(int64_t)j * ld + p] = T(0);
         gbar[p] = T(0);

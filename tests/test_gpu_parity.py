@@ -1002,3 +1002,28 @@ def test_whole_recurrence_sizes(rd, mode, tol, n, extra, pairs):
     one = G.query(s, t, cluster=False, **kw)
     assert G.last_stats()["onchip_ctas"] == 1
     assert rel(one.r, res.r).max() < tol
+
+
+@pytest.mark.parametrize("mode", ["fp32", "fp64"])
+@pytest.mark.parametrize("k_max,pairs", [(1, 3), (2, 1), (3, 5), (7, 17), (8, 1), (9, 17), (16, 2), (17, 5), (30, 33)])
+def test_potential_passes(rd, mode, k_max, pairs):
+    """The potential updated once per pass of kept vectors: bit for bit the update with every step
+    (which the launch-per-kernel loop makes), around the pass length, with one pair, pairs that
+    need no steps, and pairs that stop inside a pass; gradients and flows follow."""
+    g = F.random_connected(301, 700, 23, "lognormal")
+    s, t = F.random_pairs(g.n, pairs, 8)
+    if pairs > 4:
+        t[1] = s[1]
+    G = rd.Graph.from_csr(g)
+    for kw in (dict(k_max=k_max, fixed_k=True), dict(k_max=k_max, rel_tol=1e-3)):
+        kw = dict(kw, mode=mode, tune=False)
+        phi, r = G.potential(s, t, **kw)
+        phi0, r0 = G.potential(s, t, graph=False, **kw)
+        assert np.array_equal(r, r0)
+        assert np.array_equal(phi, phi0)
+        gw, _ = G.edge_grad(s, t, np.linspace(-1, 1, pairs), **kw)
+        gw0, _ = G.edge_grad(s, t, np.linspace(-1, 1, pairs), graph=False, **kw)
+        assert np.array_equal(gw, gw0)
+    dense_first, _ = G.potential(s, t, sparse_first=False, mode=mode, k_max=k_max, fixed_k=True, tune=False)
+    ref, _ = G.potential(s, t, sparse_first=False, graph=False, mode=mode, k_max=k_max, fixed_k=True, tune=False)
+    assert np.array_equal(dense_first, ref)
