@@ -61,6 +61,18 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b)
     return df_fast_two_sum(p, e);
 }
 
+// The product without its renormalisation (4 FP32 operations instead of 7): p + e, |e| a few units in
+// the last place of p. Good as an operand of df_sum and df_prod, which take their operands' parts
+// as they come.
+__device__ __forceinline__ df64 df_prod(df64 a, df64 b)
+{
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    return df64(p, e, 0);
+}
+
 __device__ __forceinline__ df64& operator+=(df64& a, df64 b)
 {
     a = a + b;
