@@ -364,6 +364,7 @@ struct Plan {
     bool fp64;              // 8-byte vector elements (FP64 or double-float)
     int prec = 0;           // mode_prec
     bool tuned = false;     // cfg taken from the autotuner's table
+    double us = 0.0;        // then: estimated SpMM and normalise time of a step
     SpmmCfg cfg;
     int64_t ld;
     int grid_main, grid_heavy, grid_norm, nslab;
@@ -416,7 +417,8 @@ static int64_t padded_columns(int64_t P, const SpmmCfg& c)
 // tile), and the normalise pass streams three blocks of those columns at about 6 TB/s: 70 pairs
 // ran as 128 columns when the fastest tile of the class was taken as it is, and run as 80 or 96
 // now. `max_ld` > 0: at most that many columns. NULL if none is left.
-static const SpmmCfg* best_candidate(const rd_graph* g, const rd_graph::TunedCfg& t, int64_t P, int64_t max_ld)
+static const SpmmCfg* best_candidate(const rd_graph* g, const rd_graph::TunedCfg& t, int64_t P, int64_t max_ld,
+                                     double* us_out)
 {
     const SpmmCfg* best = nullptr;
     double best_us = 0.0;
@@ -432,20 +434,21 @@ static const SpmmCfg* best_candidate(const rd_graph* g, const rd_graph::TunedCfg
             best_us = us;
         }
     }
+    *us_out = best_us;
     return best;
 }
 
 static SpmmCfg pick_cfg(const rd_graph* g, int64_t P, const rd_query_opts& o, bool fp64, bool plain,
-                        bool* from_table = nullptr, int64_t max_ld = 0)
+                        double* table_us = nullptr, int64_t max_ld = 0)
 {
     const double mdeg = g->n ? (double)g->nnz / (double)g->n : 0.0;
-    if (from_table) *from_table = false;
     if (tuning_allowed(o)) {
         const bool single = plain || P == 1;
         const rd_graph::TunedCfg* t = find_tuned(g, mode_prec(o.mode), single, tune_width(P, fp64, single));
-        const SpmmCfg* best = t ? best_candidate(g, *t, P, max_ld) : nullptr;
+        double us = 0.0;
+        const SpmmCfg* best = t ? best_candidate(g, *t, P, max_ld, &us) : nullptr;
         if (best) {
-            if (from_table) *from_table = true;
+            if (table_us) *table_us = us;
             return *best;
         }
     }
@@ -535,10 +538,11 @@ static rd_status make_plan_cfg(rd_graph* g, int64_t P, const rd_query_opts& o, c
 
 static rd_status make_plan(rd_graph* g, int64_t P, const rd_query_opts& o, bool plain, Plan* pl, int64_t max_ld = 0)
 {
-    bool from_table = false;
-    const SpmmCfg cfg = pick_cfg(g, P, o, mode_prec(o.mode) != 0, plain, &from_table, max_ld);
+    double us = 0.0;
+    const SpmmCfg cfg = pick_cfg(g, P, o, mode_prec(o.mode) != 0, plain, &us, max_ld);
     RD_TRY(make_plan_cfg(g, P, o, cfg, pl));
-    pl->tuned = from_table;
+    pl->tuned = us > 0.0;
+    pl->us = us;
     return RD_OK;
 }
 
@@ -1267,10 +1271,16 @@ static rd_status launch_step_loop(RunCtx& c, const FinArgs& base, int compact_ch
     return RD_OK;
 }
 
-// Algorithmic bytes of one SpMM launch above which rd_query polls without lag (about a
-// quarter of a millisecond of HBM traffic on this part, against a host reaction of tens of
-// microseconds).
-constexpr double kNoLagBytes = 1.5e9;
+// Steps back that the column compaction's test reads the count of active pairs. The current count
+// (0) costs a host-driven loop the host's reaction, some 25 us per step, and in either loop a
+// step that ends most pairs is followed by a narrow one at once instead of one more at full width;
+// taken when a step is long against that: 300 us by the tuner's timings (0.5 GB of algorithmic
+// bytes where there are none). R-MAT 20, 128 pairs, of which 14 go into the last step: 9.0 ms a
+// query with the count of a step earlier (the line lay at 1.5 GB).
+static int poll_lag(const RunCtx& c)
+{
+    return (c.cur.us > 0.0 ? c.cur.us > 300.0 : spmm_launch_bytes(c.g, c.cur) > 0.5e9) ? 0 : 1;
+}
 
 // Where a per-pair result is written: the caller's device array itself, or the workspace, from
 // which collect_outputs copies it once the call is known to be good.
@@ -1390,7 +1400,7 @@ static rd_status run_forward(RunCtx& c)
             while (true) {
                 const int j0 = c.steps;
                 const double bytes_per_step = spmm_launch_bytes(c.g, c.cur);
-                const int lag = bytes_per_step > kNoLagBytes ? 0 : 1;  // as the host polls below
+                const int lag = poll_lag(c);
                 RD_TRY(launch_step_loop<T>(c, fa, compact_check, lag));
                 RD_CUDA(cudaMemcpyAsync(h + 8, c.b.summary, kHostFlags * sizeof(int32_t), cudaMemcpyDeviceToHost,
                                         c.st));
@@ -1475,10 +1485,10 @@ static rd_status run_forward(RunCtx& c)
         if (c.lagged_polls) {
             // count of active pairs after step j lands in h[4 + j % kSlots]; read the count
             // of the previous step, whose copy has usually completed while step j runs --
-            // or, when a step is long enough (a step's SpMM moves more than kNoLagBytes),
+            // or, when a step is long enough (poll_lag),
             // wait for step j's own count: the GPU idles for the host's reaction time, but
             // converged pairs are packed out one step earlier
-            const int lag = spmm_launch_bytes(c.g, c.cur) > kNoLagBytes ? 0 : 1;
+            const int lag = poll_lag(c);
             const int sl = j % kSlots;
             RD_CUDA(cudaMemcpyAsync(h + 4 + sl, c.b.st.act_count + j + 1, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                     c.st));
@@ -1653,7 +1663,8 @@ static std::vector<SpmmCfg> tune_candidates(const rd_graph* g, int64_t width, bo
         c.nzl = nzl;
         c.kind = kind;
         c.order = order;
-        if (order && !g->row_order) return;
+        // (below a few thousand rows every order is as good, and rounding should not depend on a tie)
+        if (order && (!g->row_order || g->n < 4096)) return;
         if (cfg_known(c, fp64)) v.push_back(c);
     };
     if (single) {
