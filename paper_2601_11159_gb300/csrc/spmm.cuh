@@ -1038,8 +1038,9 @@ __device__ __forceinline__ void acc_add_slot(double (&acc)[2], const float4& x, 
     const double x0 = __hiloint2double(__float_as_int(x.y), __float_as_int(x.x));
     const double x1 = __hiloint2double(__float_as_int(x.w), __float_as_int(x.z));
     if constexpr (WEIGHTED) {
-        acc[0] = fma((double)wv, x0, acc[0]);
-        acc[1] = fma((double)wv, x1, acc[1]);
+        const double w = widen(wv);
+        acc[0] = fma(w, x0, acc[0]);
+        acc[1] = fma(w, x1, acc[1]);
     } else {
         acc[0] += x0;
         acc[1] += x1;

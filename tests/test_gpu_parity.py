@@ -1027,3 +1027,17 @@ def test_potential_passes(rd, mode, k_max, pairs):
     dense_first, _ = G.potential(s, t, sparse_first=False, mode=mode, k_max=k_max, fixed_k=True, tune=False)
     ref, _ = G.potential(s, t, sparse_first=False, graph=False, mode=mode, k_max=k_max, fixed_k=True, tune=False)
     assert np.array_equal(dense_first, ref)
+
+
+@pytest.mark.parametrize("kernel", ["group", "stream", "async"])
+@pytest.mark.parametrize("scale", [1.0, 1e-38, 1e-40, 1e37])
+def test_fp64_weights_of_every_size(rd, kernel, scale):
+    """FP64 steps take FP32 edge weights exactly from denormals to the largest: on a path the
+    resistance is the sum of 1/w."""
+    w = (np.array([1.0, 3.0, 20.0, 7.0]) * scale).astype(np.float32)
+    assert np.all(w > 0) and np.all(np.isfinite(w))
+    G = rd.Graph.from_csr(F.weighted(F.path(5), w))
+    ref = np.cumsum(1.0 / w.astype(np.float64))
+    s, t = np.zeros(4, np.int32), np.arange(1, 5, dtype=np.int32)
+    res = G.query(s, t, mode="fp64", k_max=50, rel_tol=0.0, resid_tol=1e-12, onchip=False, kernel=kernel)
+    assert rel(res.r, ref).max() < FP64_TOL
