@@ -169,11 +169,12 @@ static int32_t label_components(int64_t n, const std::vector<int64_t>& rp, const
 }
 
 // Heavy-row threshold and chunk length: 256 nonzeros where the graph has enough of them to fill the
-// chip many times over, on smaller graphs so many fewer that there are 32 chunk lengths per SM
+// chip many times over, on smaller graphs so many fewer that there are 128 chunk lengths per SM
 // (down to 64), since one warp then works on a chunk alone: on Chung-Lu 20k (394,000 entries, 128
 // FP64 columns) 478 chunks of 256 took 135 us a step, each being 256 rounds of additions on one
 // warp, and light rows of up to 256 left the main kernel half idle at its end; the query of 70
-// pairs takes 2.8 ms with 256 and 1.9 ms with 64. At 2M entries 128 is 4% slower than 256. A
+// pairs takes 2.8 ms with 256 and 1.9 ms with 64. A line at 32 per SM instead of 128 costs a training
+// step over 2M entries 3.02 for 2.75 ms and flows over 3.9M entries 1.03 for 0.93 ms. A
 // hub's chunks are summed by one row group, so a row has at most 128 of them. Graphs small enough
 // for the whole-recurrence kernel keep 256.
 static void choose_chunk(rd_graph* g, const std::vector<int64_t>& rp)
@@ -181,7 +182,7 @@ static void choose_chunk(rd_graph* g, const std::vector<int64_t>& rp)
     if (onchip_smem_bytes(g->n, 4) <= 220 * 1024) return;
     int64_t dmax = 0;
     for (int64_t u = 0; u < g->n; ++u) dmax = std::max<int64_t>(dmax, rp[u + 1] - rp[u]);
-    while (g->heavy_thr > 64 && g->nnz / g->heavy_thr < 32ll * g->sm_count && dmax <= 64ll * g->heavy_thr)
+    while (g->heavy_thr > 64 && g->nnz / g->heavy_thr < 128ll * g->sm_count && dmax <= 64ll * g->heavy_thr)
         g->heavy_thr /= 2;
 }
 
