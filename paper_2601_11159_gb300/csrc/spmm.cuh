@@ -268,21 +268,33 @@ __device__ __forceinline__ void gather_row(const StepArgs<T>& a, int64_t beg, in
         for (int i = 0; i < VEC; ++i) acc_finish(acc[i]);
         return;
     }
-    for (int64_t base = beg; base < end; base += G) {
-        const int cnt = (int)(end - base < G ? end - base : G);
-        const int my_col = li < cnt ? __ldg(a.col + base + li) : 0;
-        float my_w = 1.0f;
-        if constexpr (WEIGHTED) my_w = li < cnt ? __ldg(a.w + base + li) : 0.0f;
+    // a round of U gathers per nonzero lane takes NZL * U indices: with fewer column lanes than U each
+    // lane holds several (with one, half the slots of a 4-lane group stayed empty and were filled
+    // with zeros and added: 857 instructions for four rows of 12 entries at 16 FP32 columns, in a
+    // kernel that issues in 60% of its cycles)
+    constexpr int NH = GS < U ? U / GS : 1;
+    constexpr int CH = G * NH;
+    const uint32_t row_bytes = (uint32_t)(ld * (int64_t)sizeof(T));
+    const char* __restrict__ qb = reinterpret_cast<const char*>(q);
+    for (int base = (int)beg; base < (int)end; base += CH) {
+        const int cnt = (int)end - base < CH ? (int)end - base : CH;
+        int my_col[NH];
+        float my_w[NH];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            my_col[h] = h * G + li < cnt ? __ldg(a.col + base + h * G + li) : 0;
+            if constexpr (WEIGHTED) my_w[h] = h * G + li < cnt ? __ldg(a.w + base + h * G + li) : 0.0f;
+        }
         for (int k0 = 0; k0 < cnt; k0 += NZL * U) {
             T x[U][VEC];
             float wu[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int kk = k0 + zl + u * NZL;
-                const int j = __shfl_sync(mask, my_col, kk & (G - 1), G);
-                if constexpr (WEIGHTED) wu[u] = __shfl_sync(mask, my_w, kk & (G - 1), G);
+                const int kk = k0 + zl + u * NZL;  // in holder h = kk / G: 0, or u / GS with one round a chunk
+                const int j = __shfl_sync(mask, my_col[NH == 1 ? 0 : u / GS], kk & (G - 1), G);
+                if constexpr (WEIGHTED) wu[u] = __shfl_sync(mask, my_w[NH == 1 ? 0 : u / GS], kk & (G - 1), G);
                 if (kk < cnt) {
-                    ld_gather<T, VEC>(x[u], q + (int64_t)j * ld);
+                    ld_gather<T, VEC>(x[u], reinterpret_cast<const T*>(qb + (uint64_t)(uint32_t)j * row_bytes));
                 } else {
 #pragma unroll
                     for (int i = 0; i < VEC; ++i) x[u][i] = T(0);
