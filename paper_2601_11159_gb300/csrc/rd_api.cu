@@ -382,7 +382,7 @@ static int kernel_code(const SpmmCfg& c)
 {
     if (c.kind == 3) return 5;
     if (c.kind == 2) return 4;
-    if (c.kind == 1) return 2;
+    if (c.kind == 1 || c.kind == 4) return 2;
     return c.order ? 3 : 1;
 }
 
@@ -1691,6 +1691,11 @@ static std::vector<SpmmCfg> tune_candidates(const rd_graph* g, int64_t width, bo
     const int avec = fp64 ? 2 : 4;
     for (int64_t tp = std::max<int64_t>(16, width / 8); tp <= std::min<int64_t>(width, 32 * avec); tp <<= 1)
         add(avec, (int)(tp / avec), 1, 3, 0);
+    // the row pipeline, where rows are short (above eight entries its rounds past the first four wait
+    // for their gathers); its row and entry indices are 32-bit
+    if (g->nnz <= 8 * g->n && g->nnz <= INT32_MAX && g->n <= (1 << 30))
+        for (int64_t tp = std::max<int64_t>(16, width / 4); tp <= std::min<int64_t>(width, 32 * avec); tp <<= 1)
+            add(avec, (int)(tp / avec), 1, 4, 0);
     return v;
 }
 

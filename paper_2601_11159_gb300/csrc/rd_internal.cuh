@@ -37,7 +37,8 @@ rd_status cuda_status(cudaError_t e, const char* what);
 // kind 0: row-group kernel (k_spmm, grid-stride over rows); kind 1: row-stream kernel
 // (k_spmm_rows, grid-stride over tasks of consecutive rows; nzl must be 1); kind 2:
 // warp-per-task SpMV (one column); kind 3: row-stream kernel with cp.async gathers into a
-// shared-memory ring (k_spmm_async, FP32 vectors, vec 4, nzl 1).
+// shared-memory ring (k_spmm_async, FP32 vectors, vec 4, nzl 1); kind 4: row pipeline for short
+// rows (k_spmm_pipe, one 16-byte unit of columns per lane, nzl 1).
 struct SpmmCfg {
     int vec = 4, gs = 32, nzl = 1, kind = 0;
     int order = 0;  // row-group kernel: 1 = visit rows by decreasing degree (rd_graph::row_order)

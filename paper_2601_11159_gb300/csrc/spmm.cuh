@@ -271,7 +271,7 @@ __device__ __forceinline__ void gather_row(const StepArgs<T>& a, int64_t beg, in
     // a round of U gathers per nonzero lane takes NZL * U indices: with fewer column lanes than U each
     // lane holds several (with one, half the slots of a 4-lane group stayed empty and were filled
     // with zeros and added: 857 instructions for four rows of 12 entries at 16 FP32 columns, in a
-    // kernel that issues in 60% of its cycles)
+    // kernel that issues in 60% of its cycles; flows on 200,000 vertices 920 us with it, 787 now)
     constexpr int NH = GS < U ? U / GS : 1;
     constexpr int CH = G * NH;
     const uint32_t row_bytes = (uint32_t)(ld * (int64_t)sizeof(T));
@@ -1276,6 +1276,170 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
         }
         if (a.do_reduce) block_partials<T, V, GS, TP>(a, sA, sB, sC, red, slab, lane, warp, gl);
     }
+}
+
+// Row pipeline for graphs of short rows (grids, roads): a warp walks runs of consecutive rows, 32/GS
+// at a time in lockstep, with the loads of the rows ahead in registers -- row bounds three rows
+// ahead, columns and weights two, the first four gathers and the row's own operands one -- so that
+// an entry costs two shuffles, an address and a load beside its arithmetic. The async ring pays
+// about fifteen instructions an entry for its slots, waits and refills, which bounds it where a
+// row is four entries and the elements are double-float. 1024^2 road grid, 16
+// columns: 200 us a step against 243 (row-group) in double-float, 111 against 136 in FP32; 500^2 at
+// 16 FP64 columns 101 against 123; at 64 double-float columns the ring is as fast.
+constexpr int kPipeRows = 128;  // rows of a run
+
+template <typename T, int GS, bool WEIGHTED>
+__global__ void __launch_bounds__(kBlock, 2) k_spmm_pipe(const StepArgs<T> a)
+{
+    constexpr int V = kAsyncVec<T>;
+    constexpr int TP = V * GS;
+    constexpr int NG = 32 / GS;
+    constexpr int U = 4;
+    constexpr unsigned kAll = 0xffffffffu;
+    __shared__ double red[kWarps][TP];
+    if (step_inactive(a)) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int gl = lane % GS, grp = lane / GS;
+    const int nslab = (int)(a.ld / TP);
+    const int64_t ld = a.ld;
+    const uint32_t row_bytes = (uint32_t)(ld * (int64_t)sizeof(T));
+    const int n = (int)a.n;
+    const int nruns = (n + kPipeRows - 1) / kPipeRows;
+    const int nwarps = gridDim.x * kWarps;
+
+    struct Bounds {       // a row's entries; len < 0: heavy
+        int beg, len;
+    };
+    struct Cols {         // this lane's entry of the row
+        int col;
+        float w;
+    };
+    struct Own {          // the row's own operands, as loaded
+        float4 qp, qc;
+        T invd, deg;
+    };
+    auto open = [](T (&v)[V], const float4& r) { memcpy(v, &r, 16); };
+    for (int slab = 0; slab < nslab; ++slab) {
+        const int64_t c0 = (int64_t)slab * TP + gl * V;
+        const char* qb = reinterpret_cast<const char*>(a.qcur + c0);
+        T bt[V];
+        ld_plain<T, V>(bt, step_cf_beta(a) + c0);
+        Acc<T> sA[V], sB[V], sC[V];
+        auto bounds = [&](int row, int end) {
+            Bounds b{0, 0};
+            if (row < end) {
+                const int64_t e0 = a.row_ptr[row], e1 = a.row_ptr[row + 1];
+                b.beg = (int)e0;
+                b.len = e1 - e0 > a.heavy_thr ? -1 : (int)(e1 - e0);
+            }
+            return b;
+        };
+        auto columns = [&](const Bounds& b, int first) {
+            Cols c{0, 0.f};
+            if (first + gl < b.len) {
+                c.col = __ldg(a.col + b.beg + first + gl);
+                if constexpr (WEIGHTED) c.w = __ldg(a.w + b.beg + first + gl);
+            }
+            return c;
+        };
+        auto gather = [&](float4& x, const Cols& c, int k, bool take) {
+            const int j = __shfl_sync(kAll, c.col, k, GS);
+            if (take) x = __ldg(reinterpret_cast<const float4*>(qb + (uint64_t)(uint32_t)j * row_bytes));
+        };
+        float4 x[U];      // the first gathers of the current row, refilled once they are summed
+        auto start = [&](Own& o, int row, int end, const Bounds& b, const Cols& c) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) gather(x[u], c, u, u < b.len);
+            if (row < end) {
+                o.qp = __ldcs(reinterpret_cast<const float4*>(a.qprev + (int64_t)row * ld + c0));
+                o.qc = __ldg(reinterpret_cast<const float4*>(qb + (uint64_t)(uint32_t)row * row_bytes));
+                o.invd = a.invdeg[row];
+                o.deg = a.deg[row];
+            }
+        };
+        auto add = [&](T (&acc)[V], const float4& r, float w) {
+            T x[V];
+            open(x, r);
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                if constexpr (WEIGHTED) acc_mul_add_w(acc[i], w, x[i]);
+                else acc_add(acc[i], x[i]);
+            }
+        };
+        for (int run = blockIdx.x * kWarps + warp; run < nruns; run += nwarps) {
+            const int r0 = run * kPipeRows + grp;
+            const int end = run * kPipeRows + kPipeRows < n ? run * kPipeRows + kPipeRows : n;
+            Bounds b0 = bounds(r0, end), b1 = bounds(r0 + NG, end), b2 = bounds(r0 + 2 * NG, end);
+            Cols k0 = columns(b0, 0), k1 = columns(b1, 0);
+            Own cur, nxt;
+            start(cur, r0, end, b0, k0);
+            for (int row = r0; row - grp < end; row += NG) {  // uniform over the warp
+                const Bounds b3 = bounds(row + 3 * NG, end);
+                const Cols k2 = columns(b2, 0);
+                T acc[V];
+#pragma unroll
+                for (int i = 0; i < V; ++i) acc[i] = T(0);
+                const int most = NG == 1 ? b0.len : __reduce_max_sync(kAll, b0.len);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (u >= most) break;
+                    float w = 1.f;
+                    if constexpr (WEIGHTED) w = __shfl_sync(kAll, k0.w, u, GS);
+                    if (u < b0.len) add(acc, x[u], w);
+                }
+                // entries past the first four (and past the GS held by the lanes)
+                for (int f = 0; f < most; f += GS) {
+                    const Cols k = f == 0 ? k0 : columns(b0, f);
+                    for (int p = f == 0 ? U : 0; p < GS && f + p < most; p += U) {
+                        float4 x2[U];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) gather(x2[u], k, p + u, f + p + u < b0.len);
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            float w = 1.f;
+                            if constexpr (WEIGHTED) w = __shfl_sync(kAll, k.w, p + u, GS);
+                            if (f + p + u < b0.len) add(acc, x2[u], w);
+                        }
+                    }
+                }
+                start(nxt, row + NG, end, b1, k1);  // in flight behind the epilogue and the other warps
+#pragma unroll
+                for (int i = 0; i < V; ++i) acc_finish(acc[i]);
+                if (b0.len < 0) heavy_row_sum<T, V, 1>(a, row, c0, 0, acc);
+                __syncwarp();
+                if (row < end) {
+                    T qp[V], qc[V];
+                    open(qp, cur.qp);
+                    open(qc, cur.qc);
+                    async_epilogue<T, V>(a, row, c0, cur.invd, cur.deg, acc, bt, qp, qc, sA, sB, sC);
+                }
+                b0 = b1;
+                b1 = b2;
+                b2 = b3;
+                k0 = k1;
+                k1 = k2;
+                cur = nxt;
+            }
+        }
+        if (a.do_reduce) block_partials<T, V, GS, TP>(a, sA, sB, sC, red, slab, lane, warp, gl);
+    }
+}
+
+template <typename T, int GS>
+bool launch_pipe_cfg(bool weighted, int grid, cudaStream_t st, const StepArgs<T>& a)
+{
+    if (weighted) k_spmm_pipe<T, GS, true><<<grid, kBlock, 0, st>>>(a);
+    else k_spmm_pipe<T, GS, false><<<grid, kBlock, 0, st>>>(a);
+    return true;
+}
+
+template <typename T, int GS>
+int occupancy_pipe_cfg(bool weighted)
+{
+    int nb = 0;
+    if (weighted) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmm_pipe<T, GS, true>, kBlock, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmm_pipe<T, GS, false>, kBlock, 0);
+    return nb;
 }
 
 template <typename T, int GS>

@@ -42,6 +42,14 @@ bool launch_spmm_df64(const SpmmCfg& c, bool weighted, bool heavy, int grid, cud
 #undef X
         return false;
     }
+    if (c.kind == 4 && !heavy) {
+        if (c.vec != 2 || c.nzl != 1) return false;
+#define X(G) \
+    if (c.gs == G) return launch_pipe_cfg<df64, G>(weighted, grid, st, a);
+        RD_DF64_ASYNC(X)
+#undef X
+        return false;
+    }
     if (c.kind == 2 && !heavy) return launch_spmv_tasks<df64>(weighted, grid, st, a);
     if (c.kind == 1 && !heavy) {
 #define X(V, G) \
@@ -66,6 +74,14 @@ int spmm_blocks_per_sm_df64(const SpmmCfg& c, bool weighted, bool heavy)
         if (c.vec != 2 || c.nzl != 1) return 0;
 #define X(G) \
     if (c.gs == G) return occupancy_async_cfg<df64, G>(weighted, heavy);
+        RD_DF64_ASYNC(X)
+#undef X
+        return 0;
+    }
+    if (c.kind == 4 && !heavy) {
+        if (c.vec != 2 || c.nzl != 1) return 0;
+#define X(G) \
+    if (c.gs == G) return occupancy_pipe_cfg<df64, G>(weighted);
         RD_DF64_ASYNC(X)
 #undef X
         return 0;

@@ -42,6 +42,14 @@ bool launch_spmm_f64(const SpmmCfg& c, bool weighted, bool heavy, int grid, cuda
 #undef X
         return false;
     }
+    if (c.kind == 4 && !heavy) {
+        if (c.vec != 2 || c.nzl != 1) return false;
+#define X(G) \
+    if (c.gs == G) return launch_pipe_cfg<double, G>(weighted, grid, st, a);
+        RD_F64_ASYNC(X)
+#undef X
+        return false;
+    }
     if (c.kind == 2 && !heavy) return launch_spmv_tasks<double>(weighted, grid, st, a);
     if (c.kind == 1 && !heavy) {
 #define X(V, G) \
@@ -66,6 +74,14 @@ int spmm_blocks_per_sm_f64(const SpmmCfg& c, bool weighted, bool heavy)
         if (c.vec != 2 || c.nzl != 1) return 0;
 #define X(G) \
     if (c.gs == G) return occupancy_async_cfg<double, G>(weighted, heavy);
+        RD_F64_ASYNC(X)
+#undef X
+        return 0;
+    }
+    if (c.kind == 4 && !heavy) {
+        if (c.vec != 2 || c.nzl != 1) return 0;
+#define X(G) \
+    if (c.gs == G) return occupancy_pipe_cfg<double, G>(weighted);
         RD_F64_ASYNC(X)
 #undef X
         return 0;
@@ -96,7 +112,7 @@ std::vector<SpmmCfg> spmm_configs_f64()
 #define X(V, G) v.push_back(SpmmCfg{V, G, 1, 1});
     RD_F64_ROWS(X)
 #undef X
-#define X(G) v.push_back(SpmmCfg{2, G, 1, 3});
+#define X(G) v.push_back(SpmmCfg{2, G, 1, 3}), v.push_back(SpmmCfg{2, G, 1, 4});
     RD_F64_ASYNC(X)
 #undef X
     return v;

@@ -1041,3 +1041,30 @@ def test_fp64_weights_of_every_size(rd, kernel, scale):
     s, t = np.zeros(4, np.int32), np.arange(1, 5, dtype=np.int32)
     res = G.query(s, t, mode="fp64", k_max=50, rel_tol=0.0, resid_tol=1e-12, onchip=False, kernel=kernel)
     assert rel(res.r, ref).max() < FP64_TOL
+
+
+@pytest.mark.parametrize("mode,tol", [("fp32", 2e-5), ("fp64", 1e-11), ("df64", 1e-11)])
+@pytest.mark.parametrize("graph", ["grid150w", "tree", "star+path"])
+@pytest.mark.parametrize("pairs", [5, 20, 40, 70])
+def test_short_row_graphs_match_oracle_history(rd, mode, tol, graph, pairs):
+    """Graphs of short rows, where the row pipeline is a candidate of the tuner: rows of one to four
+    entries, a tree with some of more than four, a hub among rows of two, at several tile widths;
+    whatever kernel the tuner takes has the oracle's r_k after k steps (the bars that
+    test_fixed_k_matches_oracle_history sets for it) and repeats bit for bit."""
+    if graph == "grid150w":
+        g = F.grid_deleted(150, 0.05, 5)
+    elif graph == "tree":
+        g = F.random_tree(20001, 7)
+    else:
+        a, b, _ = F.star(700).undirected_edges()
+        c, d, _ = F.path(20000).undirected_edges()
+        g = to_csr(20699, np.concatenate([a, c + 699]), np.concatenate([b, d + 699]))
+    s, t = F.random_pairs(g.n, pairs, 9)
+    G = rd.Graph.from_csr(g)
+    for k in (2, 12, 25):
+        res = G.query(s, t, mode=mode, k_max=k, fixed_k=True)
+        ref = np.array([lanczos.lanczos_pair(g, int(a), int(b), k_max=k)["r"] for a, b in zip(s[:5], t[:5])])
+        m = res.iters[:5] == k
+        assert m.any()
+        assert rel(res.r[:5][m], ref[m]).max() < tol, (k, rel(res.r[:5][m], ref[m]).max())
+        assert np.array_equal(G.query(s, t, mode=mode, k_max=k, fixed_k=True).r, res.r)
