@@ -135,6 +135,37 @@ __device__ __forceinline__ void st_plain(T* p, const T (&r)[VEC])
     }
 }
 
+// A lane's VEC elements as loaded, in units the load instructions return: arrays of these stay in
+// registers where arrays of elements filled through memcpy under a condition went to local memory
+// (FP64: 70 columns on Chung-Lu 20k 1,981 -> 1,942 us a query, 50 steps of the Power Method on
+// 100,000 vertices 5,494 -> 5,242 us; FP32 the same).
+template <typename T, int VEC>
+struct RawVec {
+    static constexpr int B = (int)sizeof(T) * VEC;
+    using Unit = typename std::conditional<(B >= 16), float4, typename std::conditional<B == 8, float2, float>::type>::type;
+    static constexpr int N = B >= 16 ? B / 16 : 1;
+    Unit u[N];
+    __device__ __forceinline__ void gather(const void* p)
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) u[i] = __ldg(reinterpret_cast<const Unit*>(p) + i);
+    }
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            if constexpr (B >= 16) u[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            else if constexpr (B == 8) u[i] = make_float2(0.f, 0.f);
+            else u[i] = 0.f;
+        }
+    }
+    __device__ __forceinline__ void open(T (&v)[VEC]) const
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) memcpy(reinterpret_cast<char*>(v) + i * (B / N), &u[i], B / N);
+    }
+};
+
 // Gathers with an L2 eviction-priority hint (createpolicy + ld.global.nc.L2::cache_hint):
 // rows that many nonzeros point to are kept (evict_last), the long tail of rarely
 // gathered rows is let go first (evict_first), so the tail does not push the hot rows
@@ -286,7 +317,7 @@ __device__ __forceinline__ void gather_row(const StepArgs<T>& a, int64_t beg, in
             if constexpr (WEIGHTED) my_w[h] = h * G + li < cnt ? __ldg(a.w + base + h * G + li) : 0.0f;
         }
         for (int k0 = 0; k0 < cnt; k0 += NZL * U) {
-            T x[U][VEC];
+            RawVec<T, VEC> x[U];
             float wu[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -294,10 +325,9 @@ __device__ __forceinline__ void gather_row(const StepArgs<T>& a, int64_t beg, in
                 const int j = __shfl_sync(mask, my_col[NH == 1 ? 0 : u / GS], kk & (G - 1), G);
                 if constexpr (WEIGHTED) wu[u] = __shfl_sync(mask, my_w[NH == 1 ? 0 : u / GS], kk & (G - 1), G);
                 if (kk < cnt) {
-                    ld_gather<T, VEC>(x[u], reinterpret_cast<const T*>(qb + (uint64_t)(uint32_t)j * row_bytes));
+                    x[u].gather(qb + (uint64_t)(uint32_t)j * row_bytes);
                 } else {
-#pragma unroll
-                    for (int i = 0; i < VEC; ++i) x[u][i] = T(0);
+                    x[u].zero();
                 }
             }
 #pragma unroll
@@ -306,10 +336,12 @@ __device__ __forceinline__ void gather_row(const StepArgs<T>& a, int64_t beg, in
                 // 500^2 road grid, rows of four, 16 columns, 241 us a step with the zeros and 200
                 // without; in FP32 the test costs more (a training step 3.9 against 3.3 ms)
                 if (std::is_same<T, double>::value && k0 + zl + u * NZL >= cnt) break;
+                T e[VEC];
+                x[u].open(e);
 #pragma unroll
                 for (int i = 0; i < VEC; ++i) {
-                    if constexpr (WEIGHTED) acc_mul_add_w(acc[i], wu[u], x[u][i]);
-                    else acc_add(acc[i], x[u][i]);
+                    if constexpr (WEIGHTED) acc_mul_add_w(acc[i], wu[u], e[i]);
+                    else acc_add(acc[i], e[i]);
                 }
             }
         }
