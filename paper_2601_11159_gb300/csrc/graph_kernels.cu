@@ -236,7 +236,12 @@ static int grid_for(int64_t work, int sm)
 rd_status rows_sorted_symmetric(rd_graph* g, cudaStream_t st)
 {
     int32_t* f = nullptr;
-    if (g->w && !g->mirror) RD_CUDA(cudaMalloc((void**)&g->mirror, sizeof(int32_t) * (g->nnz > 0 ? g->nnz : 1)));
+    // without memory for the mirrors, or with entries past their 32 bits, later weights are searched
+    if (g->w && !g->mirror && g->nnz <= INT32_MAX &&
+        cudaMalloc((void**)&g->mirror, sizeof(int32_t) * (g->nnz > 0 ? g->nnz : 1)) != cudaSuccess) {
+        g->mirror = nullptr;
+        cudaGetLastError();
+    }
     RD_CUDA(cudaMallocAsync((void**)&f, sizeof(int32_t), st));
     RD_CUDA(cudaMemsetAsync(f, 0, sizeof(int32_t), st));
     if (g->n > 0)
