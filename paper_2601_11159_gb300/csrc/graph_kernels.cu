@@ -236,8 +236,8 @@ static int grid_for(int64_t work, int sm)
 rd_status rows_sorted_symmetric(rd_graph* g, cudaStream_t st)
 {
     int32_t* f = nullptr;
-    // without memory for the mirrors, or with entries past their 32 bits, later weights are searched
-    if (g->w && !g->mirror && g->nnz <= INT32_MAX &&
+    // without memory for the mirrors later weights are searched
+    if (g->w && !g->mirror &&
         cudaMalloc((void**)&g->mirror, sizeof(int32_t) * (g->nnz > 0 ? g->nnz : 1)) != cudaSuccess) {
         g->mirror = nullptr;
         cudaGetLastError();

@@ -1692,8 +1692,8 @@ static std::vector<SpmmCfg> tune_candidates(const rd_graph* g, int64_t width, bo
     for (int64_t tp = std::max<int64_t>(16, width / 8); tp <= std::min<int64_t>(width, 32 * avec); tp <<= 1)
         add(avec, (int)(tp / avec), 1, 3, 0);
     // the row pipeline, where rows are short (above eight entries its rounds past the first four wait
-    // for their gathers); its row and entry indices are 32-bit
-    if (g->nnz <= 8 * g->n && g->nnz <= INT32_MAX && g->n <= (1 << 30))
+    // for their gathers); its rows past the last are counted in 32 bits
+    if (g->nnz <= 8 * g->n && g->n <= (1 << 30))
         for (int64_t tp = std::max<int64_t>(16, width / 4); tp <= std::min<int64_t>(width, 32 * avec); tp <<= 1)
             add(avec, (int)(tp / avec), 1, 4, 0);
     return v;
