@@ -768,17 +768,16 @@ __device__ __forceinline__ void row_epilogue_b(const StepArgs<T>& a, int row, in
 // registers, which lets more warps be resident to keep gathers in flight. Three blocks (80
 // registers) hold a round's eight 16-byte gathers beside the sums; with four (64) some of them
 // wait for registers: a training step on Chung-Lu 100k 2,624 -> 2,458 us with three, flows on
-// 200,000 vertices 779 -> 728 us, FP64 unchanged.
-#ifndef RD_GROUP_MINB
-#define RD_GROUP_MINB 3
-#endif
+// 200,000 vertices 779 -> 728 us (768 with two). Elements of 8 bytes take two (128 registers; at
+// 80 the weighted kernels spill): 70 FP64 columns on Chung-Lu 20k 1,820 -> 1,792 us a query, 50
+// steps of the Power Method on 100,000 vertices 5,250 -> 5,116.
 #ifndef RD_GROUP_SMEM
 #define RD_GROUP_SMEM 1
 #endif
 template <typename T, int VEC>
 inline constexpr bool kGroupSmemAcc = RD_GROUP_SMEM && (int)sizeof(T) * VEC <= 16;
 template <typename T, int VEC>
-inline constexpr int kGroupMinBlocks = kGroupSmemAcc<T, VEC> ? RD_GROUP_MINB : 1;
+inline constexpr int kGroupMinBlocks = kGroupSmemAcc<T, VEC> ? (sizeof(T) == 4 ? 3 : 2) : 1;
 
 
 template <typename T, int VEC, int GS, int NZL, bool WEIGHTED>
