@@ -160,6 +160,86 @@ __device__ __forceinline__ void acc_finish<df64>(df64& acc)
     acc = df_two_sum(acc.hi, acc.lo);
 }
 
+// Two double-float numbers, their leading and their trailing parts each in a register pair, for the
+// packed FP32 instructions: the operations above with the same roundings, on two columns in one
+// issue slot. A difference is a multiply-add by -1, and products (df64x2n) carry minus their
+// trailing part, so that nothing is negated on the way.
+struct df64x2 {
+    float2 hi, lo;
+};
+struct df64x2n {
+    float2 hi, nlo;
+};
+
+__device__ __forceinline__ df64x2 df_pack(df64 a, df64 b)
+{
+    return df64x2{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)};
+}
+__device__ __forceinline__ void df_unpack(const df64x2& v, df64& a, df64& b)
+{
+    a = df64(v.hi.x, v.lo.x, 0);
+    b = df64(v.hi.y, v.lo.y, 0);
+}
+
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
+// s + e = a + b exactly, as df_two_sum.
+__device__ __forceinline__ df64x2 df_two_sum(float2 a, float2 b)
+{
+    const float2 s = __fadd2_rn(a, b);
+    const float2 bb = sub2(s, a);
+    return df64x2{s, __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+
+// Renormalised hi + lo of a two-sum t and the trailing parts l, as operator+ ends.
+__device__ __forceinline__ df64x2 df_renorm(float2 t, float2 l)
+{
+    const float2 s = __fadd2_rn(t, l);
+    return df64x2{s, sub2(l, sub2(s, t))};
+}
+
+__device__ __forceinline__ df64x2 operator+(const df64x2& a, const df64x2n& b)
+{
+    const df64x2 t = df_two_sum(a.hi, b.hi);
+    return df_renorm(t.hi, __fadd2_rn(sub2(a.lo, b.nlo), t.lo));
+}
+
+__device__ __forceinline__ df64x2 operator+(const df64x2n& a, const df64x2n& b)
+{
+    const df64x2 t = df_two_sum(a.hi, b.hi);
+    return df_renorm(t.hi, sub2(t.lo, __fadd2_rn(a.nlo, b.nlo)));
+}
+
+// a b unnormalised (as df_prod), with `na` = -a.
+__device__ __forceinline__ df64x2n df_prod(float2 a_hi, const df64x2& na, const df64x2& b)
+{
+    const float2 p = __fmul2_rn(a_hi, b.hi);
+    float2 m = __ffma2_rn(na.hi, b.hi, p);  // minus the exact low part of a.hi * b.hi
+    m = __ffma2_rn(na.hi, b.lo, m);
+    m = __ffma2_rn(na.lo, b.hi, m);
+    return df64x2n{p, m};
+}
+
+// acc_mul_add_w and acc_add on two columns.
+__device__ __forceinline__ void acc_mul_add_w(df64 (&acc)[2], float w, const df64x2& x)
+{
+    const float2 w2 = make_float2(w, w), nw = make_float2(-w, -w);
+    df64x2 a = df_pack(acc[0], acc[1]);
+    const float2 p = __fmul2_rn(w2, x.hi);
+    float2 m = __ffma2_rn(nw, x.hi, p);
+    m = __ffma2_rn(nw, x.lo, m);
+    const df64x2 s = df_two_sum(a.hi, p);
+    a = df64x2{s.hi, __fadd2_rn(a.lo, sub2(s.lo, m))};
+    df_unpack(a, acc[0], acc[1]);
+}
+__device__ __forceinline__ void acc_add(df64 (&acc)[2], const df64x2& x)
+{
+    df64x2 a = df_pack(acc[0], acc[1]);
+    const df64x2 s = df_two_sum(a.hi, x.hi);
+    a = df64x2{s.hi, __fadd2_rn(a.lo, __fadd2_rn(s.lo, x.lo))};
+    df_unpack(a, acc[0], acc[1]);
+}
+
 // Warp shuffles of element values (both halves move together).
 __device__ __forceinline__ float shfl_xor_t(unsigned mask, float v, int off, int width = 32)
 {

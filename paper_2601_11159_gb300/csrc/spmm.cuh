@@ -432,32 +432,39 @@ __device__ __forceinline__ void row_epilogue(const StepArgs<T>& a, int64_t row, 
     }
 }
 
-// The same in double-float, with the products left unnormalised where they go straight into a sum
-// or another product: 64 FP32 operations per element instead of 79, in kernels that are bound by
-// instruction issue (1024^2 road grid, 64 columns, 200 steps with k_spmm_async: 165.3 -> 161.7 ms).
-template <int VEC>
-__device__ __forceinline__ void row_epilogue(const StepArgs<df64>& a, int64_t row, int64_t c0, df64 invd, df64 du,
-                                             const df64 (&acc)[VEC], const df64 (&bt)[VEC], const df64 (&qp)[VEC],
-                                             const df64 (&qc)[VEC], Acc<df64> (&sA)[VEC], Acc<df64> (&sB)[VEC],
-                                             Acc<df64> (&sC)[VEC])
+// The same in double-float on the two columns of a lane slot, with the products left unnormalised where
+// they go straight into a sum or another product: 64 packed FP32 operations for both columns. 1024^2 road
+// grid, 64 columns, 200 steps with k_spmm_async: 165.3 ms with every product normalised, 161.7
+// without, 159.8 packed (343 instructions a row and warp; the kernel then issues in 60% of its
+// cycles, against 73% before, and waits for its operands).
+__device__ __forceinline__ void row_epilogue_x2(const StepArgs<df64>& a, int64_t row, int64_t c0, df64 invd, df64 du,
+                                                const df64 (&acc)[2], const df64 (&bt)[2], const df64 (&qp)[2],
+                                                const df64 (&qc)[2], Acc<df64> (&sA)[2], Acc<df64> (&sB)[2],
+                                                Acc<df64> (&sC)[2])
 {
-    df64 wv[VEC];
+    df64 wv[2];
+    df64x2 w;
     if (a.lazy_walk) {
 #pragma unroll
-        for (int i = 0; i < VEC; ++i) wv[i] = df64(0.5) * (invd * acc[i]) + df64(0.5) * qc[i];
+        for (int i = 0; i < 2; ++i) wv[i] = df64(0.5) * (invd * acc[i]) + df64(0.5) * qc[i];
+        w = df_pack(wv[0], wv[1]);
     } else {
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) wv[i] = df_prod(invd, acc[i]) - df_prod(bt[i], qp[i]);
+        const df64x2 b = df_pack(bt[0], bt[1]);
+        const df64x2n x = df_prod(make_float2(invd.hi, invd.hi), df_pack(-invd, -invd), df_pack(acc[0], acc[1]));
+        w = x + df_prod(make_float2(-b.hi.x, -b.hi.y), b, df_pack(qp[0], qp[1]));
+        df_unpack(w, wv[0], wv[1]);
     }
-    st_stream<df64, VEC>(a.w_out + row * a.ld + c0, wv);
+    st_stream<df64, 2>(a.w_out + row * a.ld + c0, wv);
     if (a.do_reduce) {
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) {
-            const df64 dw = df_prod(du, wv[i]);
-            sA[i].add(df_prod(dw, qc[i]));
-            sB[i].add(df_prod(dw, wv[i]));
-            sC[i].add(dw);
-        }
+        const df64x2 nd = df_pack(-du, -du);
+        const df64x2n dw = df_prod(make_float2(du.hi, du.hi), nd, w);
+        const df64x2 ndw{__fmul2_rn(nd.hi, w.hi), dw.nlo};
+        const df64x2 sa = df_pack(sA[0].s, sA[1].s) + df_prod(dw.hi, ndw, df_pack(qc[0], qc[1]));
+        const df64x2 sb = df_pack(sB[0].s, sB[1].s) + df_prod(dw.hi, ndw, w);
+        const df64x2 sc = df_pack(sC[0].s, sC[1].s) + dw;
+        df_unpack(sa, sA[0].s, sA[1].s);
+        df_unpack(sb, sB[0].s, sB[1].s);
+        df_unpack(sc, sC[0].s, sC[1].s);
     }
 }
 
@@ -1136,14 +1143,9 @@ __device__ __forceinline__ void acc_add_slot(double (&acc)[2], const float4& x, 
 template <bool WEIGHTED>
 __device__ __forceinline__ void acc_add_slot(df64 (&acc)[2], const float4& x, float wv)
 {
-    const df64 x0(x.x, x.y, 0), x1(x.z, x.w, 0);
-    if constexpr (WEIGHTED) {
-        acc_mul_add_w(acc[0], wv, x0);
-        acc_mul_add_w(acc[1], wv, x1);
-    } else {
-        acc_add(acc[0], x0);
-        acc_add(acc[1], x1);
-    }
+    const df64x2 v{make_float2(x.x, x.z), make_float2(x.y, x.w)};
+    if constexpr (WEIGHTED) acc_mul_add_w(acc, wv, v);
+    else acc_add(acc, v);
 }
 template <bool WEIGHTED>
 __device__ __forceinline__ void acc_add_slot(float (&acc)[4], const float4& x, float wv)
@@ -1241,7 +1243,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async_heavy(cons
 template <typename T, int V, class... X>
 __device__ __forceinline__ void async_epilogue(X&&... x)
 {
-    if constexpr (std::is_same<T, df64>::value) row_epilogue<V>(x...);
+    if constexpr (std::is_same<T, df64>::value) row_epilogue_x2(x...);
     else row_epilogue<T, V>(x...);
 }
 
@@ -1432,15 +1434,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_spmm_pipe(const StepArgs<T> a)
                 o.deg = a.deg[row];
             }
         };
-        auto add = [&](T (&acc)[V], const float4& r, float w) {
-            T x[V];
-            open(x, r);
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                if constexpr (WEIGHTED) acc_mul_add_w(acc[i], w, x[i]);
-                else acc_add(acc[i], x[i]);
-            }
-        };
+        auto add = [&](T (&acc)[V], const float4& r, float w) { acc_add_slot<WEIGHTED>(acc, r, w); };
         for (int run = blockIdx.x * kWarps + warp; run < nruns; run += nwarps) {
             const int r0 = run * kPipeRows + grp;
             const int end = run * kPipeRows + kPipeRows < n ? run * kPipeRows + kPipeRows : n;
