@@ -1363,7 +1363,10 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
 // row is four entries and the elements are double-float. 1024^2 road grid, 16
 // columns: 200 us a step against 243 (row-group) in double-float, 111 against 136 in FP32; 500^2 at
 // 16 FP64 columns 101 against 123; at 64 double-float columns the ring is as fast.
-constexpr int kPipeRows = 128;  // rows of a run
+// A run is 32 rows, or 16 where a warp has fewer than eight runs of 32: the last of a few long runs
+// leaves most warps idle (500^2 at 16 FP64 columns, 100 potential steps: 15,836 us with runs of 128 rows,
+// 15,832 with 64, 14,824 with 32, 14,685 with 16), and each run starts its loads afresh.
+__device__ __forceinline__ int pipe_run_rows(int n, int nwarps) { return n / 32 < 8 * nwarps ? 16 : 32; }
 
 template <typename T, int GS, bool WEIGHTED>
 __global__ void __launch_bounds__(kBlock, 2) k_spmm_pipe(const StepArgs<T> a)
@@ -1381,8 +1384,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_spmm_pipe(const StepArgs<T> a)
     const int64_t ld = a.ld;
     const uint32_t row_bytes = (uint32_t)(ld * (int64_t)sizeof(T));
     const int n = (int)a.n;
-    const int nruns = (n + kPipeRows - 1) / kPipeRows;
     const int nwarps = gridDim.x * kWarps;
+    const int run_rows = pipe_run_rows(n, nwarps);
+    const int nruns = (n + run_rows - 1) / run_rows;
 
     struct Bounds {       // a row's entries; len < 0: heavy
         int beg, len;
@@ -1436,8 +1440,8 @@ __global__ void __launch_bounds__(kBlock, 2) k_spmm_pipe(const StepArgs<T> a)
         };
         auto add = [&](T (&acc)[V], const float4& r, float w) { acc_add_slot<WEIGHTED>(acc, r, w); };
         for (int run = blockIdx.x * kWarps + warp; run < nruns; run += nwarps) {
-            const int r0 = run * kPipeRows + grp;
-            const int end = run * kPipeRows + kPipeRows < n ? run * kPipeRows + kPipeRows : n;
+            const int r0 = run * run_rows + grp;
+            const int end = run * run_rows + run_rows < n ? run * run_rows + run_rows : n;
             Bounds b0 = bounds(r0, end), b1 = bounds(r0 + NG, end), b2 = bounds(r0 + 2 * NG, end);
             Cols k0 = columns(b0, 0), k1 = columns(b1, 0);
             Own cur, nxt;
