@@ -186,9 +186,21 @@ static void choose_chunk(rd_graph* g, const std::vector<int64_t>& rp)
         g->heavy_thr /= 2;
 }
 
+// Nonzeros of a row-stream task: 32 rows of the mean degree, 128 to 512. A warp sweeps a task's rows one
+// after another, so on graphs of short rows a task of 512 nonzeros is 130 rows: the 1024^2 road
+// grid has 3.2 of them for each of the async kernel's warps (four rounds), and what all warps sweep at
+// once does not stay in L2. 64 double-float columns there, 200 steps: 159.6 ms with 512 a task, 156.1
+// with 256, 149.4 with 128, 150.3 with 64, 157.2 with 32. On Chung-Lu 1M (20 a row), 256 columns,
+// 512 and 256 are within 1% and 128 and 64 cost 1 and 5%.
+static int task_length(const rd_graph* g)
+{
+    return (int)std::min<int64_t>(512, std::max<int64_t>(128, g->n ? 32 * g->nnz / g->n : 0));
+}
+
 static rd_status build_heavy(rd_graph* g, const std::vector<int64_t>& rp)
 {
     choose_chunk(g, rp);
+    g->task_nnz = task_length(g);
     std::vector<int32_t> rows, first, cb, ce;
     first.push_back(0);
     for (int64_t u = 0; u < g->n; ++u) {

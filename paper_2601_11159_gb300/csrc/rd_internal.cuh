@@ -331,7 +331,7 @@ struct rd_graph {
     int32_t* chunk_beg = nullptr;
     int32_t* chunk_end = nullptr;
     // row-stream tasks: consecutive rows with at most task_nnz nonzeros, heavy rows alone
-    int task_nnz = 512;
+    int task_nnz = 512;            // (see task_length)
     int64_t ntasks = 0;
     int32_t* task_row = nullptr;
     // rows by decreasing degree (stable: equal degrees in row order)
