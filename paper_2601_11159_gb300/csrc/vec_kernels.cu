@@ -1886,13 +1886,13 @@ static int cluster_size(const OnchipArgs& a)
     return C;
 }
 
+// Rows per CTA, even so that what follows them stays 8-byte aligned.
+static int cluster_rows(const OnchipArgs& a, int C) { return (int)(((a.n + C - 1) / C + 1) & ~1ll); }
+
 // Launches the kernel with C CTAs per pair; 0 if it does not fit. For C > 1 the entries get all the
 // shared memory that is left (one CTA of a cluster then occupies an SM: the FP64 rate per SM is
 // what a cluster multiplies); for C = 1 what the graph needs, or none where it does not fit, so
 // that several pairs share an SM.
-// Rows per CTA, even so that what follows them stays 8-byte aligned.
-static int cluster_rows(const OnchipArgs& a, int C) { return (int)(((a.n + C - 1) / C + 1) & ~1ll); }
-
 template <typename T, bool WEIGHTED, bool COPY, int NT>
 static int launch_cluster_t(cudaStream_t st, const OnchipArgs& a, int C)
 {
