@@ -126,7 +126,7 @@ static void free_graph(rd_graph* g)
 {
     if (!g) return;
     void* ptrs[] = {g->row_ptr, g->col, g->w, g->keep_idx, g->deg64, g->invdeg64, g->deg32, g->invdeg32,
-                    g->comp, g->heavy_rows, g->heavy_first, g->chunk_beg, g->chunk_end, g->task_row,
+                    g->comp, g->heavy_rows, g->heavy_first, g->chunk_beg, g->chunk_end, g->task_row, g->spmv_task_row,
                     g->row_order, g->entry_row, g->degdf, g->invdegdf, g->ws.base, g->mirror, g->check_scratch};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -192,6 +192,8 @@ static void choose_chunk(rd_graph* g, const std::vector<int64_t>& rp)
 // once does not stay in L2. 64 double-float columns there, 200 steps: 159.6 ms with 512 a task, 156.1
 // with 256, 149.4 with 128, 150.3 with 64, 157.2 with 32. On Chung-Lu 1M (20 a row), 256 columns,
 // 512 and 256 are within 1% and 128 and 64 cost 1 and 5%.
+// k_spmv_tasks (one column, a lane a row) keeps 512: tasks of 34 rows take it two rounds for
+// little over one, 3,326 for 2,744 us on 30 FP64 steps of a 1000^2 road grid.
 static int task_length(const rd_graph* g)
 {
     return (int)std::min<int64_t>(512, std::max<int64_t>(128, g->n ? 32 * g->nnz / g->n : 0));
@@ -200,7 +202,6 @@ static int task_length(const rd_graph* g)
 static rd_status build_heavy(rd_graph* g, const std::vector<int64_t>& rp)
 {
     choose_chunk(g, rp);
-    g->task_nnz = task_length(g);
     std::vector<int32_t> rows, first, cb, ce;
     first.push_back(0);
     for (int64_t u = 0; u < g->n; ++u) {
@@ -216,29 +217,34 @@ static rd_status build_heavy(rd_graph* g, const std::vector<int64_t>& rp)
     }
     g->n_heavy_rows = (int64_t)rows.size();
     g->n_chunks = (int64_t)cb.size();
-    // row-stream tasks: greedy runs of consecutive light rows with at most task_nnz nonzeros
+    // row-stream tasks: greedy runs of consecutive light rows with at most `len` nonzeros
     // (a single light row longer than that stays whole); each heavy row is a task of its own
-    std::vector<int32_t> tasks;
-    tasks.push_back(0);
-    int64_t cur = 0;
-    for (int64_t u = 0; u < g->n; ++u) {
-        const int64_t d = rp[u + 1] - rp[u];
-        if (d > g->heavy_thr) {
-            if (tasks.back() != (int32_t)u) tasks.push_back((int32_t)u);
-            tasks.push_back((int32_t)(u + 1));
-            cur = 0;
-            continue;
+    auto make_tasks = [&](int len, int32_t** dev, int64_t* count) -> rd_status {
+        std::vector<int32_t> tasks;
+        tasks.push_back(0);
+        int64_t cur = 0;
+        for (int64_t u = 0; u < g->n; ++u) {
+            const int64_t d = rp[u + 1] - rp[u];
+            if (d > g->heavy_thr) {
+                if (tasks.back() != (int32_t)u) tasks.push_back((int32_t)u);
+                tasks.push_back((int32_t)(u + 1));
+                cur = 0;
+                continue;
+            }
+            if (cur > 0 && cur + d > len) {
+                tasks.push_back((int32_t)u);
+                cur = 0;
+            }
+            cur += d;
         }
-        if (cur > 0 && cur + d > g->task_nnz) {
-            tasks.push_back((int32_t)u);
-            cur = 0;
-        }
-        cur += d;
-    }
-    if (tasks.back() != (int32_t)g->n) tasks.push_back((int32_t)g->n);
-    g->ntasks = (int64_t)tasks.size() - 1;
-    RD_CUDA(cudaMalloc((void**)&g->task_row, sizeof(int32_t) * tasks.size()));
-    RD_CUDA(cudaMemcpy(g->task_row, tasks.data(), sizeof(int32_t) * tasks.size(), cudaMemcpyHostToDevice));
+        if (tasks.back() != (int32_t)g->n) tasks.push_back((int32_t)g->n);
+        *count = (int64_t)tasks.size() - 1;
+        RD_CUDA(cudaMalloc((void**)dev, sizeof(int32_t) * tasks.size()));
+        RD_CUDA(cudaMemcpy(*dev, tasks.data(), sizeof(int32_t) * tasks.size(), cudaMemcpyHostToDevice));
+        return RD_OK;
+    };
+    RD_TRY(make_tasks(task_length(g), &g->task_row, &g->ntasks));
+    RD_TRY(make_tasks(512, &g->spmv_task_row, &g->n_spmv_tasks));
     // rows by decreasing degree, stable (counting sort on the degree)
     {
         int64_t dmax = 0;
@@ -534,7 +540,7 @@ static rd_status make_plan_cfg(rd_graph* g, int64_t P, const rd_query_opts& o, c
     int64_t units = pl->cfg.kind == 1 || pl->cfg.kind == 3 ? g->ntasks : g->n;  // rows or tasks, one per row group
     int64_t per_block = rows_per_block;
     if (pl->cfg.kind == 2) {  // one task per warp
-        units = g->ntasks;
+        units = g->n_spmv_tasks;
         per_block = kWarps;
     }
     gm = std::min<int64_t>(gm, (units + per_block - 1) / per_block);
@@ -791,8 +797,9 @@ static StepArgs<T> step_args(RunCtx& c, int j, bool reduce)
     a.chunk_beg = g->chunk_beg;
     a.chunk_end = g->chunk_end;
     a.heavy_part = static_cast<T*>(c.b.heavy_part);
-    a.ntasks = g->ntasks;
-    a.task_row = g->task_row;
+    const bool spmv = c.cur.cfg.kind == 2;
+    a.ntasks = spmv ? g->n_spmv_tasks : g->ntasks;
+    a.task_row = spmv ? g->spmv_task_row : g->task_row;
     a.row_order = c.cur.cfg.kind == 0 && c.cur.cfg.order ? g->row_order : nullptr;
     // rows whose current slab fits in half of L2 are gathered with L2 priority
     a.hot_rows = g->l2_bytes > 0 ? (int64_t)(g->l2_bytes / 2) / (c.cur.cfg.tp() * (int64_t)sizeof(T)) : 0;

@@ -330,10 +330,11 @@ struct rd_graph {
     int32_t* heavy_first = nullptr;
     int32_t* chunk_beg = nullptr;
     int32_t* chunk_end = nullptr;
-    // row-stream tasks: consecutive rows with at most task_nnz nonzeros, heavy rows alone
-    int task_nnz = 512;            // (see task_length)
-    int64_t ntasks = 0;
+    // row-stream tasks: consecutive rows with at most task_length() nonzeros, heavy rows alone; the
+    // one-column SpMV has its own of at most 512
+    int64_t ntasks = 0, n_spmv_tasks = 0;
     int32_t* task_row = nullptr;
+    int32_t* spmv_task_row = nullptr;
     // rows by decreasing degree (stable: equal degrees in row order)
     int32_t* row_order = nullptr;
     // row of every stored entry (built on first use by the per-entry kernels)
