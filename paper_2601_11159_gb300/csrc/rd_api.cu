@@ -76,6 +76,19 @@ static bool is_device_ptr(const void* p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Whether kernels on `device` may use the caller's array as it is (see usable_in_place); any other
+// array is copied.
+static bool in_place(const void* p, int device, size_t align)
+{
+    if (!p) return false;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return usable_in_place(at.type, at.device, device, p, align);
+}
+
 // Ordinary host memory: not pinned (whose contents earlier work on the stream may still write).
 static bool is_pageable_ptr(const void* p)
 {
@@ -1314,8 +1327,9 @@ struct OutPtrs {
 static OutPtrs direct_outputs(const RunCtx& c, double* r_out, int32_t* iters_out, double* err_out,
                               int32_t* status_out)
 {
-    return OutPtrs{is_device_ptr(r_out) ? r_out : c.b.r, is_device_ptr(iters_out) ? iters_out : c.b.iters,
-                   is_device_ptr(err_out) ? err_out : c.b.err, is_device_ptr(status_out) ? status_out : c.b.status};
+    auto pick = [&](auto* out, auto* own) { return in_place(out, c.g->device, sizeof(*out)) ? out : own; };
+    return OutPtrs{pick(r_out, c.b.r), pick(iters_out, c.b.iters), pick(err_out, c.b.err),
+                   pick(status_out, c.b.status)};
 }
 
 // Stop rule and scalars of a run.
@@ -1533,10 +1547,17 @@ static rd_status run_forward(RunCtx& c)
 
 // Pair ids where the kernels read them: the caller's own device arrays (the call ends
 // synchronised), or a copy in stream order; of ordinary host memory in one piece through the
-// graph's pinned buffer where it fits.
-static rd_status stage_pairs(RunCtx& c, const int32_t* s, const int32_t* t)
+// graph's pinned buffer where it fits. `o`: results that a kernel writes while others still read
+// ids; ids that share memory with one of them are copied too.
+static rd_status stage_pairs(RunCtx& c, const int32_t* s, const int32_t* t, const OutPtrs* o = nullptr)
 {
-    const bool s_dev = is_device_ptr(s), t_dev = is_device_ptr(t);
+    const size_t P = (size_t)c.P;
+    auto own = [&](const int32_t* ids) {
+        if (!in_place(ids, c.g->device, sizeof(int32_t))) return false;
+        return !o || !(ranges_overlap(ids, 4 * P, o->r, 8 * P) || ranges_overlap(ids, 4 * P, o->iters, 4 * P) ||
+                       ranges_overlap(ids, 4 * P, o->err, 8 * P) || ranges_overlap(ids, 4 * P, o->status, 4 * P));
+    };
+    const bool s_dev = own(s), t_dev = own(t);
     if (c.g->h_stage && c.P <= kStagePairs && is_pageable_ptr(s) && is_pageable_ptr(t)) {
         memcpy(c.g->h_stage, s, sizeof(int32_t) * c.P);
         memcpy(c.g->h_stage + c.P, t, sizeof(int32_t) * c.P);
@@ -1862,10 +1883,10 @@ static rd_status query_batch(rd_graph* g, const int32_t* s, const int32_t* t, in
     RunCtx c;
     c.ev = ev;
     RD_TRY(prepare_run(c, g, P, o, plain, false, st, compact && !plain, lagged_polls));
-    RD_TRY(stage_pairs(c, s, t));
+    const OutPtrs op = direct_outputs(c, r_out, iters_out, err_out, status_out);
+    RD_TRY(stage_pairs(c, s, t, &op));
     // small graphs: every pair's whole recurrence in one kernel
     if ((o.flags & RD_Q_NO_ONCHIP) == 0 && onchip_smem_bytes(g->n, (int)c.pl.elem) <= 220 * 1024) {
-        const OutPtrs op = direct_outputs(c, r_out, iters_out, err_out, status_out);
         if (run_onchip(c, op)) {
             RD_TRY(collect_outputs(c, op, r_out, iters_out, err_out, status_out, call_status));
             record_stats(c);
@@ -2089,10 +2110,10 @@ static rd_status forward_and_potential(RunCtx& c, const int32_t* s, const int32_
     // z-solve and gbar; a host grad_r is staged in the output buffer (free until the end)
     const double* d_grad = nullptr;
     if (grad_r) {
-        if (is_device_ptr(grad_r)) {
+        if (in_place(grad_r, c.g->device, sizeof(double))) {
             d_grad = grad_r;
         } else {
-            RD_CUDA(cudaMemcpyAsync(c.b.r, grad_r, sizeof(double) * c.P, cudaMemcpyHostToDevice, c.st));
+            RD_CUDA(cudaMemcpyAsync(c.b.r, grad_r, sizeof(double) * c.P, cudaMemcpyDefault, c.st));
             d_grad = c.b.r;
         }
     }
@@ -2420,7 +2441,7 @@ extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* 
     RD_TRY(forward_and_potential(c, s, t, nullptr, &call));
     // phi (n x ld, q-space) -> pair-major float output
     float* stage = nullptr;
-    const bool dev_out = is_device_ptr(phi_out);
+    const bool dev_out = in_place(phi_out, g->device, sizeof(float));
     const size_t bytes = sizeof(float) * (size_t)g->n * (size_t)npairs;
     if (dev_out) {
         stage = phi_out;
@@ -2437,7 +2458,7 @@ extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* 
     launch_pair_major(st, c.pl.fp64, pa);
     ++c.launches;
     if (!dev_out) {
-        RD_CUDA(cudaMemcpyAsync(phi_out, stage, bytes, cudaMemcpyDeviceToHost, st));
+        RD_CUDA(cudaMemcpyAsync(phi_out, stage, bytes, cudaMemcpyDefault, st));
         RD_CUDA(cudaFreeAsync(stage, st));
     }
     rd_status outs = RD_OK;
@@ -2467,7 +2488,7 @@ extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, in
     rd_status call = RD_OK;
     RD_TRY(forward_and_potential(c, s, t, nullptr, &call));
     const size_t bytes = sizeof(float) * (size_t)g->nnz_in * (size_t)npairs;
-    const bool dev_out = is_device_ptr(flow_out);
+    const bool dev_out = in_place(flow_out, g->device, sizeof(float));
     float* stage = dev_out ? flow_out : nullptr;
     if (!dev_out && bytes) RD_CUDA(cudaMallocAsync((void**)&stage, bytes, st));
     if (g->keep_idx && bytes) RD_CUDA(cudaMemsetAsync(stage, 0, bytes, st));
@@ -2485,7 +2506,7 @@ extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, in
     launch_pair_major(st, c.pl.fp64, pa);
     ++c.launches;
     if (!dev_out && bytes) {
-        RD_CUDA(cudaMemcpyAsync(flow_out, stage, bytes, cudaMemcpyDeviceToHost, st));
+        RD_CUDA(cudaMemcpyAsync(flow_out, stage, bytes, cudaMemcpyDefault, st));
         RD_CUDA(cudaFreeAsync(stage, st));
     }
     rd_status outs = RD_OK;
@@ -2605,14 +2626,14 @@ extern "C" rd_status rd_triangle_weights(const rd_graph* g, float* w_out, void* 
     }
     if (g->nnz == 0) return RD_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const bool dev_out = is_device_ptr(w_out);
+    const bool dev_out = in_place(w_out, g->device, sizeof(float));
     float* stage = dev_out ? w_out : nullptr;
     int32_t* flag = nullptr;
     RD_CUDA(cudaMallocAsync((void**)&flag, sizeof(int32_t), st));
     if (!dev_out) RD_CUDA(cudaMallocAsync((void**)&stage, sizeof(float) * g->nnz, st));
     rd_status rs = triangle_weights(g->n, g->row_ptr, g->col, stage, g->sm_count, st, flag);
     if (rs == RD_OK && !dev_out)
-        RD_CUDA(cudaMemcpyAsync(w_out, stage, sizeof(float) * g->nnz, cudaMemcpyDeviceToHost, st));
+        RD_CUDA(cudaMemcpyAsync(w_out, stage, sizeof(float) * g->nnz, cudaMemcpyDefault, st));
     if (!dev_out) cudaFreeAsync(stage, st);
     cudaFreeAsync(flag, st);
     RD_CUDA(cudaStreamSynchronize(st));

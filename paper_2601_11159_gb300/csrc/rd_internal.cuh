@@ -295,6 +295,21 @@ void launch_pm_accum(cudaStream_t st, const PmArgs& a);
 
 constexpr int kStagePairs = 2048;
 
+// Whether kernels on `device` may use a caller's array at p in place: memory of that device (a peer's
+// is reached by copies alone) or managed memory, aligned to its elements as the kernels' loads
+// and stores need it (a copy takes any address).
+inline bool usable_in_place(cudaMemoryType type, int mem_device, int device, const void* p, size_t align)
+{
+    if (type != cudaMemoryTypeManaged && !(type == cudaMemoryTypeDevice && mem_device == device)) return false;
+    return reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
+inline bool ranges_overlap(const void* a, size_t na, const void* b, size_t nb)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && x < y + nb && y < x + na;
+}
+
 // --------------------------------------------------------------- graph
 struct Workspace {
     void* base = nullptr;

@@ -1068,3 +1068,59 @@ def test_short_row_graphs_match_oracle_history(rd, mode, tol, graph, pairs):
         assert m.any()
         assert rel(res.r[:5][m], ref[m]).max() < tol, (k, rel(res.r[:5][m], ref[m]).max())
         assert np.array_equal(G.query(s, t, mode=mode, k_max=k, fixed_k=True).r, res.r)
+
+
+@pytest.mark.parametrize("onchip", [True, False])
+@pytest.mark.parametrize("pairs", [5, 70])
+def test_arrays_a_copy_takes_but_a_kernel_cannot(rd, onchip, pairs):
+    """Device arrays at a byte offset (no kernel may load them) and ids whose own memory receives the
+    iteration counts give the results of ordinary arrays."""
+    import ctypes as C
+
+    import torch
+
+    g = F.grid_deleted(30, 0.05, 5)
+    s, t = F.random_pairs(g.n, pairs, 8)
+    G = rd.Graph.from_csr(g)
+    kw = dict(mode="fp64", k_max=500, rel_tol=0.0, resid_tol=1e-10, onchip=onchip, tune=False)
+    ref = G.query(s, t, **kw)
+    o = rd._opts(**kw)
+
+    def dev(x, off):
+        """A device copy of x starting `off` bytes past an aligned address."""
+        b = torch.zeros(x.nbytes + 16, dtype=torch.uint8, device="cuda")
+        b[off:off + x.nbytes] = torch.from_numpy(x.reshape(-1).view(np.uint8).copy()).cuda()
+        return b, b.data_ptr() + off
+
+    def host(b, off, like):
+        return b[off:off + like.nbytes].cpu().numpy().view(like.dtype)
+
+    s, t = s.astype(np.int32), t.astype(np.int32)
+    for oi, oo in ((1, 3), (4, 4), (2, 0)):
+        (bs, ps), (bt, pt) = dev(s, oi), dev(t, oi)
+        outs = [dev(np.zeros_like(x), oo) for x in (ref.r, ref.iters, ref.err, ref.status)]
+        torch.cuda.synchronize()
+        st = rd.lib().rd_query(G.handle, ps, pt, pairs, C.byref(o), *(p for _, p in outs), None)
+        assert st == 0
+        for (b, _), x in zip(outs, (ref.r, ref.iters, ref.err, ref.status)):
+            assert np.array_equal(host(b, oo, x), x)
+    # iteration counts into s, statuses into t
+    (bs, ps), (bt, pt) = dev(s, 0), dev(t, 0)
+    (br, pr), (be, pe) = dev(ref.r * 0, 0), dev(ref.err * 0, 0)
+    torch.cuda.synchronize()
+    assert rd.lib().rd_query(G.handle, ps, pt, pairs, C.byref(o), pr, ps, pe, pt, None) == 0
+    assert np.array_equal(host(br, 0, ref.r), ref.r) and np.array_equal(host(be, 0, ref.err), ref.err)
+    assert np.array_equal(host(bs, 0, ref.iters), ref.iters) and np.array_equal(host(bt, 0, ref.status), ref.status)
+    # potentials and gradients at a byte offset
+    kp = dict(mode="fp64", k_max=40, fixed_k=True, tune=False)
+    o = rd._opts(**kp)
+    phi, r = G.potential(s, t, **kp)
+    gr = np.linspace(-1, 1, pairs)
+    gw, _ = G.edge_grad(s, t, gr, **kp)
+    (bs, ps), (bt, pt), (bg, pg) = dev(s, 2), dev(t, 2), dev(gr, 4)
+    (bp, pp), (br, pr), (bw, pw) = dev(phi * 0, 2), dev(r * 0, 4), dev(gw * 0, 1)
+    torch.cuda.synchronize()
+    assert rd.lib().rd_potential(G.handle, ps, pt, pairs, C.byref(o), pp, pr, None) in (0, 1)
+    assert np.array_equal(host(bp, 2, phi.reshape(-1)), phi.reshape(-1)) and np.array_equal(host(br, 4, r), r)
+    assert rd.lib().rd_edge_grad(G.handle, ps, pt, pairs, pg, C.byref(o), pw, None, None) in (0, 1)
+    assert np.array_equal(host(bw, 1, gw), gw)
