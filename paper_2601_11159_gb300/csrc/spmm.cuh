@@ -307,8 +307,10 @@ __device__ __forceinline__ void gather_row(const StepArgs<T>& a, int64_t beg, in
     constexpr int CH = G * NH;
     const uint32_t row_bytes = (uint32_t)(ld * (int64_t)sizeof(T));
     const char* __restrict__ qb = reinterpret_cast<const char*>(q);
-    for (int base = (int)beg; base < (int)end; base += CH) {
-        const int cnt = (int)end - base < CH ? (int)end - base : CH;
+    // entries are counted in 32 bits without a sign: past the end of a row near 2^31 entries, `base`
+    // must not turn negative
+    for (uint32_t base = (uint32_t)beg; base < (uint32_t)end; base += CH) {
+        const int left = (int)((uint32_t)end - base), cnt = left < CH ? left : CH;
         int my_col[NH];
         float my_w[NH];
 #pragma unroll
@@ -898,11 +900,11 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
 
         for (int task = gid; task < ntasks; task += ngroups) {
             const int r0 = a.task_row[task], r1 = a.task_row[task + 1];
-            const int e_beg = (int)a.row_ptr[r0], e_end = (int)a.row_ptr[r1];
+            const uint32_t e_beg = (uint32_t)a.row_ptr[r0], e_end = (uint32_t)a.row_ptr[r1];  // (see gather_row)
             T acc[VEC], qp[VEC], qc[VEC];
 #pragma unroll
             for (int i = 0; i < VEC; ++i) acc[i] = T(0);
-            if (r1 == r0 + 1 && e_end - e_beg > a.heavy_thr) {
+            if (r1 == r0 + 1 && (int)(e_end - e_beg) > a.heavy_thr) {
                 ld_stream<T, VEC>(qp, a.qprev + (int64_t)r0 * ld + c0);
                 ld_gather<T, VEC>(qc, q + (int64_t)r0 * ld);
                 heavy_row_sum<T, VEC, 1>(a, r0, c0, 0, acc);
@@ -911,15 +913,15 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
             }
             // row window: lane gl holds row_ptr[w0 + gl + 1], 1/d and d of row w0 + gl
             int w0 = r0;
-            int my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : e_end;
+            uint32_t my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : e_end;
             T my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
-            int row_end = __shfl_sync(mask, my_end, 0, GS);
+            uint32_t row_end = __shfl_sync(mask, my_end, 0, GS);
             ld_stream<T, VEC>(qp, a.qprev + (int64_t)row * ld + c0);
             ld_gather<T, VEC>(qc, q + (int64_t)row * ld);
-            for (int base = e_beg; base < e_end; base += CH) {
-                const int cnt = e_end - base < CH ? e_end - base : CH;
+            for (uint32_t base = e_beg; base < e_end; base += CH) {
+                const int cnt = e_end - base < (uint32_t)CH ? (int)(e_end - base) : CH;
                 uint32_t my_off[NH];
                 float my_w[NH];
 #pragma unroll
@@ -959,7 +961,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                     }
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const int e = base + k0 + u;
+                        const uint32_t e = base + k0 + u;
                         if (e >= e_end) break;
                         while (e >= row_end) {  // the stream leaves `row`
                             const int wi = row - w0;
@@ -973,7 +975,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                             ++row;
                             if (row - w0 >= GS) {  // refill the row window
                                 w0 = row;
-                                my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : e_end;
+                                my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : e_end;
                                 my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                                 my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                             }
@@ -1005,7 +1007,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                 if (row >= r1) break;
                 if (row - w0 >= GS) {
                     w0 = row;
-                    my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : e_end;
+                    my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : e_end;
                     my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }
@@ -1095,7 +1097,7 @@ struct AsyncRound {
     uint32_t off[NH];
     float w[NH];
     template <class Args>
-    __device__ __forceinline__ void load(const Args& a, int base, int end, int gl, uint32_t ldv)
+    __device__ __forceinline__ void load(const Args& a, uint32_t base, uint32_t end, int gl, uint32_t ldv)
     {
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
@@ -1168,7 +1170,7 @@ __device__ __forceinline__ void acc_add_slot(float (&acc)[4], const float4& x, f
 // that end there: row epilogues) and returns the end of the segment that e is in (the first
 // nonzero of the next row); each segment is then consumed without a boundary test per nonzero.
 template <typename T, int GS, bool WEIGHTED, class Enter>
-__device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, uint32_t ldv, int eb, int ee,
+__device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, uint32_t ldv, uint32_t eb, uint32_t ee,
                                              uint32_t ring, int gl, unsigned mask, T (&acc)[kAsyncVec<T>],
                                              Enter&& enter)
 {
@@ -1183,10 +1185,10 @@ __device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, u
         if (eb + u < ee) cp_async16(ring + u * SS, reinterpret_cast<const char*>(q) + (size_t)o * 16);
         cp_async_commit();
     }
-    for (int base = eb; base < ee; base += D) {
+    for (uint32_t base = eb; base < ee; base += D) {  // (unsigned: see gather_row)
         nn.load(a, base + 2 * D, ee, gl, ldv);
-        const int cnt = ee - base < D ? ee - base : D;
-        const int refill = ee - D - base;  // slots u < refill are refilled from the next round
+        const int cnt = ee - base < (uint32_t)D ? (int)(ee - base) : D;
+        const int refill = (int)(ee - base) - D;  // slots u < refill are refilled from the next round
         auto consume = [&](int u) {
             float wv = 1.0f;
             if constexpr (WEIGHTED) wv = __shfl_sync(mask, cur.w_at(u), u % GS, GS);
@@ -1198,7 +1200,7 @@ __device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, u
             cp_async_commit();
         };
         for (int u = 0; u < cnt;) {
-            const int se = enter(base + u) - base;
+            const int se = (int)(enter(base + u) - base);
             const int stop = se < cnt ? se : cnt;
             for (; u < stop; ++u) consume(u);
         }
@@ -1232,7 +1234,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async_heavy(cons
 #pragma unroll
             for (int i = 0; i < V; ++i) acc[i] = T(0);
             async_stream<T, GS, WEIGHTED>(a, q, ldv, a.chunk_beg[ch], a.chunk_end[ch], ring, gl, mask, acc,
-                                          [](int) { return INT_MAX; });
+                                          [](uint32_t) { return (uint32_t)INT_MAX; });
 #pragma unroll
             for (int i = 0; i < V; ++i) acc_finish(acc[i]);
             st_plain<T, V>(a.heavy_part + ch * a.ld + c0, acc);
@@ -1289,17 +1291,17 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
         };
         // light rows [r0, r1): one stream of their nonzeros
         auto light_rows = [&](int r0, int r1) {
-            const int eb = (int)a.row_ptr[r0], ee = (int)a.row_ptr[r1];
+            const uint32_t eb = (uint32_t)a.row_ptr[r0], ee = (uint32_t)a.row_ptr[r1];
             T acc[V], qp[V], qc[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) acc[i] = T(0);
             // row window: lane gl holds row_ptr[w0 + gl + 1], 1/d and d of row w0 + gl
             int w0 = r0;
-            int my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : ee;
+            uint32_t my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : ee;
             T my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
-            int row_end = __shfl_sync(mask, my_end, 0, GS);
+            uint32_t row_end = __shfl_sync(mask, my_end, 0, GS);
             ld_stream<T, V>(qp, a.qprev + (int64_t)row * ld + c0);
             ld_gather<T, V>(qc, q + (int64_t)row * ld);
             // the own-row operands of the next PD rows into L2 (no registers held): short rows
@@ -1324,7 +1326,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
                 if (row >= r1) return;
                 if (row - w0 >= GS) {  // refill the row window
                     w0 = row;
-                    my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : ee;
+                    my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : ee;
                     my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }
@@ -1336,7 +1338,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
                     prefetch_l2(q + (int64_t)(row + PD) * ld);
                 }
             };
-            async_stream<T, GS, WEIGHTED>(a, q, ldv, eb, ee, ring, gl, mask, acc, [&](int e) {
+            async_stream<T, GS, WEIGHTED>(a, q, ldv, eb, ee, ring, gl, mask, acc, [&](uint32_t e) {
                 while (e >= row_end) next_row();
                 return row_end;
             });

@@ -250,3 +250,42 @@ def test_rmat24_batched_and_plain(rd):
     assert rel(res.r[idx], ref).max() < 1e-6
     plain = G.query(s[idx], t[idx], mode="fp32", k_max=200, rel_tol=1e-6, plain=True)
     assert rel(plain.r, res.r[idx]).max() < 2e-6
+
+
+def test_entry_counts_up_to_the_limit(rd):
+    """2^31 - 8 stored entries (a clique of 46,341 vertices with a path behind it, whose rows hold the
+    last entries): a kernel that steps past a row's end must not wrap round. Pairs near the path's end
+    have after three steps, without deflation, the r_k of a short path, in every kernel."""
+    import torch
+
+    k, m = 46341, 20850
+    n = k + m
+    row = torch.arange(k - 1, dtype=torch.int32, device="cuda")
+    col = (row[None, :] + (row[None, :] >= torch.arange(k, dtype=torch.int32, device="cuda")[:, None])).int().view(-1)
+    v = torch.arange(k, n, dtype=torch.int32, device="cuda")
+    path = torch.stack([v - 1, v + 1], 1).view(-1)[:-1]  # the last vertex has one neighbour
+    one = torch.tensor([k], dtype=torch.int32, device="cuda")  # the clique's last vertex meets the path
+    col = torch.cat([col, one, path])
+    deg = torch.full((n,), 2, dtype=torch.int64, device="cuda")
+    deg[:k] = k - 1
+    deg[k - 1] += 1
+    deg[-1] = 1
+    rp = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    rp[1:] = torch.cumsum(deg, 0)
+    nnz = int(rp[-1])
+    assert nnz == col.numel() == 2**31 - 8
+    G = rd.Graph(rp, col, label_components=False)
+    del col
+    short = F.path(200)
+    S = rd.Graph.from_csr(short)
+    off = np.arange(1, 18)
+    to = (off + 1) % 4
+    kw = dict(k_max=3, fixed_k=True, deflate=False, sparse_first=False, onchip=False, tune=False)
+    ref = S.query((199 - off).astype(np.int32), (199 - to).astype(np.int32), mode="fp64", **kw).r
+    s, t = (n - 1 - off).astype(np.int32), (n - 1 - to).astype(np.int32)
+    for kernel in ("group", "group_sorted", "stream", "async"):
+        for mode, tol in (("fp64", 1e-12), ("fp32", 1e-5), ("df64", 1e-11)):
+            r = G.query(s, t, mode=mode, kernel=kernel, **kw).r
+            assert rel(r, ref).max() < tol, (kernel, mode)
+    one = G.query(s[:1], t[:1], mode="fp64", kernel="tasks", **kw).r
+    assert rel(one, ref[:1]).max() < 1e-12
