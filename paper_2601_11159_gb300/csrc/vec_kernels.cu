@@ -1904,10 +1904,11 @@ static int launch_cluster_t(cudaStream_t st, const OnchipArgs& a, int C)
     constexpr size_t per = (WEIGHTED ? 4 : 0) + (COPY ? 2 : 4);
     if (base > kClusterSmemMax || a.n > 65535) return 0;
     size_t cap = (kClusterSmemMax - base) / per;
+    cap &= ~(size_t)1;  // whole words, within the limit
     if (C == 1) {
-        cap = (size_t)a.nnz <= cap ? (size_t)a.nnz : 0;
+        const size_t need = ((size_t)a.nnz + 1) & ~(size_t)1;
+        cap = need <= cap ? need : 0;
     }
-    cap = (cap + 1) & ~(size_t)1;
     L.nnz_cap = (int)cap;
     const size_t sm = base + cap * per;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemMax) != cudaSuccess)

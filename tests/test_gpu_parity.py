@@ -1124,3 +1124,17 @@ def test_arrays_a_copy_takes_but_a_kernel_cannot(rd, onchip, pairs):
     assert np.array_equal(host(bp, 2, phi.reshape(-1)), phi.reshape(-1)) and np.array_equal(host(br, 4, r), r)
     assert rd.lib().rd_edge_grad(G.handle, ps, pt, pairs, pg, C.byref(o), pw, None, None) in (0, 1)
     assert np.array_equal(host(bw, 1, gw), gw)
+
+
+@pytest.mark.parametrize("mode", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,pairs,weighted,ctas", [(129, 1, True, 4), (130, 3, True, 4), (1000, 9, True, 16),
+                                                   (1001, 30, True, 4), (1500, 20, True, 4), (4096, 19, True, 8),
+                                                   (4097, 1, True, 16), (2049, 5, False, 16)])
+def test_clusters_of_the_planned_size(rd, mode, n, pairs, weighted, ctas):
+    """The whole-recurrence kernel runs on the cluster it plans (up to 16 CTAs a pair, 64 rows a CTA, every
+    pair's cluster resident at once): the shared memory it asks for beside the vectors stays within its limit."""
+    g = F.random_connected(n, 2 * n, 3, "lognormal" if weighted else None)
+    s, t = F.random_pairs(g.n, pairs, 11)
+    G = rd.Graph.from_csr(g)
+    G.query(s, t, mode=mode, k_max=5, fixed_k=True)
+    assert G.last_stats()["onchip_ctas"] == ctas
