@@ -5,6 +5,8 @@
 // potential of Algorithm 5 and the edge-weight gradient.
 #include <math.h>
 
+#include <algorithm>
+
 #include "spmm.cuh"
 
 namespace rd {
@@ -1464,7 +1466,7 @@ __device__ __forceinline__ OnchipPair onchip_pair(const OnchipArgs& a, int p)
     return q;
 }
 
-template <typename T, bool WEIGHTED>
+template <typename T, bool WEIGHTED, bool BY4>
 __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipArgs a)
 {
     extern __shared__ __align__(16) unsigned char onchip_raw[];
@@ -1503,7 +1505,27 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
             const int64_t e0 = a.row_ptr[u], e1 = a.row_ptr[u + 1];
             if (e1 - e0 > a.heavy_thr) continue;
             T acc = T(0);
-            for (int64_t e = e0; e < e1; ++e) {
+            int64_t e = e0;
+            // BY4: four entries at a time, asked for while their lines are in the L1 (10,000 weighted FP32
+            // vertices, rows of 28, 100 pairs: 4,685 us for 30 steps one at a time, 3,845 so; 7,000
+            // unweighted FP64 vertices 3,842 and 3,386). Long rows of FP32 without weights go
+            // one at a time while the L1 holds them (10,000 vertices, rows of 56: 4,253 us, 4,630 with
+            // four; 16,000: 9,606 and 8,702)
+            for (; BY4 && e + 4 <= e1; e += 4) {
+                int v[4];
+                float we[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    v[k] = __ldg(a.col + e + k);
+                    if constexpr (WEIGHTED) we[k] = __ldg(a.w + e + k);
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if constexpr (WEIGHTED) acc += (T)we[k] * qc[v[k]];
+                    else acc += qc[v[k]];
+                }
+            }
+            for (; e < e1; ++e) {
                 if constexpr (WEIGHTED) acc += (T)__ldg(a.w + e) * qc[__ldg(a.col + e)];
                 else acc += qc[__ldg(a.col + e)];
             }
@@ -1608,12 +1630,18 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
 // 233 us before, 95 us now.
 constexpr int kClusterMax = 16;
 constexpr size_t kClusterSmemMax = 200 * 1024;  // of the 227 KB a block may have
+constexpr size_t kClusterSmemMin = 116 * 1024;  // one CTA of a cluster per SM
 
 struct ClusterLayout {
     int C;            // CTAs per pair
     int R;            // rows per CTA
+    uint32_t inv_R;   // 2^32 / R rounded up: v / R = (v inv_R) >> 32 for v < 2^16
     int nnz_cap;      // entries of the CSR a CTA can hold in shared memory
 };
+
+// What a CTA keeps beside its rows of the three vectors: a copy of q_i (see above), or none
+// (gathers); and d, 1/d and the row offsets, or, lean, not even those.
+enum ClusterForm { kGather = 0, kCopy = 1, kLean = 2 };
 
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank)
 {
@@ -1644,16 +1672,25 @@ __device__ __forceinline__ void cluster_st(uint32_t a, float v)
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// Bytes of shared memory before the entries: the copy of q_i (n elements, or none), a CTA's rows of
-// three vectors, d and 1/d, and its row offsets.
-__host__ __device__ inline size_t cluster_base_bytes(int64_t ncopy, int R, int elem)
+// Bytes of shared memory before the entries: the copy of q_i, a CTA's rows of three vectors, d and 1/d,
+// and its row offsets.
+__host__ __device__ inline size_t cluster_base_bytes(ClusterForm form, int64_t n, int R, int elem)
 {
-    return ((((size_t)ncopy + 5 * (size_t)R) * elem + (size_t)4 * (R + 1)) + 15) & ~(size_t)15;
+    if (form == kLean) return ((size_t)3 * R * elem + 15) & ~(size_t)15;
+    return ((((size_t)(form == kCopy ? n : 0) + 5 * (size_t)R) * elem + (size_t)4 * (R + 1)) + 15) & ~(size_t)15;
 }
 
-template <typename T, bool WEIGHTED, bool COPY, int NT>
-__global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, const ClusterLayout L)
+// Blocks per SM the kernel is compiled for: two of 512 threads (64 registers) where single CTAs share an
+// SM; gathers, which run in clusters alone, and FP64 vectors on small blocks get more registers (at
+// 64 they spill: 951 FP64 vertices on 16 CTAs, 30 steps, 436 for 300 us).
+template <typename T, ClusterForm FORM, int NT>
+inline constexpr int kClusterMinBlocks = FORM == kGather ? (NT == 256 ? 3 : 1)
+                                         : FORM == kCopy && NT == 256 ? (sizeof(T) == 8 ? 3 : 0) : 1024 / NT;
+
+template <typename T, bool WEIGHTED, ClusterForm FORM, int NT>
+__global__ void __launch_bounds__(NT, (kClusterMinBlocks<T, FORM, NT>)) k_lanczos_cluster(const OnchipArgs a, const ClusterLayout L)
 {
+    constexpr bool COPY = FORM == kCopy, LEAN = FORM == kLean;
     extern __shared__ __align__(16) unsigned char cl_raw[];
     __shared__ double part[3][kClusterMax];       // every CTA's sums of the step, by rank
     __shared__ double tpart[3][NT];               // per-thread partial sums of the step
@@ -1679,24 +1716,33 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
     int* s_rp = reinterpret_cast<int*>(s_deg + R);
     // the entries: weights, then the column (COPY) or the address of its element in buffer 0
     using Col = typename std::conditional<COPY, uint16_t, uint32_t>::type;
-    float* s_w = reinterpret_cast<float*>(cl_raw + cluster_base_bytes(ncopy, R, (int)E));
+    float* s_w = reinterpret_cast<float*>(cl_raw + cluster_base_bytes(FORM, n, R, (int)E));
     Col* s_col = reinterpret_cast<Col*>(WEIGHTED ? s_w + L.nnz_cap : s_w);
     if (tid < C) rbase[tid] = cluster_addr(smem_addr(full), tid);  // buf0 where there is no copy
     for (int u = tid; u < ncopy + 3 * R; u += nthr) full[u] = T(0);
     const int64_t ebase = nrow > 0 ? a.row_ptr[row0] : 0;
-    for (int u = tid; u <= nrow; u += nthr) s_rp[u] = nrow > 0 ? (int)(a.row_ptr[row0 + u] - ebase) : 0;
-    for (int u = tid; u < nrow; u += nthr) {
-        s_invd[u] = E == 8 ? (T)a.invdeg64[row0 + u] : (T)a.invdeg32[row0 + u];
-        s_deg[u] = E == 8 ? (T)a.deg64[row0 + u] : (T)a.deg32[row0 + u];
+    auto g_rp = [&](int u) { return nrow > 0 ? (int)(a.row_ptr[row0 + u] - ebase) : 0; };
+    auto g_invd = [&](int u) { return E == 8 ? (T)a.invdeg64[row0 + u] : (T)a.invdeg32[row0 + u]; };
+    auto g_deg = [&](int u) { return E == 8 ? (T)a.deg64[row0 + u] : (T)a.deg32[row0 + u]; };
+    if constexpr (!LEAN) {
+        for (int u = tid; u <= nrow; u += nthr) s_rp[u] = g_rp(u);
+        for (int u = tid; u < nrow; u += nthr) {
+            s_invd[u] = g_invd(u);
+            s_deg[u] = g_deg(u);
+        }
     }
+    auto rp = [&](int u) {
+        if constexpr (LEAN) return g_rp(u);
+        else return s_rp[u];
+    };
     if (tid == 0) stop_s = 0;
     __syncthreads();
-    const int nent = s_rp[nrow];
-    const bool cached = nent <= L.nnz_cap;
+    const int nent = rp(nrow);
+    const bool cached = !LEAN && nent <= L.nnz_cap;
     auto locate = [&](int e) -> uint32_t {
         const int v = __ldg(a.col + ebase + e);
         if constexpr (COPY) return (uint32_t)v;
-        const int r = v / R;
+        const int r = (int)__umulhi((uint32_t)v, L.inv_R);
         return rbase[r] + (uint32_t)(v - r * R) * E;
     };
     if (cached)
@@ -1734,9 +1780,9 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
         double pa = 0.0, pb = 0.0, pc = 0.0;
         bool first = true;
         auto close_row = [&](int ul, T acc) {
-            const T wv = s_invd[ul] * acc - bt * qp[ul];
+            const T wv = (LEAN ? g_invd(ul) : s_invd[ul]) * acc - bt * qp[ul];
             W[ul] = wv;
-            const T dw = s_deg[ul] * wv;
+            const T dw = (LEAN ? g_deg(ul) : s_deg[ul]) * wv;
             if (first) {  // no FP64 addition to zero
                 pa = (double)(dw * qc[ul]);
                 pb = (double)(dw * wv);
@@ -1761,27 +1807,32 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
                 else return locate(e);
             };
             auto weight = [&](int e) {
-                if constexpr (decltype(held)::value) return (T)s_w[e];
-                else return (T)__ldg(a.w + ebase + e);
+                if constexpr (decltype(held)::value) return s_w[e];
+                else return __ldg(a.w + ebase + e);
             };
             for (int ul = tid; ul < nrow; ul += nthr) {
-                int e = s_rp[ul];
-                const int e1 = s_rp[ul + 1];
+                int e = rp(ul);
+                const int e1 = rp(ul + 1);
                 if (e1 - e > a.heavy_thr) continue;
                 T acc = T(0);
                 // gathers in flight four at a time, added in order; the first is not added to zero
                 auto four = [&](bool open) {
                     uint32_t at[4];
+                    float we[4];
                     T x[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) at[u] = where(e + u);
+                    for (int u = 0; u < 4; ++u) {
+                        at[u] = where(e + u);
+                        if constexpr (WEIGHTED && !decltype(held)::value) we[u] = weight(e + u);
+                    }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) x[u] = fetch(at[u]);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         if constexpr (WEIGHTED) {
-                            if (open && u == 0) acc = weight(e) * x[0];
-                            else acc += weight(e + u) * x[u];
+                            if constexpr (decltype(held)::value) we[u] = weight(e + u);
+                            if (open && u == 0) acc = (T)we[0] * x[0];
+                            else acc += (T)we[u] * x[u];
                         } else {
                             if (open && u == 0) acc = x[0];
                             else acc += x[u];
@@ -1793,7 +1844,7 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
                 while (e + 4 <= e1) four(false);
                 for (; e < e1; ++e) {
                     const T x = fetch(where(e));
-                    if constexpr (WEIGHTED) acc += weight(e) * x;
+                    if constexpr (WEIGHTED) acc += (T)weight(e) * x;
                     else acc += x;
                 }
                 close_row(ul, acc);
@@ -1802,9 +1853,10 @@ __global__ void __launch_bounds__(NT) k_lanczos_cluster(const OnchipArgs a, cons
                 const int ul = a.heavy_rows[h] - row0;
                 if (ul < 0 || ul >= nrow) continue;
                 T acc = T(0);
-                for (int e = s_rp[ul] + lane; e < s_rp[ul + 1]; e += 32) {
+                const int e1 = rp(ul + 1);
+                for (int e = rp(ul) + lane; e < e1; e += 32) {
                     const T x = fetch(where(e));
-                    if constexpr (WEIGHTED) acc += weight(e) * x;
+                    if constexpr (WEIGHTED) acc += (T)weight(e) * x;
                     else acc += x;
                 }
 #pragma unroll
@@ -1889,31 +1941,84 @@ static int cluster_size(const OnchipArgs& a)
 // Rows per CTA, even so that what follows them stays 8-byte aligned.
 static int cluster_rows(const OnchipArgs& a, int C) { return (int)(((a.n + C - 1) / C + 1) & ~1ll); }
 
-// Launches the kernel with C CTAs per pair; 0 if it does not fit. For C > 1 the entries get all the
-// shared memory that is left (one CTA of a cluster then occupies an SM: the FP64 rate per SM is
-// what a cluster multiplies); for C = 1 what the graph needs, or none where it does not fit, so
-// that several pairs share an SM.
-template <typename T, bool WEIGHTED, bool COPY, int NT>
+// Threads per CTA: a row each up to 512 rows: the products wait on shared-memory latency, and more
+// warps hide it (1,000 vertices on 2 CTAs, FP32: 10,300 cycles a step with two rows a thread).
+static int cluster_threads(const OnchipArgs& a, int C) { return cluster_rows(a, C) <= 256 ? 256 : 512; }
+
+static size_t cluster_entry_bytes(const OnchipArgs& a, ClusterForm form)
+{
+    return (a.weighted ? 4 : 0) + (form == kCopy ? 2 : 4);
+}
+
+// Entries a CTA of this form has room for (whole words, within the limit); -1 if its rows do not fit.
+static int64_t cluster_room(const OnchipArgs& a, int C, ClusterForm form)
+{
+    const size_t base = cluster_base_bytes(form, a.n, cluster_rows(a, C), a.elem_size);
+    if (base > kClusterSmemMax || a.n > 65535) return -1;
+    return form == kLean ? 0 : (int64_t)((kClusterSmemMax - base) / cluster_entry_bytes(a, form)) & ~(int64_t)1;
+}
+
+// KB of an SM's 256 that shared memory takes when `bytes` of it are in use; the L1 has the rest.
+static int smem_split(size_t bytes)
+{
+    for (int kb : {8, 16, 32, 64, 100, 132, 164, 196})
+        if (bytes <= (size_t)kb * 1024) return kb;
+    return 228;
+}
+
+// How far over the L1 the lines are that the threads of an SM read entries from (12 KB of it left to
+// the rest): a thread walks its row in order, so until it leaves a 128-byte line the line has to
+// stay. `blocks` of `smem` bytes and `threads` threads are resident.
+static double l1_pressure(const OnchipArgs& a, int blocks, int threads, size_t smem)
+{
+    const double row = a.n > 0 ? 4.0 * (double)a.nnz / (double)a.n : 0.0;
+    return blocks * threads * std::min(row, 128.0) * (a.weighted ? 2 : 1) / (1024.0 * (244 - smem_split(blocks * smem)));
+}
+
+// Bytes of an SM that one block takes.
+static size_t cluster_footprint(const OnchipArgs& a, int C, size_t dynamic)
+{
+    return dynamic + 24 * (size_t)cluster_threads(a, C) + 512 + 1024;  // tpart, the rest, the system's
+}
+
+// Blocks of `smem` bytes that share an SM, at most `most` (by their registers).
+static int resident_blocks(const OnchipArgs& a, size_t smem, int64_t most)
+{
+    const int64_t want = ((int64_t)a.npairs + a.sm_count - 1) / a.sm_count, fit = (int64_t)(228 * 1024 / smem);
+    return (int)std::max<int64_t>(1, std::min({want, fit, most}));
+}
+
+// Launches the kernel with C CTAs per pair; 0 if it does not fit. Where the entries fit on average, for
+// C > 1 they get all the shared memory that is left (one CTA of a cluster then occupies an SM: the
+// FP64 rate per SM is what a cluster multiplies), and for C = 1 what the graph needs, so that several
+// pairs share an SM. Where they do not, they are read from global memory and the space is left to
+// the L1 cache, but for what keeps a cluster's CTAs on SMs of their own: 64 pairs, weighted, rows
+// of 28 entries, FP32, 4,000 vertices: 2,351 us with all of it reserved, 934 now (8,000: 4,469 and 2,045).
+template <typename T, bool WEIGHTED, ClusterForm FORM, int NT>
 static int launch_cluster_t(cudaStream_t st, const OnchipArgs& a, int C)
 {
-    auto k = k_lanczos_cluster<T, WEIGHTED, COPY, NT>;
+    auto k = k_lanczos_cluster<T, WEIGHTED, FORM, NT>;
     ClusterLayout L;
     L.C = C;
     L.R = cluster_rows(a, C);
-    const size_t base = cluster_base_bytes(COPY ? a.n : 0, L.R, (int)sizeof(T));
-    constexpr size_t per = (WEIGHTED ? 4 : 0) + (COPY ? 2 : 4);
-    if (base > kClusterSmemMax || a.n > 65535) return 0;
-    size_t cap = (kClusterSmemMax - base) / per;
-    cap &= ~(size_t)1;  // whole words, within the limit
-    if (C == 1) {
-        const size_t need = ((size_t)a.nnz + 1) & ~(size_t)1;
-        cap = need <= cap ? need : 0;
-    }
-    L.nnz_cap = (int)cap;
-    const size_t sm = base + cap * per;
+    L.inv_R = (uint32_t)(((1ull << 32) + L.R - 1) / L.R);
+    const int64_t room = cluster_room(a, C, FORM);
+    if (room < 0) return 0;
+    const bool held = a.nnz <= room * C;
+    L.nnz_cap = !held ? 0 : (int)(C > 1 ? room : (a.nnz + 1) & ~(int64_t)1);
+    size_t sm = cluster_base_bytes(FORM, a.n, L.R, (int)sizeof(T)) + L.nnz_cap * cluster_entry_bytes(a, FORM);
+    if (C > 1) sm = std::max(sm, kClusterSmemMin);
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemMax) != cudaSuccess)
         return 0;
     if (C > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
+    // no more of the SM than the resident blocks take (100 FP64 pairs of 4,000 weighted vertices, rows of
+    // 56 entries, lean: 10,108 us with the default split, 5,454 so)
+    int carve = cudaSharedmemCarveoutDefault;
+    if (!held) {
+        const size_t foot = cluster_footprint(a, C, sm);
+        carve = 100 * smem_split((C > 1 ? 1 : resident_blocks(a, foot, 2)) * foot) / 228;
+    }
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.npairs * C), 1, 1);
     cfg.blockDim = dim3(NT, 1, 1);
@@ -1938,42 +2043,87 @@ static int launch_cluster_t(cudaStream_t st, const OnchipArgs& a, int C)
     return C;
 }
 
-template <typename T, bool WEIGHTED, bool COPY>
+template <typename T, bool WEIGHTED, ClusterForm FORM>
 static int launch_cluster_n(cudaStream_t st, const OnchipArgs& a, int C)
 {
-    // a row per thread up to 512 rows: the products wait on shared-memory latency, and more warps
-    // hide it (1,000 vertices on 2 CTAs, FP32: 10,300 cycles a step with two rows a thread)
-    return cluster_rows(a, C) <= 256 ? launch_cluster_t<T, WEIGHTED, COPY, 256>(st, a, C)
-                                     : launch_cluster_t<T, WEIGHTED, COPY, 512>(st, a, C);
+    return cluster_threads(a, C) == 256 ? launch_cluster_t<T, WEIGHTED, FORM, 256>(st, a, C)
+                                        : launch_cluster_t<T, WEIGHTED, FORM, 512>(st, a, C);
 }
 
-template <typename T>
-static int launch_cluster_e(cudaStream_t st, const OnchipArgs& a, int C, bool copy)
+template <typename T, bool WEIGHTED>
+static int launch_cluster_f(cudaStream_t st, const OnchipArgs& a, int C, ClusterForm form)
 {
-    if (copy) return a.weighted ? launch_cluster_n<T, true, true>(st, a, C) : launch_cluster_n<T, false, true>(st, a, C);
-    return a.weighted ? launch_cluster_n<T, true, false>(st, a, C) : launch_cluster_n<T, false, false>(st, a, C);
+    return form == kCopy ? launch_cluster_n<T, WEIGHTED, kCopy>(st, a, C)
+           : form == kGather ? launch_cluster_n<T, WEIGHTED, kGather>(st, a, C)
+                             : launch_cluster_n<T, WEIGHTED, kLean>(st, a, C);
+}
+
+static int launch_cluster(cudaStream_t st, const OnchipArgs& a, int C, ClusterForm form)
+{
+    if (a.elem_size == 8)
+        return a.weighted ? launch_cluster_f<double, true>(st, a, C, form) : launch_cluster_f<double, false>(st, a, C, form);
+    return a.weighted ? launch_cluster_f<float, true>(st, a, C, form) : launch_cluster_f<float, false>(st, a, C, form);
+}
+
+// The form for C CTAs per pair, or kOneBlock: k_lanczos_onchip on one CTA. Where the entries fit, copies
+// where a pair's CTAs write fewer elements than they would gather (see above). Where they do not, an
+// SM's L1 decides. 30 fixed steps, us, FP32 (unweighted | weighted), pressures in brackets:
+//  - one CTA, 100 pairs, copies against kOneBlock: 4,000 vertices, rows of 56: 1,729 | 3,072 (0.6 | 1.2)
+//    and 1,875 | 3,315; 7,000 vertices, rows of 14: 1,188 | 1,557 (1.8 | 3.6) and 969 | 1,266, of 28: 2,528 |
+//    7,246 and 1,585 | 2,715; 300 pairs, two on an SM, 2,500 vertices, rows of 28: 1,047 | 1,957 (1.4 |
+//    2.9) and 1,571 | 2,151, of 56: 1,919 | 4,349 (1.6 | 3.3) and 2,523 | 4,060;
+//  - kOneBlock against lean: 100 pairs, 13,000 weighted vertices, rows of 28: 5,170 (2.9) and 5,786; 8,400
+//    FP64 vertices, rows of 56: 9,575 (8.2) and 6,713; on two CTAs, 64 pairs, 18,000 vertices, rows of 14:
+//    2,165 | 4,877 (3.6 | 7.2) and 3,036 | 3,120. FP64 steps are bound by the SM's FP64 unit, of which two
+//    CTAs always have twice as much;
+//  - two CTAs, 64 pairs, copies against lean: 12,000 vertices, rows of 28: 2,381 | 4,144 (3.6 | 7.2) and
+//    3,957 | 4,113, of 56: 6,136 | 10,746 (4.1 | 8.2) and 7,396 | 7,790.
+enum { kOneBlock = -1, kNoForm = -2 };
+static int cluster_form(const OnchipArgs& a, int C)
+{
+    const ClusterForm wish = a.n * (C - 1) <= a.nnz ? kCopy : kGather;
+    const int64_t room = cluster_room(a, C, wish);
+    if (room >= 0 && a.nnz <= room * C) return wish;
+    int resident = 1;
+    auto pressure = [&](ClusterForm f) {
+        if (cluster_room(a, C, f) < 0) return 1e30;
+        size_t sm = cluster_base_bytes(f, a.n, cluster_rows(a, C), a.elem_size);
+        if (C > 1) sm = std::max(sm, kClusterSmemMin);
+        const size_t foot = cluster_footprint(a, C, sm);
+        resident = C > 1 ? 1 : resident_blocks(a, foot, 2);
+        return l1_pressure(a, resident, cluster_threads(a, C), foot);
+    };
+    const double lean = pressure(kLean), copy = pressure(kCopy);
+    if (copy <= (C > 1 ? 6.0 : (resident > 1 ? 3.1 : (a.elem_size == 8 ? 2.0 : 1.4)))) return kCopy;
+    const size_t one = onchip_smem_bytes(a.n, a.elem_size) + 2048;
+    const double block = one > 222 * 1024 ? 1e30 : l1_pressure(a, 1, kOnchipThreads, one);
+    if (block <= (C > 1 && a.weighted ? 2.0 : 4.0) && (C == 1 || a.elem_size == 4)) return kOneBlock;
+    if (lean < block || (C > 1 && lean < 1e30)) return kLean;
+    return block < 1e30 ? kOneBlock : kNoForm;
 }
 
 int launch_onchip(cudaStream_t st, const OnchipArgs& a)
 {
     for (int C = cluster_size(a); C >= 1; C >>= 1) {
-        // copies of q_i against gathers from the other CTAs (see the kernel)
-        const bool copy = a.n * (C - 1) <= a.nnz;
-        const int used = a.elem_size == 8 ? launch_cluster_e<double>(st, a, C, copy)
-                                          : launch_cluster_e<float>(st, a, C, copy);
+        const int form = cluster_form(a, C);
+        if (form == kOneBlock) break;
+        const int used = form == kNoForm ? 0 : launch_cluster(st, a, C, (ClusterForm)form);
         if (used) return used;
     }
-    // graphs whose three vectors fit in one SM but not the degrees beside them
+    // kOneBlock, and graphs whose three vectors fit in one SM but nothing beside them
     const size_t sm = onchip_smem_bytes(a.n, a.elem_size);
     if (sm > 220 * 1024) return 0;
+    auto launch = [&](auto k) {
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k<<<a.npairs, kOnchipThreads, sm, st>>>(a);
+    };
     if (a.elem_size == 8) {
-        auto k = a.weighted ? k_lanczos_onchip<double, true> : k_lanczos_onchip<double, false>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k<<<a.npairs, kOnchipThreads, sm, st>>>(a);
+        launch(a.weighted ? k_lanczos_onchip<double, true, true> : k_lanczos_onchip<double, false, true>);
+    } else if (a.weighted) {
+        launch(k_lanczos_onchip<float, true, true>);
     } else {
-        auto k = a.weighted ? k_lanczos_onchip<float, true> : k_lanczos_onchip<float, false>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k<<<a.npairs, kOnchipThreads, sm, st>>>(a);
+        const bool by4 = a.nnz <= 40 * a.n || l1_pressure(a, 1, kOnchipThreads, sm + 2048) > 2.0;
+        launch(by4 ? k_lanczos_onchip<float, false, true> : k_lanczos_onchip<float, false, false>);
     }
     return 1;
 }

@@ -1138,3 +1138,23 @@ def test_clusters_of_the_planned_size(rd, mode, n, pairs, weighted, ctas):
     G = rd.Graph.from_csr(g)
     G.query(s, t, mode=mode, k_max=5, fixed_k=True)
     assert G.last_stats()["onchip_ctas"] == ctas
+
+
+@pytest.mark.parametrize("mode,n,deg,pairs,weighted,ctas", [
+    ("fp64", 7500, 6, 64, False, 2), ("fp64", 8001, 28, 70, True, 2),   # copies of q_i do not fit on two CTAs
+    ("fp32", 14001, 28, 64, True, 2), ("fp32", 18001, 28, 64, False, 2),
+    ("fp32", 6000, 56, 64, True, 2), ("fp32", 9001, 56, 30, True, 4),   # copies fit, the entries do not
+    ("fp64", 8400, 56, 80, False, 1), ("fp32", 2500, 28, 300, True, 1), ("fp32", 7000, 28, 80, True, 1)])
+def test_small_graphs_whose_entries_do_not_fit_on_chip(rd, mode, n, deg, pairs, weighted, ctas):
+    """The whole-recurrence kernels that read the entries from global memory -- with copies of q_i, without, on
+    one CTA and on clusters of the planned size -- give what the step kernels give after 30 steps."""
+    g = F.random_connected(n, n * (deg // 2 - 1), 3, "lognormal" if weighted else None)
+    s, t = F.random_pairs(g.n, pairs, 11)
+    G = rd.Graph.from_csr(g)
+    kw = dict(mode=mode, k_max=30, fixed_k=True)
+    res = G.query(s, t, **kw)
+    assert G.last_stats()["onchip_ctas"] == ctas
+    ref = G.query(s, t, onchip=False, tune=False, **kw)
+    assert G.last_stats()["onchip_ctas"] == 0
+    assert rel(res.r, ref.r).max() < (FP64_TOL if mode == "fp64" else FP32_TOL)
+    assert np.array_equal(G.query(s, t, **kw).r, res.r)
