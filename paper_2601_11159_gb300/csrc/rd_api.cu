@@ -1353,7 +1353,8 @@ static FinArgs fin_args(const RunCtx& c, bool fp64, bool df)
 }
 
 // The whole-recurrence kernel, which takes the ids and writes the results itself: one memset, one
-// kernel and one read of the flags are the whole call. False if no configuration fits.
+// kernel (two for a large batch) and one read of the flags are the whole call. False if no
+// configuration fits.
 static bool run_onchip(RunCtx& c, const OutPtrs& o)
 {
     const rd_graph* g = c.g;
@@ -1385,6 +1386,7 @@ static bool run_onchip(RunCtx& c, const OutPtrs& o)
     oa.status_out = o.status;
     oa.summary = c.b.summary;
     cudaMemsetAsync(c.b.summary, 0, kHostFlags * sizeof(int32_t), c.st);
+    if (launch_check_ids(c.st, oa)) ++c.launches;
     c.onchip_ctas = launch_onchip(c.st, oa);
     if (c.onchip_ctas == 0) return false;
     ++c.launches;

@@ -255,6 +255,8 @@ size_t onchip_smem_bytes(int64_t n, int elem_size);
 // Launches the whole-recurrence kernel; returns the CTAs per pair used (1: one CTA per pair,
 // 2..16: a thread-block cluster per pair), or 0 if the graph does not fit.
 int launch_onchip(cudaStream_t st, const OnchipArgs& a);
+// The kernel that looks a large batch's ids over before launch_onchip; false if the batch needs none.
+bool launch_check_ids(cudaStream_t st, const OnchipArgs& a);
 
 // Column compaction: keep the slots whose pair is still active, in slot order.
 struct CompactArgs {

@@ -1158,3 +1158,43 @@ def test_small_graphs_whose_entries_do_not_fit_on_chip(rd, mode, n, deg, pairs, 
     assert G.last_stats()["onchip_ctas"] == 0
     assert rel(res.r, ref.r).max() < (FP64_TOL if mode == "fp64" else FP32_TOL)
     assert np.array_equal(G.query(s, t, **kw).r, res.r)
+
+
+def test_large_batches_on_a_small_graph(rd):
+    """Whole-recurrence batches on both sides of the line above which one launch checks the ids: every pair
+    has the answer it has in a small batch, a bad id at any place is refused with the results left as they
+    were, and 16 times the pairs take nowhere near 256 times as long."""
+    import time
+
+    import torch
+
+    g = F.grid(5)
+    G = rd.Graph.from_csr(g)
+    kw = dict(mode="fp64", k_max=4, fixed_k=True)
+    s0, t0 = (x.astype(np.int32) for x in np.divmod(np.arange(g.n * g.n), g.n))
+    ref = np.concatenate([G.query(s0[i:i + 125], t0[i:i + 125], **kw).r for i in range(0, s0.size, 125)])
+    seconds = {}
+    for P in (1 << 14, (1 << 14) + 1, 1 << 16, 1 << 20):
+        i = np.arange(P) % s0.size
+        s, t = torch.from_numpy(s0[i]).cuda(), torch.from_numpy(t0[i]).cuda()
+        best = np.inf
+        for _ in range(3):
+            torch.cuda.synchronize()
+            at = time.perf_counter()
+            r = G.query(s, t, **kw).r
+            best = min(best, time.perf_counter() - at)
+        seconds[P] = best
+        assert G.last_stats()["onchip_ctas"] == 1
+        assert np.array_equal(r.cpu().numpy(), ref[i])
+    assert seconds[1 << 20] < 48 * seconds[1 << 16], seconds
+    import ctypes as C
+
+    o = rd._opts(**kw)
+    for P, at in ((512, 511), (1 << 14, 0), ((1 << 14) + 1, 1 << 14), (70001, 4321)):
+        i = np.arange(P) % s0.size
+        s, t = torch.from_numpy(s0[i]).cuda(), torch.from_numpy(t0[i]).cuda()
+        t[at] = g.n if at % 2 else -1
+        r = torch.full((P,), 7.0, dtype=torch.float64, device="cuda")
+        assert rd.lib().rd_query(G.handle, s.data_ptr(), t.data_ptr(), P, C.byref(o), r.data_ptr(), None, None,
+                                 None, rd._stream_ptr()) == rd.RD_ERR_INVALID_ARG
+        assert bool((r == 7.0).all())
