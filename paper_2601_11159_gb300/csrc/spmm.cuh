@@ -434,36 +434,22 @@ __device__ __forceinline__ void row_epilogue(const StepArgs<T>& a, int64_t row, 
     }
 }
 
-// The same in double-float on the two columns of a lane slot, with the products left unnormalised where
-// they go straight into a sum or another product: 64 packed FP32 operations for both columns. 1024^2 road
-// grid, 64 columns, 200 steps with k_spmm_async: 165.3 ms with every product normalised, 161.7
-// without, 159.8 packed (343 instructions a row and warp; the kernel then issues in 60% of its
-// cycles, against 73% before, and waits for its operands).
+// The same in double-float on the two columns of a lane slot, in packed FP32 operations with the scalar
+// ones' roundings. (Lazy-walk steps are never double-float: the Power Method runs that mode in FP64.)
+// 1024^2 road grid, 64 columns, 200 steps with k_spmm_async: 153.6 ms, 150.3 with products left
+// unnormalised (see df_row); in scalar operations, with tasks of 512 entries, 165.3 and 161.7.
 __device__ __forceinline__ void row_epilogue_x2(const StepArgs<df64>& a, int64_t row, int64_t c0, df64 invd, df64 du,
                                                 const df64 (&acc)[2], const df64 (&bt)[2], const df64 (&qp)[2],
                                                 const df64 (&qc)[2], Acc<df64> (&sA)[2], Acc<df64> (&sB)[2],
                                                 Acc<df64> (&sC)[2])
 {
     df64 wv[2];
-    df64x2 w;
-    if (a.lazy_walk) {
-#pragma unroll
-        for (int i = 0; i < 2; ++i) wv[i] = df64(0.5) * (invd * acc[i]) + df64(0.5) * qc[i];
-        w = df_pack(wv[0], wv[1]);
-    } else {
-        const df64x2 b = df_pack(bt[0], bt[1]);
-        const df64x2n x = df_prod(make_float2(invd.hi, invd.hi), df_pack(-invd, -invd), df_pack(acc[0], acc[1]));
-        w = x + df_prod(make_float2(-b.hi.x, -b.hi.y), b, df_pack(qp[0], qp[1]));
-        df_unpack(w, wv[0], wv[1]);
-    }
+    const df64x2 w = df_row(invd, df_pack(acc[0], acc[1]), df_pack(bt[0], bt[1]), df_pack(qp[0], qp[1]));
+    df_unpack(w, wv[0], wv[1]);
     st_stream<df64, 2>(a.w_out + row * a.ld + c0, wv);
     if (a.do_reduce) {
-        const df64x2 nd = df_pack(-du, -du);
-        const df64x2n dw = df_prod(make_float2(du.hi, du.hi), nd, w);
-        const df64x2 ndw{__fmul2_rn(nd.hi, w.hi), dw.nlo};
-        const df64x2 sa = df_pack(sA[0].s, sA[1].s) + df_prod(dw.hi, ndw, df_pack(qc[0], qc[1]));
-        const df64x2 sb = df_pack(sB[0].s, sB[1].s) + df_prod(dw.hi, ndw, w);
-        const df64x2 sc = df_pack(sC[0].s, sC[1].s) + dw;
+        df64x2 sa = df_pack(sA[0].s, sA[1].s), sb = df_pack(sB[0].s, sB[1].s), sc = df_pack(sC[0].s, sC[1].s);
+        df_row_sums(du, w, df_pack(qc[0], qc[1]), sa, sb, sc);
         df_unpack(sa, sA[0].s, sA[1].s);
         df_unpack(sb, sB[0].s, sB[1].s);
         df_unpack(sc, sC[0].s, sC[1].s);
