@@ -7,6 +7,7 @@
 
 #include <algorithm>
 
+#include "estimate.cuh"
 #include "spmm.cuh"
 
 namespace rd {
@@ -168,9 +169,7 @@ __device__ __forceinline__ StepCoef step_coef(const FinArgs& a, double A, double
 // stop tests; returns true when the pair stops. The state in `s` is advanced exactly as
 // pair_update advances the stored state. Divisions are what this chain is made of, so
 // 1/delta_{i-1} is kept from the previous step, 1/sum(d) is passed in, 1/delta_i serves every
-// quotient by it, the largest increment ratio rho = num/den is found by cross-multiplication
-// (increments are positive), and the estimate incr rho / (1 - rho)^2 / S is one quotient,
-// incr num den / ((den - num)^2 S).
+// quotient by it, and the estimate is one quotient (tail_estimate).
 __device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int j, const StepCoef& k, PairStepOut& o)
 {
     const double alpha = k.alpha;
@@ -220,22 +219,8 @@ __device__ __forceinline__ bool pair_core(const FinArgs& a, PairScalars& s, int 
     double est = 0.0;
     if (!breakdown && (use_est || stop || j + 1 >= a.k_max)) {
         if (!a.est_delayed && j + 1 >= kRing) {
-            // the largest num/den over the last kRing-1 pairs of consecutive increments
-            double bn = s.ring(j % kRing), bd = s.ring((j - 1) % kRing);
-            for (int q = 2; q < kRing; ++q) {
-                const double num = s.ring((j - q + 1) % kRing);
-                const double den = s.ring((j - q) % kRing);
-                if (num * bd > bn * den) {
-                    bn = num;
-                    bd = den;
-                }
-            }
-            if (bn + bn <= bd) {  // rho at its floor 1/2
-                bn = 1.0;
-                bd = 2.0;
-            }
-            const double gap = bd - bn;
-            est = bn < bd ? incr * bn * bd / (gap * gap * S) : INFINITY;
+            est = tail_estimate(s.ring(j % kRing), s.ring((j - 1) % kRing), s.ring((j - 2) % kRing),
+                                s.ring((j - 3) % kRing), S);
         } else {
             double tail = 0.0;
             const int nr = j + 1 < kRing ? j + 1 : kRing;

@@ -1198,3 +1198,16 @@ def test_large_batches_on_a_small_graph(rd):
         assert rd.lib().rd_query(G.handle, s.data_ptr(), t.data_ptr(), P, C.byref(o), r.data_ptr(), None, None,
                                  None, rd._stream_ptr()) == rd.RD_ERR_INVALID_ARG
         assert bool((r == 7.0).all())
+
+
+@pytest.mark.parametrize("onchip", [True, False])
+def test_error_estimate_of_long_fixed_runs(rd, onchip):
+    """Runs of fixed length that go on long after they have converged: the increments fall through the
+    whole range of FP64, and the estimate with them: a number below the run's rounding, or infinite where an
+    increment rose (as rho >= 1 gives by definition), never NaN."""
+    g = F.grid(16)
+    s, t = F.random_pairs(g.n, 9, 8)
+    G = rd.Graph.from_csr(g)
+    for k in range(400, 2600, 75):
+        res = G.query(s, t, mode="fp64", k_max=k, fixed_k=True, onchip=onchip, tune=False)
+        assert np.all(res.status == 0) and np.all((res.err == np.inf) | (res.err < 1e-12)), (k, res.err)

@@ -67,3 +67,38 @@ int main()
 }
 """)
     assert out == "0"
+
+
+def test_error_estimate_of_increments_of_any_size(tmp_path):
+    """The geometric tail estimate against its definition in long double, for increments that fall (or
+    rise) at any ratio from their first size to the last denormal: no NaN, and the same value."""
+    out = host_cc.run(tmp_path, r"""
+int main()
+{
+    std::mt19937_64 g(5);
+    double worst = 0.0;
+    long n = 0, bad = 0;
+    for (double ratio : {1e-3, 0.3, 0.499, 0.5, 0.501, 0.6, 0.9, 0.99, 0.9999, 1.0, 1.2})
+        for (int k = 0; k < 4000; ++k) {
+            // a stretch that starts at 2^-1074 .. 1, its ratios a little uneven
+            double i[4];
+            i[3] = std::ldexp(1.0 + (double)(g() >> 12) * 0x1p-52, -(int)(g() % 1075));
+            for (int q = 2; q >= 0; --q) i[q] = i[q + 1] * ratio * (1.0 + 1e-3 * ((double)(g() % 2001) - 1000.0) * 1e-3);
+            const double S = 0.5 + (double)(g() % 1000);
+            const double est = rd::tail_estimate(i[0], i[1], i[2], i[3], S);
+            long double rho = 0.5L;
+            for (int q = 0; q < 3; ++q)
+                if (i[q + 1] != 0.0) rho = std::fmax(rho, (long double)i[q] / (long double)i[q + 1]);
+                else if (i[q] != 0.0) rho = INFINITY;
+            const long double ref = rho < 1.0L ? (long double)i[0] * rho / ((1.0L - rho) * (1.0L - rho)) / S : INFINITY;
+            ++n;
+            if (std::isnan(est) || std::isinf(est) != std::isinf((double)ref)) { ++bad; continue; }
+            if (std::isinf(est)) continue;
+            // the last digits of a denormal estimate are its spacing's; (1 - rho)^-2 magnifies rounding
+            const long double tol = 0x1p-1073L + std::fabs(ref) * 16 * 0x1p-52L / (rho < 1.0L ? 1.0L - rho : 1.0L);
+            worst = std::fmax(worst, (double)(std::fabs((long double)est - ref) / tol));
+        }
+    printf("%ld %ld %d", n, bad, worst <= 1.0);
+}
+""", headers=("estimate.cuh",))
+    assert out == "44000 0 1"
