@@ -292,8 +292,10 @@ __host__ __device__ inline int fin_cols_per_block(int64_t ld)
 // rd_query's host polls do, so that both pack the columns at the same step; when one is due, the
 // step's normalise pass is left to the host, which runs it fused with the packing. To stop, record
 // j (or j + 1 when nothing is left to do), the count the test read, the count entering the next
-// step and which of the two it is in saved[0..3], and park the step index at the sentinel
-// k_max + 1, whose active count is always 0, so that the remaining kernels of the body return.
+// step and which of the two it is in saved[0..3], and park both indices at the sentinel
+// k_max + 1, whose active count is always 0, so that the remaining kernels of the body return: the
+// normalise pass of this step too, whose vector nobody reads, and with it that of the body's other
+// orientation (64 FP32 columns of a 1500^2 grid: 0.27 ms each).
 template <typename T>
 __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
 {
@@ -400,7 +402,7 @@ __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
     const bool compact_due = a.loop_compact && jn >= a.loop_lag + 1 && jn >= *a.loop_cfrom && a.ld > 16 &&
                              (int64_t)act_lag * 2 <= a.ld;
     const bool pack = more && compact_due;
-    *a.loop_norm = pack ? a.k_max + 1 : j;
+    *a.loop_norm = pack || !more ? a.k_max + 1 : j;
     *a.loop_step = more && !pack ? jn : a.k_max + 1;
     if (pack || !more) {
         a.loop_saved[0] = pack ? j : jn;

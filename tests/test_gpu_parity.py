@@ -1211,3 +1211,26 @@ def test_error_estimate_of_long_fixed_runs(rd, onchip):
     for k in range(400, 2600, 75):
         res = G.query(s, t, mode="fp64", k_max=k, fixed_k=True, onchip=onchip, tune=False)
         assert np.all(res.status == 0) and np.all((res.err == np.inf) | (res.err < 1e-12)), (k, res.err)
+
+
+def test_device_loop_makes_no_pass_after_the_last_step(rd):
+    """A fixed-length query ends in either orientation of the device loop's body, and neither runs a normalise
+    pass more than the other: a step costs the same from 2 to 3 steps as from 3 to 4 (with a pass or
+    two after the last step they differed by two passes, 1.7 to 1)."""
+    import time
+
+    import torch
+
+    G = rd.Graph.from_csr(F.grid(1500), label_components=False)
+    s, t = (torch.from_numpy(x.astype(np.int32)).cuda() for x in F.random_pairs(G.n, 64, 8))
+    best = {}
+    for k in (2, 3, 4):
+        ts = []
+        for _ in range(25):
+            torch.cuda.synchronize()
+            at = time.perf_counter()
+            G.query(s, t, mode="fp32", k_max=k, fixed_k=True, tune=False)
+            ts.append(time.perf_counter() - at)
+        best[k] = min(ts[5:])
+        assert G.last_stats()["device_loop"] == 1
+    assert abs((best[4] - best[3]) - (best[3] - best[2])) < 0.25 * (best[4] - best[2]) / 2, best
