@@ -17,7 +17,7 @@ struct CheckFlags {
     int32_t asymmetric;
     uint32_t ticket;              // k_degrees: blocks done
     unsigned long long self_loops;
-    double sumdeg;
+    double sumdeg, inv_sumdeg;    // sum of the degrees and its reciprocal (0 if there is none)
 };
 
 static_assert(sizeof(CheckFlags) <= kCheckFlagsBytes, "CheckFlags has its own scratch");
@@ -218,7 +218,10 @@ __global__ void __launch_bounds__(256) k_degrees(const DegArgs a)
         if (tid < s) sd[tid] += sd[tid + s];
         __syncthreads();
     }
-    if (tid == 0) a.f->sumdeg = sd[0];
+    if (tid == 0) {
+        a.f->sumdeg = sd[0];
+        a.f->inv_sumdeg = sd[0] > 0.0 ? 1.0 / sd[0] : 0.0;
+    }
 }
 
 static int grid_for(int64_t work, int sm)
@@ -293,7 +296,8 @@ rd_status check_csr(rd_graph* g, cudaStream_t st, int64_t* self_loops)
 int degree_grid(const rd_graph* g) { return grid_for(g->n, g->sm_count); }
 
 // Degrees (and, with check_weights, the weight checks of rd_graph_set_weights) with one launch and
-// one wait; `flags_dev` holds a CheckFlags and `block_sums_dev` degree_grid(g) doubles.
+// one wait; `flags_dev` holds a CheckFlags, in which the kernels of a step find the degrees' sum from
+// then on, and `block_sums_dev` degree_grid(g) doubles.
 rd_status compute_degrees(rd_graph* g, cudaStream_t st, void* flags_dev, double* block_sums_dev, bool check_weights)
 {
     CheckFlags* f = static_cast<CheckFlags*>(flags_dev);
@@ -321,7 +325,7 @@ rd_status compute_degrees(rd_graph* g, cudaStream_t st, void* flags_dev, double*
         set_error("edge weights must be finite and > 0");
         return RD_ERR_INVALID_ARG;
     }
-    g->sumdeg = h.sumdeg;
+    g->inv_sumdeg = &f->inv_sumdeg;
     g->mean_deg = g->n ? h.sumdeg / (double)g->n : 0.0;
     if (a.mirror) g->rows_sorted_sym = h.asymmetric == 0;
     if (h.zero_degree && g->n > 1) {

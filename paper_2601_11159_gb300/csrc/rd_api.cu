@@ -1346,8 +1346,7 @@ static FinArgs fin_args(const RunCtx& c, bool fp64, bool df)
     fa.rel_tol = c.o.rel_tol;
     fa.resid_tol = c.o.resid_tol;
     fa.est_delayed = (c.o.flags & RD_Q_EST_DELAYED) ? 1 : 0;
-    fa.sumdeg = c.g->sumdeg;
-    fa.inv_sumdeg = c.g->sumdeg > 0.0 ? 1.0 / c.g->sumdeg : 0.0;
+    fa.inv_sumdeg = c.g->inv_sumdeg;
     fa.elem_size = (int)c.pl.elem;
     return fa;
 }

@@ -194,8 +194,9 @@ struct FinArgs {
     int64_t ld;
     int npairs, tp, nblocks, step;      // step: 0-based index of the step just reduced
     int k_max, deflate, fixed_k, fp64;
-    double rel_tol, resid_tol, sumdeg;
-    double inv_sumdeg;                  // 1 / sumdeg
+    double rel_tol, resid_tol;
+    const double* inv_sumdeg;           // 1 / sum of the degrees, on the device: new weights leave the
+                                        // arguments, and with them the captured graphs, as they are
     int est_delayed;                    // 1: delayed-sum error estimate (RD_Q_EST_DELAYED)
     const double* block_part;
     PairState st;
@@ -334,7 +335,7 @@ struct rd_graph {
     float* invdeg32 = nullptr;
     rd::df64* degdf = nullptr;        // double-float copies (built on first use)
     rd::df64* invdegdf = nullptr;
-    double sumdeg = 0.0;
+    const double* inv_sumdeg = nullptr;  // 1 / sum of the degrees (device, in compute_degrees' flags)
     int32_t* mirror = nullptr;        // weighted graphs: entry (v, u) of each entry (u, v)
     bool mirror_ok = false;           // rows sorted and the structure symmetric: mirror is whole
     void* check_scratch = nullptr;    // flags and block sums of compute_degrees

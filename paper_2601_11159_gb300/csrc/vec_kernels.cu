@@ -142,11 +142,11 @@ struct StepCoef {
 // beta_{i+1} and its reciprocal by one rsqrt (366 cycles) with a Newton correction each, which
 // leaves both within rounding of sqrt and 1/sqrt (610 and 365 cycles): this chain stands between
 // the sums and the next vector.
-__device__ __forceinline__ StepCoef step_coef(const FinArgs& a, double A, double B, double C)
+__device__ __forceinline__ StepCoef step_coef(const FinArgs& a, double inv_sumdeg, double A, double B, double C)
 {
     StepCoef k;
     k.alpha = A;
-    k.cdef = a.deflate ? C * a.inv_sumdeg : 0.0;
+    k.cdef = a.deflate ? C * inv_sumdeg : 0.0;
     const double gamma2 = a.deflate ? C * k.cdef : 0.0;
     const double b2 = B - A * A - gamma2;
     k.beta2 = b2;
@@ -263,11 +263,11 @@ __device__ __forceinline__ void pair_store(const PairState& st, int p, int j, in
 
 // One step of pair p on the stored state: writes the pair's state and history; returns true when
 // the pair stops (then active = 0). `k` and `o` receive the step's coefficients and results.
-__device__ __forceinline__ bool pair_update(const FinArgs& a, const PairState& st, int p, int j, double A, double B,
+__device__ __forceinline__ bool pair_update(const FinArgs& a, const PairState& st, int p, int j, double isd, double A, double B,
                                             double C, StepCoef& k, PairStepOut& o)
 {
     PairScalars s = pair_load(st, p, a.pstride);
-    k = step_coef(a, A, B, C);
+    k = step_coef(a, isd, A, B, C);
     const bool stop = pair_core(a, s, j, k, o);
     pair_store(st, p, j, a.pstride, s, o, stop);
     return stop;
@@ -311,6 +311,7 @@ __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
         if (a.loop == 2 && blockIdx.x == 0 && threadIdx.x == 0) *a.loop_norm = a.k_max + 1;
         return;
     }
+    const double isd = __ldg(a.inv_sumdeg);
     // block partials b = split, split + nsplit, ...: four rows of loads in flight, summed
     // in block order (the order depends only on nblocks and ld, so runs are repeatable)
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
@@ -361,7 +362,7 @@ __global__ void __launch_bounds__(256) k_finalize(const FinArgs a)
         const double lam = a.xcf && j > 0 ? st.beta[p] * st.inv_delta[p] : 0.0;
         StepCoef k;
         PairStepOut o;
-        const bool stop = pair_update(a, st, p, j, A, B, C, k, o);
+        const bool stop = pair_update(a, st, p, j, isd, A, B, C, k, o);
         if (a.xcf && o.ok) {
             // p_i = q_i + lambda_i p_{i-1}, x += mu_i p_i (a stopping step still contributes)
             T* xc = static_cast<T*>(a.xcf) + (int64_t)j * 2 * ld;
@@ -1474,7 +1475,7 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
 {
     extern __shared__ __align__(16) unsigned char onchip_raw[];
     __shared__ double red[3][kOnchipThreads / 32];
-    __shared__ double coef[4];
+    __shared__ double coef[4], isd;
     __shared__ int stop_s;
     const int p = blockIdx.x;
     if (!onchip_start<kOnchipThreads>(a, p, threadIdx.x == 0)) return;  // uniform over the block
@@ -1490,6 +1491,7 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
     __syncthreads();
     OnchipPair pr;
     if (tid == 0) {
+        isd = __ldg(a.fin.inv_sumdeg);
         pr = onchip_pair(a, p);
         const int32_t s = a.s[p], t = a.t[p];
         const double ds = a.deg64[s], dt = a.deg64[t];
@@ -1580,7 +1582,7 @@ __global__ void __launch_bounds__(kOnchipThreads) k_lanczos_onchip(const OnchipA
                 B += red[1][w];
                 C += red[2][w];
             }
-            const StepCoef k = step_coef(a.fin, A, B, C);
+            const StepCoef k = step_coef(a.fin, isd, A, B, C);
             stop_s = onchip_update(a, pr, p, j, k, true) ? 1 : 0;
             coef[0] = k.alpha;
             coef[1] = k.cdef;
@@ -1698,6 +1700,7 @@ __global__ void __launch_bounds__(NT, (kClusterMinBlocks<T, FORM, NT>)) k_lanczo
     __shared__ double part[3][kClusterMax];       // every CTA's sums of the step, by rank
     __shared__ double tpart[3][NT];               // per-thread partial sums of the step
     __shared__ StepCoef coef;                     // of the step last summed
+    __shared__ double isd;                        // 1 / sum of the degrees
     __shared__ T next[4];                         // its 1/beta, alpha, c and beta as vector elements
     __shared__ int stop_s;
     __shared__ uint32_t rbase[kClusterMax];       // address of every rank's vectors
@@ -1738,7 +1741,10 @@ __global__ void __launch_bounds__(NT, (kClusterMinBlocks<T, FORM, NT>)) k_lanczo
         if constexpr (LEAN) return g_rp(u);
         else return s_rp[u];
     };
-    if (tid == 0) stop_s = 0;
+    if (tid == 0) {
+        stop_s = 0;
+        isd = __ldg(a.fin.inv_sumdeg);
+    }
     __syncthreads();
     const int nent = rp(nrow);
     const bool cached = !LEAN && nent <= L.nnz_cap;
@@ -1901,7 +1907,7 @@ __global__ void __launch_bounds__(NT, (kClusterMinBlocks<T, FORM, NT>)) k_lanczo
             for (int off = (C < 8 ? C : 8) >> 1; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
             const double A = __shfl_sync(0xffffffffu, s, 0), B = __shfl_sync(0xffffffffu, s, 8);
             const double Cs = __shfl_sync(0xffffffffu, s, 16);
-            const StepCoef k = step_coef(a.fin, A, B, Cs);
+            const StepCoef k = step_coef(a.fin, isd, A, B, Cs);
             if (lane == 0) {
                 coef = k;
                 next[0] = (T)k.inv_beta;

@@ -1234,3 +1234,38 @@ def test_device_loop_makes_no_pass_after_the_last_step(rd):
         best[k] = min(ts[5:])
         assert G.last_stats()["device_loop"] == 1
     assert abs((best[4] - best[3]) - (best[3] - best[2])) < 0.25 * (best[4] - best[2]) / 2, best
+
+
+@pytest.mark.parametrize("call", ["query", "edge_grad"])
+def test_new_weights_keep_the_captured_graphs(rd, call):
+    """A call after new weights costs what it costs after the same weights (a step's captured graphs took
+    the sum of the degrees as an argument, so every optimiser step captured them anew, at a third of the
+    price of the call on a graph this small), and follows them: the results are a fresh graph's."""
+    import time
+
+    import torch
+
+    g = F.random_connected(300, 900, 3, None)
+    s, t = (torch.from_numpy(x.astype(np.int32)).cuda() for x in F.random_pairs(g.n, 2, 8))
+    ws = [torch.from_numpy(F.weighted(g, F.lognormal_edge_weights(g.m, 0.0, 0.5, k)).w).cuda() for k in range(24)]
+    kw = dict(mode="fp64", k_max=3 if call == "query" else 9, fixed_k=True, kernel="group")
+
+    def run(G):
+        if call == "query":
+            return G.query(s, t, onchip=False, **kw).r
+        return G.edge_grad(s, t, **kw)[0]
+
+    G = rd.Graph(g.row_ptr, g.col, ws[0])
+    median = {}
+    for name, seq in (("first", ws[:4]), ("same", [ws[0]] * 24), ("new", ws), ("same again", [ws[0]] * 24)):
+        ts = []
+        for w in seq:
+            G.set_weights(w)
+            torch.cuda.synchronize()
+            at = time.perf_counter()
+            out = run(G)
+            ts.append(time.perf_counter() - at)
+        median[name] = np.median(ts)
+    assert median["new"] < 1.15 * max(median["same"], median["same again"]), median
+    G.set_weights(ws[7])
+    assert torch.equal(run(G), run(rd.Graph(g.row_ptr, g.col, ws[7])))
