@@ -153,9 +153,12 @@ typedef struct {
                               of a warp then hold rows of equal length), 4 = warp-per-task SpMV
                               (one column only: RD_Q_PLAIN or one pair; RD_ERR_UNSUPPORTED
                               otherwise), 5 = row-stream with asynchronous copies of the gathered
-                              rows into a shared-memory ring (FP32 vectors and 16 to 128 columns per
-                              slab only; RD_ERR_UNSUPPORTED otherwise; with one column it takes 4);
-                              with one column the fixed rule (RD_Q_NO_TUNE) takes 4 */
+                              rows into a shared-memory ring (16 to 128 FP32 columns per slab, 16 to
+                              64 of 8-byte elements; RD_ERR_UNSUPPORTED otherwise; with one column it takes 4),
+                              6 = row pipeline (a warp walks runs of consecutive rows in lockstep with
+                              the loads of the rows ahead in registers; for short rows; tiles, and one
+                              column, as 5; n <= 2^30); with one column the fixed rule (RD_Q_NO_TUNE)
+                              takes 4 */
 } rd_query_opts;
 
 /* Per-call statistics of the last rd_query / rd_edge_grad / rd_potential on g. */
@@ -167,7 +170,7 @@ typedef struct {
     int32_t rhs_tile;        /* configuration used */
     int32_t rows_per_warp;
     int32_t nnz_lanes;       /* lanes that share one row's nonzeros */
-    int32_t kernel;          /* SpMM kernel used, numbered as rd_query_opts::kernel (1 .. 5) */
+    int32_t kernel;          /* SpMM kernel used, numbered as rd_query_opts::kernel (1 .. 6) */
     int64_t ld;              /* padded number of right-hand-side columns (vector row stride) */
     double spmm_bytes;       /* algorithmic bytes of all SpMM launches of the call, each
                                 4*nnz (+4*nnz weights) + 8*(n+1) + 3*ld*n*sizeof(element) with the

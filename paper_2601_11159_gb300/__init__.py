@@ -109,7 +109,7 @@ def _opts(k_max=1000, rel_tol=1e-7, resid_tol=0.0, mode="fp32", rhs_tile=0, rows
     """rd_query_opts from keywords (each documented in include/rd.h): k_max, rel_tol,
     resid_tol, mode ("fp32" FP32 vectors with FP64 scalars, "fp64", "df64"), rhs_tile,
     rows_per_warp, chunk_steps, kernel ("tuned", "group", "stream", "group_sorted", "tasks",
-    "async" or its number); the booleans clear or set one flag each: fixed_k (RD_Q_FIXED_K),
+    "async", "pipe" or its number); the booleans clear or set one flag each: fixed_k (RD_Q_FIXED_K),
     deflate (RD_Q_NO_DEFLATE), plain (RD_Q_PLAIN), profile (RD_Q_PROFILE), compact
     (RD_Q_NO_COMPACT), onchip (RD_Q_NO_ONCHIP), tune (RD_Q_NO_TUNE), graph (RD_Q_NO_GRAPH),
     sparse_first (RD_Q_DENSE_FIRST), cluster (RD_Q_NO_CLUSTER), device_loop
@@ -131,7 +131,8 @@ def _opts(k_max=1000, rel_tol=1e-7, resid_tol=0.0, mode="fp32", rhs_tile=0, rows
     o.rhs_tile = int(rhs_tile)
     o.rows_per_warp = int(rows_per_warp)
     o.chunk_steps = int(chunk_steps)
-    o.kernel = ({"tuned": 0, "group": 1, "stream": 2, "group_sorted": 3, "tasks": 4, "async": 5}.get(kernel, kernel)
+    o.kernel = ({"tuned": 0, "group": 1, "stream": 2, "group_sorted": 3, "tasks": 4, "async": 5,
+                 "pipe": 6}.get(kernel, kernel)
                 if isinstance(kernel, str) else int(kernel))
     o.flags = ((RD_Q_FIXED_K if fixed_k else 0) | (0 if deflate else RD_Q_NO_DEFLATE) |
                (RD_Q_PLAIN if plain else 0) | (RD_Q_PROFILE if profile else 0) |

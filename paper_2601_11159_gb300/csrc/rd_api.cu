@@ -413,7 +413,8 @@ static int kernel_code(const SpmmCfg& c)
 {
     if (c.kind == 3) return 5;
     if (c.kind == 2) return 4;
-    if (c.kind == 1 || c.kind == 4) return 2;
+    if (c.kind == 4) return 6;
+    if (c.kind == 1) return 2;
     return c.order ? 3 : 1;
 }
 
@@ -488,8 +489,8 @@ static SpmmCfg pick_cfg(const rd_graph* g, int64_t P, const rd_query_opts& o, bo
     if (plain || P == 1) {
         c.vec = 1;
         c.gs = 1;
-        // warp-per-task SpMV (also for kernel 5, whose slabs need more than one column)
-        if ((o.kernel == 0 || o.kernel == 4 || o.kernel == 5) && g->ntasks > 0) {
+        // warp-per-task SpMV (also for kernels 5 and 6, whose slabs need more than one column)
+        if ((o.kernel == 0 || o.kernel >= 4) && g->ntasks > 0) {
             c.nzl = 1;
             c.kind = 2;
             return c;
@@ -509,12 +510,13 @@ static SpmmCfg pick_cfg(const rd_graph* g, int64_t P, const rd_query_opts& o, bo
         c.vec = 2;
         return c;
     }
-    if (o.kernel == 5) {  // async row-stream: tiles of 16 to 128 FP32 columns, 16 to 64 of 8-byte elements
+    // async row-stream and row pipeline: tiles of 16 to 128 FP32 columns, 16 to 64 of 8-byte elements
+    if (o.kernel == 5 || o.kernel == 6) {
         int tpa = o.rhs_tile > 0 ? o.rhs_tile : (P <= 16 ? 16 : (P <= 32 ? 32 : (P <= 64 || fp64 ? 64 : 128)));
         c.vec = fp64 ? 2 : 4;
         c.gs = std::max(1, tpa / c.vec);
         c.nzl = 1;
-        c.kind = 3;
+        c.kind = o.kernel == 5 ? 3 : 4;
         return c;
     }
     int tp = o.rhs_tile;
@@ -537,6 +539,10 @@ static rd_status make_plan_cfg(rd_graph* g, int64_t P, const rd_query_opts& o, c
     pl->fp64 = pl->prec != 0;
     pl->elem = pl->fp64 ? 8 : 4;
     pl->cfg = cfg;
+    if (cfg.kind == 4 && g->n > (1 << 30)) {  // its rows past the last are counted in 32 bits
+        set_error("the row pipeline takes graphs of up to 2^30 vertices");
+        return RD_ERR_UNSUPPORTED;
+    }
     if (!cfg_known(pl->cfg, pl->fp64)) {
         set_error("no SpMM kernel for rhs_tile/rows_per_warp = " + std::to_string(pl->cfg.tp()) + "/" +
                   std::to_string(pl->cfg.rpw()));
@@ -1669,8 +1675,8 @@ static rd_status validate_common(rd_graph* g, const int32_t* s, const int32_t* t
         set_error("k_max must be in [1, 2^22]");
         return RD_ERR_INVALID_ARG;
     }
-    if (o->kernel < 0 || o->kernel > 5) {
-        set_error("kernel must be 0, 1, 2, 3, 4 or 5");
+    if (o->kernel < 0 || o->kernel > 6) {
+        set_error("kernel must be 0, 1, 2, 3, 4, 5 or 6");
         return RD_ERR_INVALID_ARG;
     }
     if (o->mode != RD_MODE_FP64 && o->mode != RD_MODE_FP32V_FP64S && o->mode != RD_MODE_DF64) {

@@ -1269,3 +1269,59 @@ def test_new_weights_keep_the_captured_graphs(rd, call):
     assert median["new"] < 1.15 * max(median["same"], median["same again"]), median
     G.set_weights(ws[7])
     assert torch.equal(run(G), run(rd.Graph(g.row_ptr, g.col, ws[7])))
+
+
+@pytest.mark.parametrize("mode,bar", [("fp32", 2e-5), ("fp64", 1e-11), ("df64", 1e-11)])
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("n", [1999, 2017, 20033])
+def test_row_pipeline_by_name(rd, mode, bar, weighted, n):
+    """The row pipeline asked for by its number: rows of one to five entries, of a lane group and one more at
+    every tile width, long light rows and heavy ones; vertex counts no multiple of a run or of the rows
+    in flight; several slabs. Each tile has the row-group kernel's r_k (the bars that
+    test_short_row_graphs_match_oracle_history sets on graphs of this kind) and repeats bit for bit."""
+    a, b = [np.arange(n - 1)], [np.arange(1, n)]  # a path, and fans whose hubs lie anywhere in it
+    hubs = {7: 2, 201: 3, 411: 6, 621: 7, 801: 14, 1001: 15, 1201: 30, 1403: 31, 1601: 250, 33: 700, n - 1: 300}
+    for h, d in hubs.items():
+        a.append(np.full(d, h))
+        b.append((h + 3 + 2 * np.arange(d)) % n)
+    a, b = np.concatenate(a), np.concatenate(b)
+    lo, hi = np.minimum(a, b), np.maximum(a, b)
+    key = np.unique((lo * n + hi)[lo != hi])
+    g = to_csr(n, key // n, key % n)
+    if weighted:
+        g = F.weighted(g, F.lognormal_edge_weights(g.m, 0.0, 0.5, 6))
+    d = np.diff(g.row_ptr)
+    assert {1, 2, 3, 4, 5, 8, 9, 16, 17, 32, 33, 252} <= set(d) and (d > 256).sum() == 2
+    s, t = F.random_pairs(g.n, 75, 9)
+    G = rd.Graph.from_csr(g)
+    for tile in (16, 32, 64, 128):
+        if tile == 128 and mode != "fp32":
+            with pytest.raises(rd.RDError) as e:
+                G.query(s, t, mode=mode, kernel="pipe", rhs_tile=tile, k_max=2, onchip=False)
+            assert e.value.status == rd.RD_ERR_UNSUPPORTED
+            continue
+        for sparse_first in (True, False):
+            kw = dict(mode=mode, rhs_tile=tile, k_max=8, fixed_k=True, compact=False, onchip=False,
+                      sparse_first=sparse_first)
+            res = G.query(s, t, kernel="pipe", **kw)
+            st = G.last_stats()
+            assert st["kernel"] == 6 and st["rhs_tile"] == tile and st["ld"] == -(-75 // tile) * tile
+            assert rel(res.r, G.query(s, t, kernel="group", **kw).r).max() < bar
+            assert np.array_equal(G.query(s, t, kernel="pipe", **kw).r, res.r)
+    one = G.query(s[:1], t[:1], mode=mode, kernel="pipe", k_max=8, fixed_k=True, onchip=False)
+    assert G.last_stats()["kernel"] == 4 and rel(one.r, res.r[:1]).max() < bar
+
+
+def test_tuner_names_the_row_pipeline(rd):
+    """Where the tuner takes the row pipeline its number comes back, and asking for that configuration runs it."""
+    G = rd.Graph.from_csr(F.grid_deleted(400, 0.05, 5))
+    s, t = F.random_pairs(G.n, 16, 9)
+    for mode in ("fp32", "fp64", "df64"):
+        pick = G.autotune(16, mode=mode)
+        again = G.query(s, t, mode=mode, k_max=10, fixed_k=True, kernel=pick["kernel"], rhs_tile=pick["rhs_tile"],
+                        rows_per_warp=pick["rows_per_warp"])
+        st = G.last_stats()
+        assert (st["kernel"], st["rhs_tile"], st["rows_per_warp"]) == tuple(pick[k] for k in ("kernel", "rhs_tile",
+                                                                                           "rows_per_warp"))
+        assert np.array_equal(again.r, G.query(s, t, mode=mode, k_max=10, fixed_k=True).r)
+        assert G.last_stats()["kernel"] == pick["kernel"]
