@@ -588,7 +588,7 @@ static rd_status make_plan(rd_graph* g, int64_t P, const rd_query_opts& o, bool 
 struct Buffers {
     void* q[2];               // current q_{i-1}/W (slot 0) and q_i (slot 1)
     void* region_a;           // the two n x ld0 blocks q[] start in (the pass's blocks with pot_steps)
-    void* region_x;           // two n x packed_columns(ld0) blocks: target of a column compaction (NULL if off)
+    void* region_x;           // two n x pack_ld blocks: target of a column compaction (NULL if none can come)
     void* heavy_part;
     double* block_part;
     void* cf_hist;            // [k_max+1][4][ld0] (fixed layout: gradient, potential, no-alloc)
@@ -633,9 +633,11 @@ static int64_t block_bytes(int64_t n, int64_t ld, size_t elem)
 }
 
 // Widest layout a column compaction of an ld-column block packs into: half the columns, rounded up
-// to a tile that every width class has a candidate for (16 columns, 32 above 128).
+// to a tile that every width class has a candidate for (16 columns, 32 above 128). Blocks of up to 16
+// columns are never packed.
 static int64_t packed_columns(int64_t ld)
 {
+    if (ld <= 16) return 0;
     const int64_t half = (ld + 1) / 2, tile = half > 128 ? 32 : 16;
     return (half + tile - 1) / tile * tile;
 }
@@ -650,14 +652,14 @@ static int pot_steps_for(const rd_graph* g, const Plan& pl)
 }
 
 static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, bool grad, Buffers* b,
-                    bool compact = false, int pot_steps = 0)
+                    bool compact = false, int pot_steps = 0, int64_t pack_ld = 0)
 {
     const int64_t ld = pl.ld, n = g->n, K = pl.k_max;
     b->region_a = c.take<char>(std::max(2, pot_steps + 1) * block_bytes(n, ld, pl.elem));
     b->q[0] = b->region_a;
     b->q[1] = static_cast<char*>(b->region_a) + block_bytes(n, ld, pl.elem);
     // spare region: two packed blocks
-    b->region_x = compact ? c.take<char>(2 * block_bytes(n, packed_columns(ld), pl.elem)) : nullptr;
+    b->region_x = pack_ld > 0 ? c.take<char>(2 * block_bytes(n, pack_ld, pl.elem)) : nullptr;
     b->heavy_part = c.take<char>(std::max<int64_t>(g->n_chunks, 1) * ld * pl.elem);
     // sized for any column tile and any grid of up to 8 blocks of kBlock threads per SM
     b->block_part = c.take<double>((size_t)ld * 3 * (size_t)std::max(pl.grid_main, g->sm_count * 8));
@@ -754,6 +756,7 @@ struct RunCtx {
     double spmm_bytes = 0.0;
     bool profile = false;
     bool compact = false;   // coefficients by slot in cf_cur, columns packed as pairs finish
+    int64_t pack_ld = 0;    // into at most this many (0: none)
     bool lagged_polls = false;
     int cf_sel = 0, slot_sel = -1;  // slot_sel < 0: identity slot map
     bool in_region_x = false;
@@ -1029,7 +1032,8 @@ static rd_status enqueue_compaction(RunCtx& c, int active_upper, int fuse_step =
     Plan np;
     rd_query_opts o2 = c.o;
     o2.rhs_tile = 0;
-    const int64_t fit = packed_columns(c.pl.ld);  // what the spare region holds twice
+    const int64_t fit = c.pack_ld;  // what the spare region holds twice
+    if (fit == 0) return RD_OK;
     RD_TRY(make_plan(c.g, active_upper, o2, false, &np, fit));
     if (np.ld >= c.cur.ld || np.ld > fit) return RD_OK;
     if (fuse_step >= 0 && np.ld % (16 / (int64_t)np.elem) != 0) return RD_OK;
@@ -1869,15 +1873,18 @@ static rd_status prepare_run(RunCtx& c, rd_graph* g, int64_t P, const rd_query_o
     // a gradient or potential call that steps from captured graphs keeps a pass's vectors, memory
     // permitting
     c.pot_steps = grad && !c.profile && !(o.flags & (RD_Q_NO_GRAPH | RD_Q_REPLAY_POTENTIAL)) ? pot_steps_for(g, c.pl) : 0;
+    c.pack_ld = compact ? packed_columns(c.pl.ld) : 0;
     for (;;) {
         Carver dry(nullptr);
-        const rd_status ws = ensure_ws(g, carve(dry, g, c.pl, P, grad, &c.b, compact, c.pot_steps));
+        const rd_status ws = ensure_ws(g, carve(dry, g, c.pl, P, grad, &c.b, compact, c.pot_steps, c.pack_ld));
         if (ws >= 0) break;
-        if (c.pot_steps == 0) return ws;
-        c.pot_steps = 0;
+        // without the memory: no kept vectors, packing into no more than half the columns
+        if (c.pot_steps > 0) c.pot_steps = 0;
+        else if (c.pack_ld > c.pl.ld / 2) c.pack_ld = c.pl.ld / 2;
+        else return ws;
     }
     Carver real(g->ws.base);
-    carve(real, g, c.pl, P, grad, &c.b, compact, c.pot_steps);
+    carve(real, g, c.pl, P, grad, &c.b, compact, c.pot_steps, c.pack_ld);
     return RD_OK;
 }
 

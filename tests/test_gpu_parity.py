@@ -1325,3 +1325,21 @@ def test_tuner_names_the_row_pipeline(rd):
                                                                                            "rows_per_warp"))
         assert np.array_equal(again.r, G.query(s, t, mode=mode, k_max=10, fixed_k=True).r)
         assert G.last_stats()["kernel"] == pick["kernel"]
+
+
+def test_narrow_queries_hold_no_packing_space(rd):
+    """A query of up to 16 columns never packs them, and its workspace holds no blocks to pack into: one pair
+    on a large graph takes a few vectors, 16 and 17 pairs what their blocks need."""
+    import torch
+
+    g = F.grid(2000)
+    G = rd.Graph.from_csr(g, label_components=False)
+    n4 = 4.0 * g.n
+    s, t = F.random_pairs(g.n, 17, 8)
+    used = 0.0
+    for pairs, columns in ((1, 2), (16, 32), (17, 2 * 32 + 2 * 16)):
+        free = torch.cuda.mem_get_info()[0]
+        G.query(s[:pairs], t[:pairs], mode="fp32", k_max=3, fixed_k=True, tune=False)
+        used += free - torch.cuda.mem_get_info()[0]
+        # beside the vector blocks: heavy-row sums, the mask of the first pass (a bit a column and row)
+        assert used < (columns + (columns + 31) // 32 + 1) * n4 + 64e6, (pairs, used / n4)
