@@ -724,6 +724,21 @@ static size_t carve(Carver& c, const rd_graph* g, const Plan& pl, int64_t P, boo
     return c.off + 256;
 }
 
+// Whether a workspace of `with` bytes may take the place of one of `without`: it is there already, or it
+// leaves three quarters of what would be free beside the smaller one (the graph holds it from then
+// on, and the caller's other allocations need that memory).
+static bool room_for_passes(const rd_graph* g, size_t with, size_t without)
+{
+    if (with <= g->ws.bytes) return true;
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    const size_t avail = free_bytes + g->ws.bytes;
+    return avail > without && with - without <= (avail - without) / 4;
+}
+
 struct EventPool {
     std::vector<cudaEvent_t> ev;
     size_t used = 0;
@@ -1857,7 +1872,7 @@ static rd_status ensure_tuned(rd_graph* g, int64_t P, const rd_query_opts& o, bo
 }
 
 static rd_status prepare_run(RunCtx& c, rd_graph* g, int64_t P, const rd_query_opts& o, bool plain, bool grad,
-                             cudaStream_t st, bool compact = false, bool lagged_polls = false)
+                             cudaStream_t st, bool compact = false, bool lagged_polls = false, bool passes = true)
 {
     c.g = g;
     c.o = o;
@@ -1872,7 +1887,14 @@ static rd_status prepare_run(RunCtx& c, rd_graph* g, int64_t P, const rd_query_o
     c.cur = c.pl;
     // a gradient or potential call that steps from captured graphs keeps a pass's vectors, memory
     // permitting
-    c.pot_steps = grad && !c.profile && !(o.flags & (RD_Q_NO_GRAPH | RD_Q_REPLAY_POTENTIAL)) ? pot_steps_for(g, c.pl) : 0;
+    c.pot_steps = grad && passes && !c.profile && !(o.flags & (RD_Q_NO_GRAPH | RD_Q_REPLAY_POTENTIAL))
+                      ? pot_steps_for(g, c.pl)
+                      : 0;
+    if (c.pot_steps > 0) {
+        Carver with(nullptr), without(nullptr);
+        const size_t w = carve(with, g, c.pl, P, grad, &c.b, compact, c.pot_steps);
+        if (!room_for_passes(g, w, carve(without, g, c.pl, P, grad, &c.b, compact))) c.pot_steps = 0;
+    }
     c.pack_ld = compact ? packed_columns(c.pl.ld) : 0;
     for (;;) {
         Carver dry(nullptr);
@@ -1886,6 +1908,20 @@ static rd_status prepare_run(RunCtx& c, rd_graph* g, int64_t P, const rd_query_o
     Carver real(g->ws.base);
     carve(real, g, c.pl, P, grad, &c.b, compact, c.pot_steps, c.pack_ld);
     return RD_OK;
+}
+
+// Runs call(passes, &used), and where it keeps a pass's vectors (used) and any allocation of the call then
+// fails -- staged outputs, entry rows -- gives the workspace back and runs it again without them.
+template <class Call>
+static rd_status retry_without_passes(rd_graph* g, Call&& call)
+{
+    bool used = false;
+    const rd_status rs = call(true, &used);
+    if (rs != RD_ERR_OOM || !used) return rs;
+    cudaFree(g->ws.base);
+    g->ws.base = nullptr;
+    g->ws.bytes = 0;
+    return call(false, &used);
 }
 
 // Host-side query of a batch of pairs (all device work on st).
@@ -2357,8 +2393,11 @@ rd_status rd_autotune(rd_graph* g, int64_t npairs, const rd_query_opts* opts, in
     return RD_OK;
 }
 
-rd_status rd_edge_grad(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs, const double* grad_r,
-                       const rd_query_opts* opts, float* grad_w_out, double* r_out, void* stream)
+}  // extern "C"
+
+static rd_status edge_grad(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs, const double* grad_r,
+                           const rd_query_opts* opts, float* grad_w_out, double* r_out, void* stream, bool passes,
+                           bool* used)
 {
     g_last_error.clear();
     rd_query_opts o;
@@ -2378,7 +2417,8 @@ rd_status rd_edge_grad(rd_graph* g, const int32_t* s, const int32_t* t, int64_t 
     EventPool ev;
     RunCtx c;
     c.ev = &ev;
-    RD_TRY(prepare_run(c, g, npairs, o, false, true, st));
+    RD_TRY(prepare_run(c, g, npairs, o, false, true, st, false, false, passes));
+    *used = c.pot_steps > 0;
     rd_status call = RD_OK;
     RD_TRY(forward_and_potential(c, s, t, grad_r, &call));
     // edge kernel over internal entries, then map to the caller's entry order
@@ -2431,10 +2471,16 @@ rd_status rd_edge_grad(rd_graph* g, const int32_t* s, const int32_t* t, int64_t 
     return outs;
 }
 
-}  // extern "C"
+extern "C" rd_status rd_edge_grad(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs, const double* grad_r,
+                                  const rd_query_opts* opts, float* grad_w_out, double* r_out, void* stream)
+{
+    return retry_without_passes(g, [&](bool passes, bool* used) {
+        return edge_grad(g, s, t, npairs, grad_r, opts, grad_w_out, r_out, stream, passes, used);
+    });
+}
 
-extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs,
-                                  const rd_query_opts* opts, float* phi_out, double* r_out, void* stream)
+static rd_status potential(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs, const rd_query_opts* opts,
+                           float* phi_out, double* r_out, void* stream, bool passes, bool* used)
 {
     g_last_error.clear();
     rd_query_opts o;
@@ -2450,7 +2496,8 @@ extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* 
     EventPool ev;
     RunCtx c;
     c.ev = &ev;
-    RD_TRY(prepare_run(c, g, npairs, o, false, true, st));
+    RD_TRY(prepare_run(c, g, npairs, o, false, true, st, false, false, passes));
+    *used = c.pot_steps > 0;
     rd_status call = RD_OK;
     RD_TRY(forward_and_potential(c, s, t, nullptr, &call));
     // phi (n x ld, q-space) -> pair-major float output
@@ -2481,8 +2528,16 @@ extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* 
     return outs;
 }
 
-extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs,
-                             const rd_query_opts* opts, float* flow_out, double* r_out, void* stream)
+extern "C" rd_status rd_potential(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs,
+                                  const rd_query_opts* opts, float* phi_out, double* r_out, void* stream)
+{
+    return retry_without_passes(g, [&](bool passes, bool* used) {
+        return potential(g, s, t, npairs, opts, phi_out, r_out, stream, passes, used);
+    });
+}
+
+static rd_status flow(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs, const rd_query_opts* opts,
+                      float* flow_out, double* r_out, void* stream, bool passes, bool* used)
 {
     g_last_error.clear();
     rd_query_opts o;
@@ -2498,15 +2553,16 @@ extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, in
     EventPool ev;
     RunCtx c;
     c.ev = &ev;
-    RD_TRY(prepare_run(c, g, npairs, o, false, true, st));
+    RD_TRY(prepare_run(c, g, npairs, o, false, true, st, false, false, passes));
+    *used = c.pot_steps > 0;
     rd_status call = RD_OK;
     RD_TRY(forward_and_potential(c, s, t, nullptr, &call));
+    RD_TRY(ensure_entry_rows(c));
     const size_t bytes = sizeof(float) * (size_t)g->nnz_in * (size_t)npairs;
     const bool dev_out = in_place(flow_out, g->device, sizeof(float));
     float* stage = dev_out ? flow_out : nullptr;
     if (!dev_out && bytes) RD_CUDA(cudaMallocAsync((void**)&stage, bytes, st));
     if (g->keep_idx && bytes) RD_CUDA(cudaMemsetAsync(stage, 0, bytes, st));
-    RD_TRY(ensure_entry_rows(c));
     PairMajorArgs pa{};
     pa.items = g->nnz;
     pa.ld = c.pl.ld;
@@ -2527,6 +2583,14 @@ extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, in
     RD_TRY(finish_outputs(c, r_out, nullptr, nullptr, nullptr, &outs));
     record_stats(c);
     return outs;
+}
+
+extern "C" rd_status rd_flow(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npairs,
+                             const rd_query_opts* opts, float* flow_out, double* r_out, void* stream)
+{
+    return retry_without_passes(g, [&](bool passes, bool* used) {
+        return flow(g, s, t, npairs, opts, flow_out, r_out, stream, passes, used);
+    });
 }
 
 // ============================================================ Power Method

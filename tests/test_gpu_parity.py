@@ -1343,3 +1343,33 @@ def test_narrow_queries_hold_no_packing_space(rd):
         used += free - torch.cuda.mem_get_info()[0]
         # beside the vector blocks: heavy-row sums, the mask of the first pass (a bit a column and row)
         assert used < (columns + (columns + 31) // 32 + 1) * n4 + 64e6, (pairs, used / n4)
+
+
+def test_kept_vectors_give_way_to_the_calls_outputs(rd):
+    """Flows handed out in host memory with little device memory left: the vectors kept for a pass are given
+    up, in the plan (they may take a quarter of what would be free) or once the staged output does not
+    fit, and the call succeeds with the same flows; with room for them they are kept."""
+    import torch
+
+    g = F.random_connected(400_000, 4_400_000, 3, None)
+    s, t = F.random_pairs(g.n, 32, 8)
+    kw = dict(mode="fp32", k_max=9, fixed_k=True, kernel="group", rhs_tile=32)
+    G = rd.Graph.from_csr(g, label_components=False)
+    ref, r = G.flow(s, t, **kw)
+    passes = G.last_stats()["launches"]
+    G.close()
+    # in vector blocks: 2 for the steps, 2 for the potential, 7 more for kept vectors; the flows 24
+    block = 4 * g.n * 32
+    assert 23.9 < 4 * g.nnz * 32 / block < 24.1
+    torch.cuda.synchronize()
+    for left, kept in ((30, False), (33, False), (60, True)):
+        G = rd.Graph.from_csr(g, label_components=False)
+        torch.cuda.empty_cache()
+        hog = torch.empty(int(torch.cuda.mem_get_info()[0] - left * block - 8 * g.nnz - 16e6), dtype=torch.uint8,
+                          device="cuda")
+        f, r2 = G.flow(s, t, **kw)
+        assert np.array_equal(f, ref) and np.array_equal(r2, r), left
+        assert (G.last_stats()["launches"] == passes) == kept, left
+        del hog
+        G.close()
+    torch.cuda.empty_cache()
