@@ -143,9 +143,11 @@ typedef struct {
     int32_t mode;          /* rd_mode */
     int32_t rhs_tile;      /* right-hand-side columns per SpMM sweep; 0 = tuned */
     int32_t rows_per_warp; /* rows a warp works on at once; 0 = tuned */
-    int32_t chunk_steps;   /* steps between synchronous host convergence polls where those are used
-                              (rd_edge_grad, rd_potential, rd_query_noalloc); 0 = default (8).
-                              rd_query polls every step, one step behind the device. */
+    int32_t chunk_steps;   /* steps between host convergence polls where those are used (rd_edge_grad,
+                              rd_potential, rd_flow, rd_query_noalloc); 0 = default (8). Where the
+                              first three keep the vectors of a pass of up to 8 steps, the poll comes at
+                              the end of the pass it falls into. rd_query reads the counts on the
+                              device. */
     uint32_t flags;        /* RD_Q_* */
     int32_t kernel;        /* SpMM kernel: 0 = tuned, 1 = row-group (warp lanes split a row's
                               nonzeros), 2 = row-stream (row groups walk runs of consecutive rows),

@@ -1963,8 +1963,10 @@ static void launch_pot_pass_t(int grid, cudaStream_t st, const PotPassArgs<doubl
 // The forward steps of a gradient or potential call in passes of c.pot_steps steps whose vectors
 // are kept (see PotPassArgs): each pass is one CUDA graph -- the steps, each writing W into the
 // next block, and k_potential_pass -- the first of them without step 0, which is launched before
-// it (the sparse first step where it applies). The host waits for the count of active pairs after
-// each pass; steps after the last active pair return at once.
+// it (the sparse first step where it applies). The host reads the count of active pairs after
+// chunk_steps steps, rounded up to whole passes: in runs of fixed length, where only breakdowns end a
+// pair early, while the next pass runs; otherwise it waits for it. Steps after the last active pair
+// return at once.
 template <typename T>
 static rd_status run_potential(RunCtx& c)
 {
@@ -2041,8 +2043,11 @@ static rd_status run_potential(RunCtx& c)
     pa.act_count = c.b.st.act_count;
     pa.base = c.b.pot_base;
     pa.ticket = c.b.pot_ticket;
-    int* h = g->h_pinned;
-    for (int done = 0; done < c.pl.k_max; done += m) {
+    int* h = g->h_pinned;  // [0] error flag, [1] active count, [4 .. 5] counts of fixed-length runs
+    const int every = std::max(1, ((c.o.chunk_steps > 0 ? c.o.chunk_steps : m) + m - 1) / m);
+    cudaEvent_t poll_ev[2] = {};
+    int polls = 0;
+    for (int done = 0, pass = 1; done < c.pl.k_max; done += m, ++pass) {
         const int first = done == 0 ? 1 : 0;  // position the pass's graph starts at
         step_o(first, &sa, &fa, &na);
         int misc[9] = {c.cur.cfg.vec, c.cur.cfg.gs, c.cur.cfg.nzl, c.cur.cfg.kind, c.cur.grid_main, c.cur.grid_heavy,
@@ -2097,9 +2102,21 @@ static rd_status run_potential(RunCtx& c)
         c.spmm_bytes += spmm_launch_bytes(g, c.cur) * steps;
         c.steps = std::min(c.pl.k_max, done + m);
         if (c.steps == c.pl.k_max && done > 0) break;
-        if (done > 0 && base.fixed_k) continue;  // every pair goes on but for breakdowns
+        if (done > 0 && pass % every != 0) continue;
+        const int32_t* count = c.b.st.act_count + c.steps;
+        if (done > 0 && base.fixed_k) {
+            const int sl = polls & 1;
+            if (!poll_ev[sl]) poll_ev[sl] = c.ev->get();
+            RD_CUDA(cudaMemcpyAsync(h + 4 + sl, count, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+            RD_CUDA(cudaEventRecord(poll_ev[sl], c.st));
+            if (polls++ > 0) {  // the count of the poll before, whose copy this pass ran behind
+                RD_CUDA(cudaEventSynchronize(poll_ev[1 - sl]));
+                if (h[4 + 1 - sl] == 0) break;
+            }
+            continue;
+        }
         RD_CUDA(cudaMemcpyAsync(h, c.b.err_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
-        RD_CUDA(cudaMemcpyAsync(h + 1, c.b.st.act_count + c.steps, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+        RD_CUDA(cudaMemcpyAsync(h + 1, count, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
         RD_CUDA(cudaStreamSynchronize(c.st));
         if (h[0]) {
             set_error("a pair id is outside [0, n)");

@@ -1373,3 +1373,37 @@ def test_kept_vectors_give_way_to_the_calls_outputs(rd):
         del hog
         G.close()
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("call", ["potential", "edge_grad", "flow"])
+def test_pass_calls_poll_as_asked(rd, call):
+    """Runs of fixed length end soon after every pair has ended (here: broken down in the first pass, or, without
+    deflation, lost definiteness in the fifteenth), not at k_max, and chunk_steps sets the
+    steps between polls, rounded up to passes of 8; the outputs are those of the launch-per-kernel loop."""
+    side = np.repeat(np.arange(4), 4)  # complete bipartite: pairs on one side break down exactly at once
+    G = rd.Graph.from_csr(to_csr(8, side, 4 + np.tile(np.arange(4), 4)))
+    s, t = np.array([0, 1, 0, 4, 6], np.int32), np.array([1, 2, 3, 5, 7], np.int32)
+    kw = dict(mode="fp64", kernel="group")
+    out, _ = getattr(G, call)(s, t, k_max=20000, fixed_k=True, **kw)
+    assert G.last_stats()["steps"] <= 32
+    ref, _ = getattr(G, call)(s, t, k_max=40, fixed_k=True, graph=False, **kw)
+    assert np.array_equal(out, ref)
+    h = F.grid(20)
+    H = rd.Graph.from_csr(h)
+    s, t = F.random_pairs(h.n, 5, 8)
+    lost = dict(mode="fp32", kernel="group", fixed_k=True, deflate=False)
+    last = int(H.query(s, t, k_max=20000, onchip=False, **lost).iters.max())
+    assert 16 < last < 400
+    out, _ = getattr(H, call)(s, t, k_max=20000, **lost)
+    assert H.last_stats()["steps"] <= last + 3 * 8
+    ref, _ = getattr(H, call)(s, t, k_max=last + 40, graph=False, **lost)
+    assert np.array_equal(out, ref, equal_nan=True)
+    kw = dict(kw, k_max=4000, rel_tol=0.0, resid_tol=1e-10)
+    ref, _ = getattr(H, call)(s, t, **kw)
+    needed = H.last_stats()["steps"]  # within a pass of the last pair's
+    assert needed % 8 == 0 and 32 < needed < 400
+    for chunk in (1, 8, 9, 64, 100):
+        out, _ = getattr(H, call)(s, t, chunk_steps=chunk, **kw)
+        every = -(-chunk // 8) * 8
+        assert H.last_stats()["steps"] == -(-needed // every) * every
+        assert np.array_equal(out, ref)
