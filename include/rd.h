@@ -21,7 +21,9 @@
  *    rd_last_error() returns a human-readable detail for the calling thread.
  *  - Pointers marked "host or device" may be either; the library tells them
  *    apart with cudaPointerGetAttributes and stages host buffers itself.
- *    Device pointers must be device memory of the current CUDA device.
+ *    Device pointers should be device memory of the current CUDA device,
+ *    aligned to their elements: those are read and written in place, any
+ *    others (a peer's, a byte offset) are copied.
  *  - Streams: `stream` is a cudaStream_t passed as void* (NULL = legacy
  *    default stream). All device work of a call is ordered on that stream.
  *    rd_query, rd_edge_grad and rd_potential synchronize that stream before
@@ -91,16 +93,19 @@ typedef enum {
 #define RD_Q_NO_COMPACT 16u /* rd_query: keep every pair's column until the end instead of packing
                                the still-active pairs into a narrower block as pairs converge */
 #define RD_Q_NO_ONCHIP 32u  /* rd_query: do not run small graphs (three vectors fit in one SM's
-                               shared memory) as one whole-recurrence kernel with one block per pair */
+                               shared memory) as one whole-recurrence kernel (one CTA per pair, or a
+                               thread-block cluster of them: see RD_Q_NO_CLUSTER) */
 #define RD_Q_NO_TUNE 64u    /* with rhs_tile, rows_per_warp and kernel all 0: pick the SpMM
                                configuration by a fixed rule instead of the autotuner (see
                                rd_autotune) */
 #define RD_Q_EST_DELAYED 256u /* rel_tol test on the sum of the last 4 increments of
                                e_1^T (I-T_k)^{-1} e_1 (the error of the estimate 4 steps back)
                                instead of the default geometric tail estimate (see rel_tol) */
-#define RD_Q_NO_GRAPH 128u  /* rd_query: launch every kernel of every step from the host instead
-                               of replaying a captured CUDA graph of one step (the results are
-                               bitwise the same; RD_Q_PROFILE also turns the graphs off) */
+#define RD_Q_NO_GRAPH 128u  /* launch every kernel of every step from the host instead of replaying
+                               captured CUDA graphs (rd_query: of the step loop or of one step;
+                               rd_edge_grad, rd_potential, rd_flow: of a pass of up to 8 steps whose
+                               vectors are kept). The results are bitwise the same; RD_Q_PROFILE also
+                               turns the graphs off */
 #define RD_Q_DENSE_FIRST 512u /* compute the first step's product D^{-1} A q_1 with the SpMM over
                                every row. By default, when the graph's rows are sorted by column
                                and its entries symmetric (checked by rd_graph_create and
@@ -115,11 +120,11 @@ typedef enum {
                                from the LDL^T factors of I - T_i; one extra vector, no second pass);
                                the two agree to rounding */
 #define RD_Q_NO_CLUSTER 2048u /* rd_query: run the whole-recurrence kernel of small graphs with one CTA
-                               per pair. By default, when few pairs are asked (pairs x 2 x CTAs <= SMs),
+                               per pair. By default, when few pairs are asked (pairs x CTAs <= SMs),
                                each pair's recurrence runs on a thread-block cluster of up to 16 CTAs
-                               (one per SM), each holding a slice of the three vectors in its shared
-                               memory and reading the others' through distributed shared memory; the
-                               two agree to rounding */
+                               (one per SM, at least 64 rows each), each holding a slice of the three
+                               vectors in its shared memory and reading the others' through distributed
+                               shared memory or a copy of its own; the two agree to rounding */
 #define RD_Q_NO_DEVICE_LOOP 4096u /* rd_query: launch each step's CUDA graph from the host and poll
                                the active count between steps. By default the steps after the first
                                run in one graph whose conditional (while) node repeats the step on
@@ -245,6 +250,10 @@ rd_status rd_query(rd_graph* g, const int32_t* s, const int32_t* t, int64_t npai
  * delta * (sum of the two). phi is built during the forward steps from the LDL^T factors of
  * I - T_i (no basis V_k is kept and no second pass runs); RD_Q_REPLAY_POTENTIAL instead
  * rebuilds it by a second Lanczos pass that replays the stored alpha/beta.
+ * Memory (this call, rd_potential and rd_flow): the vectors of a pass of up to 8 steps are kept
+ * and the potential updated once per pass, where they take at most 8 GB and at most a quarter of
+ * the memory that would be free without them; they stay in g's workspace. Otherwise, and where
+ * another allocation of the call fails, the potential is updated with every step.
  *  grad_r     : double[npairs] host or device, or NULL for all ones.
  *  grad_w_out : float[nnz_created] host or device (nnz as passed to create; entries that
  *               were self-loops get 0).
@@ -326,11 +335,15 @@ rd_status rd_query_noalloc(int64_t n, int64_t nnz, const int64_t* row_ptr, const
 /* SpMM autotuner. No counterpart in the paper: it picks the right-hand-side tile, the rows
  * per warp and the kernel of the SpMM step of Algorithm 3 for this graph and GPU by
  * timing, not by a fixed rule. For a query of npairs pairs in opts->mode it times every
- * instantiated candidate (tiles from a quarter of the pair count's power-of-two width up to
- * that width; the row-stream kernel and the row-group kernel with 1, 2 or 4 nonzero lanes
- * per row group; for one column the warp-per-task SpMV, the row-stream and the row-group
- * SpMV) on g's own CSR with zeroed vectors, one warm-up and three timed launches each (CUDA
- * events on `stream`), and keeps the fastest per width class in g. Without RD_Q_PLAIN (and
+ * instantiated candidate (tiles from a quarter -- on small graphs and for the async kernel an
+ * eighth -- of the pair count's power-of-two width up to that width; the row-stream kernel, the
+ * row-group kernel with 1, 2 or 4 nonzero lanes per row group in natural and degree order, the
+ * async kernel and, where rows average eight entries or fewer, the row pipeline; for one column
+ * the warp-per-task SpMV, the row-stream and the row-group SpMV) on g's own CSR with zeroed
+ * vectors, one warm-up and three timed launches each (CUDA events on `stream`; a candidate whose
+ * warm-up takes over twice the best is out), and keeps every candidate's time per width class in
+ * g: a call takes the one that carries its own pairs, rounded up to the candidate's tile, through
+ * a step in the least time, a lead within 3% deciding nothing. Without RD_Q_PLAIN (and
  * npairs > 1) the narrower classes a compacting query passes through are tuned as well,
  * unless RD_Q_NO_COMPACT is set. Calls on g whose opts leave rhs_tile, rows_per_warp and
  * kernel at 0 without RD_Q_NO_TUNE use the table, and tune a missing class on first use.

@@ -188,8 +188,8 @@ static int32_t label_components(int64_t n, const std::vector<int64_t>& rp, const
 // warp, and light rows of up to 256 left the main kernel half idle at its end; the query of 70
 // pairs takes 2.8 ms with 256 and 1.9 ms with 64. A line at 32 per SM instead of 128 costs a training
 // step over 2M entries 3.02 for 2.75 ms and flows over 3.9M entries 1.03 for 0.93 ms. A
-// hub's chunks are summed by one row group, so a row has at most 128 of them. Graphs small enough
-// for the whole-recurrence kernel keep 256.
+// hub's chunks are summed by one row group, so shorter chunks are not taken where a row would have more
+// than 128 of them. Graphs small enough for the whole-recurrence kernel keep 256.
 static void choose_chunk(rd_graph* g, const std::vector<int64_t>& rp)
 {
     if (onchip_smem_bytes(g->n, 4) <= 220 * 1024) return;

@@ -764,8 +764,8 @@ __device__ __forceinline__ void row_epilogue_b(const StepArgs<T>& a, int row, in
 // registers) hold a round's eight 16-byte gathers beside the sums; with four (64) some of them
 // wait for registers: a training step on Chung-Lu 100k 2,624 -> 2,458 us with three, flows on
 // 200,000 vertices 779 -> 728 us (768 with two). Elements of 8 bytes take two (128 registers; at
-// 80 the weighted kernels spill): 70 FP64 columns on Chung-Lu 20k 1,820 -> 1,792 us a query, 50
-// steps of the Power Method on 100,000 vertices 5,250 -> 5,116.
+// 80 the weighted kernels spill): 70 FP64 columns on Chung-Lu 20k 1,820 -> 1,806 us a query, 50
+// steps of the Power Method on 100,000 vertices 5,250 -> 5,126.
 #ifndef RD_GROUP_SMEM
 #define RD_GROUP_SMEM 1
 #endif
