@@ -812,6 +812,8 @@ static StepArgs<T> step_args(RunCtx& c, int j, bool reduce)
     a.row_ptr = g->row_ptr;
     a.col = g->col;
     a.w = g->w;
+    a.col_mid = g->col + kMidEntry;
+    a.w_mid = g->w ? g->w + kMidEntry : nullptr;
     if constexpr (std::is_same<T, df64>::value) {
         a.invdeg = g->invdegdf;
         a.deg = g->degdf;

@@ -886,11 +886,11 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
 
         for (int task = gid; task < ntasks; task += ngroups) {
             const int r0 = a.task_row[task], r1 = a.task_row[task + 1];
-            const uint32_t e_beg = (uint32_t)a.row_ptr[r0], e_end = (uint32_t)a.row_ptr[r1];  // (see gather_row)
+            const int e_beg = mid_entry(a.row_ptr[r0]), e_end = mid_entry(a.row_ptr[r1]);
             T acc[VEC], qp[VEC], qc[VEC];
 #pragma unroll
             for (int i = 0; i < VEC; ++i) acc[i] = T(0);
-            if (r1 == r0 + 1 && (int)(e_end - e_beg) > a.heavy_thr) {
+            if (r1 == r0 + 1 && e_end - e_beg > a.heavy_thr) {
                 ld_stream<T, VEC>(qp, a.qprev + (int64_t)r0 * ld + c0);
                 ld_gather<T, VEC>(qc, q + (int64_t)r0 * ld);
                 heavy_row_sum<T, VEC, 1>(a, r0, c0, 0, acc);
@@ -899,23 +899,23 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
             }
             // row window: lane gl holds row_ptr[w0 + gl + 1], 1/d and d of row w0 + gl
             int w0 = r0;
-            uint32_t my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : e_end;
+            int my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : e_end;
             T my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
-            uint32_t row_end = __shfl_sync(mask, my_end, 0, GS);
+            int row_end = __shfl_sync(mask, my_end, 0, GS);
             ld_stream<T, VEC>(qp, a.qprev + (int64_t)row * ld + c0);
             ld_gather<T, VEC>(qc, q + (int64_t)row * ld);
-            for (uint32_t base = e_beg; base < e_end; base += CH) {
-                const int cnt = e_end - base < (uint32_t)CH ? (int)(e_end - base) : CH;
+            for (int base = e_beg; base < e_end; base += CH) {
+                const int cnt = e_end - base < CH ? e_end - base : CH;
                 uint32_t my_off[NH];
                 float my_w[NH];
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
                     const int idx = h * GS + gl;
-                    const uint32_t j = idx < cnt ? (uint32_t)__ldg(a.col + base + idx) : 0u;
+                    const uint32_t j = idx < cnt ? (uint32_t)__ldg(a.col_mid + base + idx) : 0u;
                     my_off[h] = j * ldv;
-                    if constexpr (WEIGHTED) my_w[h] = idx < cnt ? __ldg(a.w + base + idx) : 0.0f;
+                    if constexpr (WEIGHTED) my_w[h] = idx < cnt ? __ldg(a.w_mid + base + idx) : 0.0f;
 #if RD_ROWS_PREFETCH
                     if (idx < cnt) {
                         const char* rowp = reinterpret_cast<const char*>(qslab + (int64_t)j * ld);
@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                     }
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const uint32_t e = base + k0 + u;
+                        const int e = base + k0 + u;
                         if (e >= e_end) break;
                         while (e >= row_end) {  // the stream leaves `row`
                             const int wi = row - w0;
@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                             ++row;
                             if (row - w0 >= GS) {  // refill the row window
                                 w0 = row;
-                                my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : e_end;
+                                my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : e_end;
                                 my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                                 my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                             }
@@ -993,7 +993,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                 if (row >= r1) break;
                 if (row - w0 >= GS) {
                     w0 = row;
-                    my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : e_end;
+                    my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : e_end;
                     my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }
@@ -1083,14 +1083,14 @@ struct AsyncRound {
     uint32_t off[NH];
     float w[NH];
     template <class Args>
-    __device__ __forceinline__ void load(const Args& a, uint32_t base, uint32_t end, int gl, uint32_t ldv)
+    __device__ __forceinline__ void load(const Args& a, int base, int end, int gl, uint32_t ldv)
     {
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
             const int pos = h * GS + gl;
             const bool ok = pos < kAsyncDepth && base + pos < end;
-            off[h] = ok ? (uint32_t)__ldg(a.col + base + pos) * ldv : 0u;
-            if constexpr (WEIGHTED) w[h] = ok ? __ldg(a.w + base + pos) : 0.0f;
+            off[h] = ok ? (uint32_t)__ldg(a.col_mid + base + pos) * ldv : 0u;
+            if constexpr (WEIGHTED) w[h] = ok ? __ldg(a.w_mid + base + pos) : 0.0f;
         }
     }
     // value held for round position u by its owner lane (u / GS selects the register)
@@ -1151,12 +1151,13 @@ __device__ __forceinline__ void acc_add_slot(float (&acc)[4], const float4& x, f
     }
 }
 
-// Stream the nonzeros [eb, ee) of one row group through the ring: acc += w_e * q[col_e, slab].
+// Stream the nonzeros [eb, ee) (from the middle: mid_entry) of one row group through the ring:
+// acc += w_e * q[col_e, slab].
 // `enter(e)` runs before nonzero e is added when e may open a new row (it closes the rows
 // that end there: row epilogues) and returns the end of the segment that e is in (the first
 // nonzero of the next row); each segment is then consumed without a boundary test per nonzero.
 template <typename T, int GS, bool WEIGHTED, class Enter>
-__device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, uint32_t ldv, uint32_t eb, uint32_t ee,
+__device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, uint32_t ldv, int eb, int ee,
                                              uint32_t ring, int gl, unsigned mask, T (&acc)[kAsyncVec<T>],
                                              Enter&& enter)
 {
@@ -1171,10 +1172,10 @@ __device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, u
         if (eb + u < ee) cp_async16(ring + u * SS, reinterpret_cast<const char*>(q) + (size_t)o * 16);
         cp_async_commit();
     }
-    for (uint32_t base = eb; base < ee; base += D) {  // (unsigned: see gather_row)
+    for (int base = eb; base < ee; base += D) {
         nn.load(a, base + 2 * D, ee, gl, ldv);
-        const int cnt = ee - base < (uint32_t)D ? (int)(ee - base) : D;
-        const int refill = (int)(ee - base) - D;  // slots u < refill are refilled from the next round
+        const int cnt = ee - base < D ? ee - base : D;
+        const int refill = ee - D - base;  // slots u < refill are refilled from the next round
         auto consume = [&](int u) {
             float wv = 1.0f;
             if constexpr (WEIGHTED) wv = __shfl_sync(mask, cur.w_at(u), u % GS, GS);
@@ -1186,7 +1187,7 @@ __device__ __forceinline__ void async_stream(const StepArgs<T>& a, const T* q, u
             cp_async_commit();
         };
         for (int u = 0; u < cnt;) {
-            const int se = (int)(enter(base + u) - base);
+            const int se = enter(base + u) - base;
             const int stop = se < cnt ? se : cnt;
             for (; u < stop; ++u) consume(u);
         }
@@ -1219,8 +1220,8 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async_heavy(cons
             T acc[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) acc[i] = T(0);
-            async_stream<T, GS, WEIGHTED>(a, q, ldv, a.chunk_beg[ch], a.chunk_end[ch], ring, gl, mask, acc,
-                                          [](uint32_t) { return (uint32_t)INT_MAX; });
+            const int eb = mid_entry(a.chunk_beg[ch]), ee = mid_entry(a.chunk_end[ch]);
+            async_stream<T, GS, WEIGHTED>(a, q, ldv, eb, ee, ring, gl, mask, acc, [&](int) { return ee; });
 #pragma unroll
             for (int i = 0; i < V; ++i) acc_finish(acc[i]);
             st_plain<T, V>(a.heavy_part + ch * a.ld + c0, acc);
@@ -1277,17 +1278,17 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
         };
         // light rows [r0, r1): one stream of their nonzeros
         auto light_rows = [&](int r0, int r1) {
-            const uint32_t eb = (uint32_t)a.row_ptr[r0], ee = (uint32_t)a.row_ptr[r1];
+            const int eb = mid_entry(a.row_ptr[r0]), ee = mid_entry(a.row_ptr[r1]);
             T acc[V], qp[V], qc[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) acc[i] = T(0);
             // row window: lane gl holds row_ptr[w0 + gl + 1], 1/d and d of row w0 + gl
             int w0 = r0;
-            uint32_t my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : ee;
+            int my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : ee;
             T my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
-            uint32_t row_end = __shfl_sync(mask, my_end, 0, GS);
+            int row_end = __shfl_sync(mask, my_end, 0, GS);
             ld_stream<T, V>(qp, a.qprev + (int64_t)row * ld + c0);
             ld_gather<T, V>(qc, q + (int64_t)row * ld);
             // the own-row operands of the next PD rows into L2 (no registers held): short rows
@@ -1312,7 +1313,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
                 if (row >= r1) return;
                 if (row - w0 >= GS) {  // refill the row window
                     w0 = row;
-                    my_end = (w0 + gl < r1) ? (uint32_t)a.row_ptr[w0 + gl + 1] : ee;
+                    my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : ee;
                     my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }
@@ -1324,7 +1325,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
                     prefetch_l2(q + (int64_t)(row + PD) * ld);
                 }
             };
-            async_stream<T, GS, WEIGHTED>(a, q, ldv, eb, ee, ring, gl, mask, acc, [&](uint32_t e) {
+            async_stream<T, GS, WEIGHTED>(a, q, ldv, eb, ee, ring, gl, mask, acc, [&](int e) {
                 while (e >= row_end) next_row();
                 return row_end;
             });
