@@ -213,7 +213,9 @@ rd_status rd_graph_create(rd_graph** out, int64_t n, int64_t nnz, const int64_t*
                           const int32_t* col_idx, const float* weights, uint32_t flags, void* stream);
 
 /* Replace the edge weights (same structure, float[nnz] in the order given at create, before
- * self-loop removal), host or device; recomputes degrees. Same weight errors as create. */
+ * self-loop removal), host or device; recomputes degrees. Same weight errors as create. A
+ * weighted graph keeps 4 bytes an entry to check new weights by (the place of each entry's other
+ * copy), given back when a call's workspace does not fit beside them. */
 rd_status rd_graph_set_weights(rd_graph* g, const float* weights, void* stream);
 
 /* Free everything the graph owns. NULL is accepted. */

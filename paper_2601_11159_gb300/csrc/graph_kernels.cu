@@ -238,21 +238,19 @@ static int grid_for(int64_t work, int sm)
 // weights are compared.
 rd_status rows_sorted_symmetric(rd_graph* g, cudaStream_t st)
 {
-    int32_t* f = nullptr;
+    int32_t* f = &static_cast<CheckFlags*>(g->check_scratch)->asymmetric;
     // without memory for the mirrors later weights are searched
-    if (g->w && !g->mirror &&
+    if (g->w && !g->mirror && g->keep_mirror &&
         cudaMalloc((void**)&g->mirror, sizeof(int32_t) * (g->nnz > 0 ? g->nnz : 1)) != cudaSuccess) {
         g->mirror = nullptr;
         cudaGetLastError();
     }
-    RD_CUDA(cudaMallocAsync((void**)&f, sizeof(int32_t), st));
     RD_CUDA(cudaMemsetAsync(f, 0, sizeof(int32_t), st));
     if (g->n > 0)
         k_rows_not_sorted_symmetric<<<grid_for(g->n, g->sm_count), 256, 0, st>>>(g->n, g->row_ptr, g->col, g->w,
                                                                                  g->mirror, f);
     int32_t h = 0;
     RD_CUDA(cudaMemcpyAsync(&h, f, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    RD_CUDA(cudaFreeAsync(f, st));
     RD_CUDA(cudaStreamSynchronize(st));
     g->rows_sorted_sym = h == 0;
     // the search stops at a row's first fault, so the mirrors are whole only without one

@@ -1902,10 +1902,19 @@ static rd_status prepare_run(RunCtx& c, rd_graph* g, int64_t P, const rd_query_o
         Carver dry(nullptr);
         const rd_status ws = ensure_ws(g, carve(dry, g, c.pl, P, grad, &c.b, compact, c.pot_steps, c.pack_ld));
         if (ws >= 0) break;
-        // without the memory: no kept vectors, packing into no more than half the columns
-        if (c.pot_steps > 0) c.pot_steps = 0;
-        else if (c.pack_ld > c.pl.ld / 2) c.pack_ld = c.pl.ld / 2;
-        else return ws;
+        // without the memory: no kept vectors, packing into no more than half the columns, no mirrors
+        if (c.pot_steps > 0) {
+            c.pot_steps = 0;
+        } else if (c.pack_ld > c.pl.ld / 2) {
+            c.pack_ld = c.pl.ld / 2;
+        } else if (g->mirror) {
+            cudaFree(g->mirror);
+            g->mirror = nullptr;
+            g->mirror_ok = false;
+            g->keep_mirror = false;
+        } else {
+            return ws;
+        }
     }
     Carver real(g->ws.base);
     carve(real, g, c.pl, P, grad, &c.b, compact, c.pot_steps, c.pack_ld);

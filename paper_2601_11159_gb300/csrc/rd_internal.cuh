@@ -347,6 +347,7 @@ struct rd_graph {
     const double* inv_sumdeg = nullptr;  // 1 / sum of the degrees (device, in compute_degrees' flags)
     int32_t* mirror = nullptr;        // weighted graphs: entry (v, u) of each entry (u, v)
     bool mirror_ok = false;           // rows sorted and the structure symmetric: mirror is whole
+    bool keep_mirror = true;          // false: given back for a workspace that did not fit beside it
     void* check_scratch = nullptr;    // flags and block sums of compute_degrees
     int32_t* comp = nullptr;
     int32_t ncomp = 0;

@@ -1407,3 +1407,38 @@ def test_pass_calls_poll_as_asked(rd, call):
         every = -(-chunk // 8) * 8
         assert H.last_stats()["steps"] == -(-needed // every) * every
         assert np.array_equal(out, ref)
+
+
+def test_mirrors_give_way_to_a_workspace(rd):
+    """A weighted graph's mirrors (4 bytes an entry, to check new weights by) are given back when a query's
+    workspace does not fit beside them; new weights are then searched for their mirrors and followed."""
+    import torch
+
+    g = F.random_connected(300_000, 6_000_000, 3, "lognormal")
+    w2 = F.weighted(g, F.lognormal_edge_weights(g.m, 0.0, 0.5, 9)).w
+    s, t = F.random_pairs(g.n, 64, 8)
+    kw = dict(mode="fp32", k_max=5, fixed_k=True, kernel="group", rhs_tile=64, compact=False)
+    ref = {}
+    G = rd.Graph.from_csr(g, label_components=False)
+    free = torch.cuda.mem_get_info()[0]
+    ref["w"] = G.query(s, t, **kw).r
+    need = free - torch.cuda.mem_get_info()[0]
+    G.set_weights(w2)
+    ref["w2"] = G.query(s, t, **kw).r
+    G.close()
+    mirrors = 4 * g.nnz
+    assert need > mirrors > 40e6
+    G = rd.Graph.from_csr(g, label_components=False)
+    torch.cuda.empty_cache()
+    hog = torch.empty(int(torch.cuda.mem_get_info()[0] - need + mirrors / 2), dtype=torch.uint8, device="cuda")
+    assert np.array_equal(G.query(s, t, **kw).r, ref["w"])
+    G.set_weights(w2)
+    assert np.array_equal(G.query(s, t, **kw).r, ref["w2"])
+    assert G.last_stats()["sparse_first"] == 1
+    bad = w2.copy()
+    bad[-1] *= 2.0
+    G.set_weights(bad)
+    G.query(s, t, **kw)
+    assert G.last_stats()["sparse_first"] == 0
+    del hog
+    torch.cuda.empty_cache()
