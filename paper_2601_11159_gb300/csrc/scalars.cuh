@@ -1,10 +1,29 @@
-// The estimated relative error of a pair's running value S_k = e_1^T (I - T_k)^{-1} e_1.
+// Scalars of a pair's recurrence: beta_{i+1}, and the estimated relative error of its running value
+// S_k = e_1^T (I - T_k)^{-1} e_1.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <math.h>
 
 namespace rd {
+
+// root = sqrt(x) and inv = 1 / root by one rsqrt (366 cycles) with a Newton correction each, instead of a
+// square root (610) and a division (365): the root within 0.53 units in its last place, its reciprocal
+// rounded correctly. Zero, negative, denormal and non-finite x (told by the exponent bits): the plain
+// forms, or a step that stops and uses neither (it is a breakdown when the root is 0).
+__device__ __forceinline__ void root_and_inverse(double x, double* root, double* inv)
+{
+    const int hi = __double2hiint(x);
+    if (hi >= 0x00200000 && hi < 0x7ff00000) {
+        const double r = rsqrt(x);
+        const double b = x * r;
+        *root = fma(0.5 * r, fma(-b, b, x), b);
+        *inv = fma(r, fma(-*root, r, 1.0), r);
+    } else {
+        *root = sqrt(fmax(x, 0.0));
+        *inv = 1.0 / *root;
+    }
+}
 
 // The increments still to come as a geometric series: i0 is the newest increment of S, i1 to i3 those before
 // it; rho, the largest of the three ratios num/den of neighbours and at least 1/2, gives

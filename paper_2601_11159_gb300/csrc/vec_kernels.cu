@@ -7,7 +7,7 @@
 
 #include <algorithm>
 
-#include "estimate.cuh"
+#include "scalars.cuh"
 #include "spmm.cuh"
 
 namespace rd {
@@ -139,9 +139,7 @@ struct StepCoef {
     double alpha, cdef, beta2, beta, inv_beta;
 };
 
-// beta_{i+1} and its reciprocal by one rsqrt (366 cycles) with a Newton correction each, which
-// leaves both within rounding of sqrt and 1/sqrt (610 and 365 cycles): this chain stands between
-// the sums and the next vector.
+// The chain between the sums and the next vector.
 __device__ __forceinline__ StepCoef step_coef(const FinArgs& a, double inv_sumdeg, double A, double B, double C)
 {
     StepCoef k;
@@ -150,18 +148,7 @@ __device__ __forceinline__ StepCoef step_coef(const FinArgs& a, double inv_sumde
     const double gamma2 = a.deflate ? C * k.cdef : 0.0;
     const double b2 = B - A * A - gamma2;
     k.beta2 = b2;
-    // zero, negative, denormal and non-finite squares (decided on the exponent bits): the plain
-    // forms, or a step that stops and uses neither
-    const int hi = __double2hiint(b2);
-    if (hi >= 0x00200000 && hi < 0x7ff00000) {
-        const double r = rsqrt(b2);
-        const double b = b2 * r;
-        k.beta = fma(0.5 * r, fma(-b, b, b2), b);
-        k.inv_beta = fma(r, fma(-k.beta, r, 1.0), r);
-    } else {
-        k.beta = sqrt(fmax(b2, 0.0));
-        k.inv_beta = 1.0 / k.beta;  // not used when beta is 0 (the step is a breakdown) or not finite
-    }
+    root_and_inverse(b2, &k.beta, &k.inv_beta);
     return k;
 }
 

@@ -36,7 +36,13 @@ static inline int __double2hiint(double d) { uint64_t b; memcpy(&b, &d, 8); retu
 template <typename T> static inline T __shfl_xor_sync(unsigned, T v, int, int = 32) { return v; }
 template <typename T> static inline T __shfl_sync(unsigned, T v, int, int = 32) { return v; }
 using std::fma; using std::fmax; using std::fabs; using std::sqrt;
-static inline double rsqrt(double x) { return 1.0 / std::sqrt(x); }
+static int rsqrt_off = 0;  // units in the last place by which rsqrt is made to miss
+static inline double rsqrt(double x)
+{
+    double r = 1.0 / std::sqrt(x);
+    for (int i = 0; i < std::abs(rsqrt_off); ++i) r = std::nextafter(r, rsqrt_off > 0 ? INFINITY : 0.0);
+    return r;
+}
 """
 
 

@@ -100,5 +100,34 @@ int main()
         }
     printf("%ld %ld %d", n, bad, worst <= 1.0);
 }
-""", headers=("estimate.cuh",))
+""", headers=("scalars.cuh",))
     assert out == "44000 0 1"
+
+
+def test_root_and_inverse_within_rounding(tmp_path):
+    """beta and 1/beta from one reciprocal square root: with that root off by up to two units in its last place
+    either way (CUDA states one), both come out within one unit in the last place of the root and of the
+    reciprocal of the root as rounded (what a square root and a division give within half a unit), over
+    the whole range of exponents."""
+    out = host_cc.run(tmp_path, r"""
+int main()
+{
+    std::mt19937_64 g(7);
+    double worst_root = 0.0, worst_inv = 0.0;
+    for (int i = 0; i < 300000; ++i) {
+        const double x = std::ldexp(1.0 + (double)(g() >> 12) * 0x1p-52, (int)(g() % 2040) - 1019);
+        rsqrt_off = (int)(g() % 5) - 2;
+        double root, inv;
+        rd::root_and_inverse(x, &root, &inv);
+        const long double s = std::sqrt((long double)x), q = 1.0L / root;  // the reciprocal of beta as rounded
+        worst_root = std::fmax(worst_root, (double)(std::fabs(root - s) / (std::nextafter((double)s, INFINITY) - (double)s)));
+        worst_inv = std::fmax(worst_inv, (double)(std::fabs(inv - q) / (std::nextafter((double)q, INFINITY) - (double)q)));
+    }
+    double root, inv;
+    rd::root_and_inverse(-1e-20, &root, &inv);
+    const bool neg = root == 0.0;
+    rd::root_and_inverse(4e-310, &root, &inv);
+    printf("%d %d %d %d", worst_root <= 1.0, worst_inv <= 1.0, neg, root == std::sqrt(4e-310));
+}
+""", headers=("scalars.cuh",))
+    assert out == "1 1 1 1"
