@@ -2680,15 +2680,19 @@ extern "C" rd_status rd_power_method(rd_graph* g, const int32_t* s, const int32_
     rd_query_opts_init(&o);
     o.mode = mode;
     o.k_max = steps + 1;
-    // row-group kernel, rows by degree: the rows of a warp then end together (100,000 vertices of mean
-    // degree 23, 16 FP64 columns: 130 us a step in natural order, 111 by degree)
-    o.kernel = 3;
+    o.kernel = 1;
     if (steps < 0 || steps >= (1 << 22)) {
         set_error("steps must be in [0, 2^22)");
         return RD_ERR_INVALID_ARG;
     }
     RD_TRY(validate_common(g, s, t, npairs, &o, &o));
     if (o.mode == RD_MODE_DF64) o.mode = RD_MODE_FP64;  // double-float vectors: rd_query only
+    // row-group kernel; rows by degree where their lengths differ and several columns make the row's
+    // work: the rows of a warp then end together (200,000 vertices of mean degree 24, 16 FP64 columns, 30
+    // steps 7,042 us in natural order, 6,053 by degree; R-MAT 18 17,360 and 9,686). On graphs of short
+    // rows of one length the order only scatters neighbours (1024^2 road grid, 16 columns, FP32 2,947
+    // and 3,537, FP64 9,797 and 11,056), and one column gains nothing (20,000 vertices 400 and 445)
+    if (npairs > 1 && (g->nnz > 8 * g->n || g->n_heavy_rows > 0)) o.kernel = 3;
     if (npairs > 0 && !r_out) {
         set_error("r_out must not be NULL");
         return RD_ERR_INVALID_ARG;

@@ -1442,3 +1442,22 @@ def test_mirrors_give_way_to_a_workspace(rd):
     assert G.last_stats()["sparse_first"] == 0
     del hog
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("mode", ["fp32", "fp64"])
+def test_power_method_row_order(rd, mode):
+    """The Power Method visits rows by degree where they differ in length and several columns share them, and in
+    their own order on grids, where neighbours belong together, and for one column; the estimates are the
+    oracle's."""
+    for g, by_degree in ((F.grid_deleted(40, 0.05, 5), 0), (F.random_connected(900, 9000, 3, None), 1),
+                         (F.star(700), 1)):
+        G = rd.Graph.from_csr(g)
+        s, t = F.random_pairs(g.n, 6, 8)
+        r, hist = G.power_method(s, t, 12, mode=mode, history=True)
+        assert G.last_stats()["row_order"] == by_degree
+        for p in range(6):
+            one, h1 = G.power_method(s[p:p + 1], t[p:p + 1], 12, mode=mode, history=True)
+            assert G.last_stats()["row_order"] == 0
+            ref = power.power_method(g, int(s[p]), int(t[p]), 12)
+            assert np.abs(hist[:, p] - ref).max() < (1e-11 if mode == "fp64" else 1e-5) * np.abs(ref).max()
+            assert np.abs(h1[:, 0] - ref).max() < (1e-11 if mode == "fp64" else 1e-5) * np.abs(ref).max()
