@@ -539,6 +539,10 @@ static rd_status make_plan_cfg(rd_graph* g, int64_t P, const rd_query_opts& o, c
     pl->fp64 = pl->prec != 0;
     pl->elem = pl->fp64 ? 8 : 4;
     pl->cfg = cfg;
+    if ((cfg.kind == 1 || cfg.kind == 3) && g->nnz > kStreamEntries) {
+        pl->cfg.kind = 0;
+        if (!cfg_known(pl->cfg, pl->fp64)) pl->cfg.nzl = 32 / cfg.gs;
+    }
     if (cfg.kind == 4 && g->n > (1 << 30)) {  // its rows past the last are counted in 32 bits
         set_error("the row pipeline takes graphs of up to 2^30 vertices");
         return RD_ERR_UNSUPPORTED;
@@ -812,8 +816,6 @@ static StepArgs<T> step_args(RunCtx& c, int j, bool reduce)
     a.row_ptr = g->row_ptr;
     a.col = g->col;
     a.w = g->w;
-    a.col_mid = g->col + kMidEntry;
-    a.w_mid = g->w ? g->w + kMidEntry : nullptr;
     if constexpr (std::is_same<T, df64>::value) {
         a.invdeg = g->invdegdf;
         a.deg = g->degdf;

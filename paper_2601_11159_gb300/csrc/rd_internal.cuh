@@ -69,12 +69,12 @@ constexpr int kWarps = kBlock / 32;
 constexpr int kRing = 4;           // increments kept for the delayed error estimate
 
 // Argument block of one Lanczos step's SpMM (q-space: q = D^{-1/2} v).
-// Entries counted from the middle of their range, as the row-stream kernels count them in a signed
-// 32-bit number: from the front, a loop that steps past a row's end near 2^31 entries would turn
-// negative, and unsigned counters cost the weighted async kernel 3% (a gradient over 79.8M entries 17.2 ->
-// 17.7 ms).
-constexpr int64_t kMidEntry = int64_t(1) << 30;
-__host__ __device__ __forceinline__ int mid_entry(int64_t e) { return (int)(e - kMidEntry); }
+// The row-stream and async kernels count entries in a signed 32-bit number and step (or look) up to this far
+// past a row's end: graphs of more entries than 2^31 - 1 less this take the row-group kernel, whose
+// counter has no sign, in their place. (Counting without a sign, from the middle of the range, or by what is
+// left costs those two 3-5%: a gradient over 79.8M entries 17.2 -> 17.7 ms.)
+constexpr int64_t kStreamReach = 1024;
+constexpr int64_t kStreamEntries = (int64_t(1) << 31) - 1 - kStreamReach;
 
 template <typename T>
 struct StepArgs {
@@ -82,8 +82,6 @@ struct StepArgs {
     const int64_t* row_ptr;
     const int32_t* col;
     const float* w;                // nullable (unweighted)
-    const int32_t* col_mid;        // col + kMidEntry, w + kMidEntry
-    const float* w_mid;
     const T* invdeg;               // 1/d_u
     const T* deg;                  // d_u
     const T* qcur;                 // q_i  (n x ld)

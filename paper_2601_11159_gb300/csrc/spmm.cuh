@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
 
         for (int task = gid; task < ntasks; task += ngroups) {
             const int r0 = a.task_row[task], r1 = a.task_row[task + 1];
-            const int e_beg = mid_entry(a.row_ptr[r0]), e_end = mid_entry(a.row_ptr[r1]);
+            const int e_beg = (int)a.row_ptr[r0], e_end = (int)a.row_ptr[r1];
             T acc[VEC], qp[VEC], qc[VEC];
 #pragma unroll
             for (int i = 0; i < VEC; ++i) acc[i] = T(0);
@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
             }
             // row window: lane gl holds row_ptr[w0 + gl + 1], 1/d and d of row w0 + gl
             int w0 = r0;
-            int my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : e_end;
+            int my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : e_end;
             T my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
@@ -913,9 +913,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
                     const int idx = h * GS + gl;
-                    const uint32_t j = idx < cnt ? (uint32_t)__ldg(a.col_mid + base + idx) : 0u;
+                    const uint32_t j = idx < cnt ? (uint32_t)__ldg(a.col + base + idx) : 0u;
                     my_off[h] = j * ldv;
-                    if constexpr (WEIGHTED) my_w[h] = idx < cnt ? __ldg(a.w_mid + base + idx) : 0.0f;
+                    if constexpr (WEIGHTED) my_w[h] = idx < cnt ? __ldg(a.w + base + idx) : 0.0f;
 #if RD_ROWS_PREFETCH
                     if (idx < cnt) {
                         const char* rowp = reinterpret_cast<const char*>(qslab + (int64_t)j * ld);
@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                             ++row;
                             if (row - w0 >= GS) {  // refill the row window
                                 w0 = row;
-                                my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : e_end;
+                                my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : e_end;
                                 my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                                 my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                             }
@@ -993,7 +993,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks<T, VEC>) k_spmm_rows(const 
                 if (row >= r1) break;
                 if (row - w0 >= GS) {
                     w0 = row;
-                    my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : e_end;
+                    my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : e_end;
                     my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }
@@ -1089,8 +1089,8 @@ struct AsyncRound {
         for (int h = 0; h < NH; ++h) {
             const int pos = h * GS + gl;
             const bool ok = pos < kAsyncDepth && base + pos < end;
-            off[h] = ok ? (uint32_t)__ldg(a.col_mid + base + pos) * ldv : 0u;
-            if constexpr (WEIGHTED) w[h] = ok ? __ldg(a.w_mid + base + pos) : 0.0f;
+            off[h] = ok ? (uint32_t)__ldg(a.col + base + pos) * ldv : 0u;
+            if constexpr (WEIGHTED) w[h] = ok ? __ldg(a.w + base + pos) : 0.0f;
         }
     }
     // value held for round position u by its owner lane (u / GS selects the register)
@@ -1151,8 +1151,7 @@ __device__ __forceinline__ void acc_add_slot(float (&acc)[4], const float4& x, f
     }
 }
 
-// Stream the nonzeros [eb, ee) (from the middle: mid_entry) of one row group through the ring:
-// acc += w_e * q[col_e, slab].
+// Stream the nonzeros [eb, ee) of one row group through the ring: acc += w_e * q[col_e, slab].
 // `enter(e)` runs before nonzero e is added when e may open a new row (it closes the rows
 // that end there: row epilogues) and returns the end of the segment that e is in (the first
 // nonzero of the next row); each segment is then consumed without a boundary test per nonzero.
@@ -1220,8 +1219,8 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async_heavy(cons
             T acc[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) acc[i] = T(0);
-            const int eb = mid_entry(a.chunk_beg[ch]), ee = mid_entry(a.chunk_end[ch]);
-            async_stream<T, GS, WEIGHTED>(a, q, ldv, eb, ee, ring, gl, mask, acc, [&](int) { return ee; });
+            async_stream<T, GS, WEIGHTED>(a, q, ldv, a.chunk_beg[ch], a.chunk_end[ch], ring, gl, mask, acc,
+                                          [](int) { return INT_MAX; });
 #pragma unroll
             for (int i = 0; i < V; ++i) acc_finish(acc[i]);
             st_plain<T, V>(a.heavy_part + ch * a.ld + c0, acc);
@@ -1278,13 +1277,13 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
         };
         // light rows [r0, r1): one stream of their nonzeros
         auto light_rows = [&](int r0, int r1) {
-            const int eb = mid_entry(a.row_ptr[r0]), ee = mid_entry(a.row_ptr[r1]);
+            const int eb = (int)a.row_ptr[r0], ee = (int)a.row_ptr[r1];
             T acc[V], qp[V], qc[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) acc[i] = T(0);
             // row window: lane gl holds row_ptr[w0 + gl + 1], 1/d and d of row w0 + gl
             int w0 = r0;
-            int my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : ee;
+            int my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : ee;
             T my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
             T my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
             int row = r0;
@@ -1313,7 +1312,7 @@ __global__ void __launch_bounds__(kBlock, RD_ASYNC_MINB) k_spmm_async(const Step
                 if (row >= r1) return;
                 if (row - w0 >= GS) {  // refill the row window
                     w0 = row;
-                    my_end = (w0 + gl < r1) ? mid_entry(a.row_ptr[w0 + gl + 1]) : ee;
+                    my_end = (w0 + gl < r1) ? (int)a.row_ptr[w0 + gl + 1] : ee;
                     my_invd = (w0 + gl < r1) ? a.invdeg[w0 + gl] : T(0);
                     my_deg = (w0 + gl < r1) ? a.deg[w0 + gl] : T(0);
                 }

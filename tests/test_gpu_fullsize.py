@@ -255,7 +255,7 @@ def test_rmat24_batched_and_plain(rd):
 def test_entry_counts_up_to_the_limit(rd):
     """2^31 - 8 stored entries (a clique of 46,341 vertices with a path behind it, whose rows hold the
     last entries): a kernel that steps past a row's end must not wrap round. Pairs near the path's end
-    have after three steps, without deflation, the r_k of a short path, in every kernel."""
+    have after three steps, without deflation, the r_k of a short path, whatever kernel is asked for."""
     import torch
 
     k, m = 46341, 20850
@@ -283,9 +283,11 @@ def test_entry_counts_up_to_the_limit(rd):
     kw = dict(k_max=3, fixed_k=True, deflate=False, sparse_first=False, onchip=False, tune=False)
     ref = S.query((199 - off).astype(np.int32), (199 - to).astype(np.int32), mode="fp64", **kw).r
     s, t = (n - 1 - off).astype(np.int32), (n - 1 - to).astype(np.int32)
-    for kernel in ("group", "group_sorted", "stream", "async"):
+    for kernel in ("group", "group_sorted", "stream", "async", "pipe"):
         for mode, tol in (("fp64", 1e-12), ("fp32", 1e-5), ("df64", 1e-11)):
             r = G.query(s, t, mode=mode, kernel=kernel, **kw).r
             assert rel(r, ref).max() < tol, (kernel, mode)
+            # the row-stream kernels leave the last 1,024 entries of the range to the row-group kernel
+            assert G.last_stats()["kernel"] == {"group_sorted": 3, "pipe": 6}.get(kernel, 1)
     one = G.query(s[:1], t[:1], mode="fp64", kernel="tasks", **kw).r
     assert rel(one, ref[:1]).max() < 1e-12
