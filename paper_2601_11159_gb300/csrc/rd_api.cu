@@ -539,7 +539,8 @@ static rd_status make_plan_cfg(rd_graph* g, int64_t P, const rd_query_opts& o, c
     pl->fp64 = pl->prec != 0;
     pl->elem = pl->fp64 ? 8 : 4;
     pl->cfg = cfg;
-    if ((cfg.kind == 1 || cfg.kind == 3) && g->nnz > kStreamEntries) {
+    if ((cfg.kind == 1 || cfg.kind == 3) &&
+        (g->nnz > kStreamEntries || g->n * (padded_columns(P, cfg) / cfg.vec) > kStreamUnits)) {
         pl->cfg.kind = 0;
         if (!cfg_known(pl->cfg, pl->fp64)) pl->cfg.nzl = 32 / cfg.gs;
     }

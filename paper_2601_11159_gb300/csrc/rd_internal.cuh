@@ -75,6 +75,9 @@ constexpr int kRing = 4;           // increments kept for the delayed error esti
 // left costs those two 3-5%: a gradient over 79.8M entries 17.2 -> 17.7 ms.)
 constexpr int64_t kStreamReach = 1024;
 constexpr int64_t kStreamEntries = (int64_t(1) << 31) - 1 - kStreamReach;
+// They hold the offset of a gathered row as 32 bits of the lane's VEC elements: blocks of more units (64 GB at
+// 16 bytes a lane) take the row-group kernel as well, whose offsets have 64 bits.
+constexpr int64_t kStreamUnits = int64_t(1) << 32;
 
 template <typename T>
 struct StepArgs {

@@ -291,3 +291,31 @@ def test_entry_counts_up_to_the_limit(rd):
             assert G.last_stats()["kernel"] == {"group_sorted": 3, "pipe": 6}.get(kernel, 1)
     one = G.query(s[:1], t[:1], mode="fp64", kernel="tasks", **kw).r
     assert rel(one, ref[:1]).max() < 1e-12
+
+
+def test_blocks_past_32_bit_row_offsets(rd):
+    """A path of 2^24 + 4,096 vertices with 4 KB of a vector block to a row (1,024 FP32 or 512 FP64
+    columns): the last rows start 2^32 16-byte units and more into a block. Pairs near the path's end have after three
+    steps, without deflation, the r_k of a short path, whatever kernel is asked for."""
+    import torch
+
+    n = 2**24 + 4096
+    torch.cuda.empty_cache()
+    v = torch.arange(n, dtype=torch.int32, device="cuda")
+    col = torch.stack([v - 1, v + 1], 1).view(-1)[1:-1].contiguous()  # the ends have one neighbour
+    rp = torch.arange(n + 1, dtype=torch.int64, device="cuda") * 2 - 1
+    rp[0], rp[-1] = 0, 2 * n - 2
+    assert col.numel() == 2 * n - 2
+    G = rd.Graph(rp, col, label_components=False)
+    S = rd.Graph.from_csr(F.path(200))
+    kw = dict(k_max=3, fixed_k=True, deflate=False, sparse_first=False, onchip=False, tune=False)
+    for mode, columns, tol in (("fp32", 1024, 1e-5), ("fp64", 512, 1e-12), ("df64", 512, 1e-11)):
+        off = 1 + np.arange(columns) % 17
+        to = (off + 1) % 4
+        ref = S.query((199 - off[:17]).astype(np.int32), (199 - to[:17]).astype(np.int32), mode="fp64", **kw).r
+        ref = ref[np.arange(columns) % 17]
+        s, t = (n - 1 - off).astype(np.int32), (n - 1 - to).astype(np.int32)
+        for kernel in ("group", "stream", "async"):
+            r = G.query(s, t, mode=mode, kernel=kernel, rhs_tile=64, **kw).r
+            assert rel(r, ref).max() < tol, (kernel, mode)
+            assert G.last_stats()["kernel"] == 1
